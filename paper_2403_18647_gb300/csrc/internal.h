@@ -171,7 +171,11 @@ struct PfGemmParams {
   int N;                    // output features (MAP_GATEUP: F)
   int kc;                   // 64-column chunks of K
   int n_wtiles, n_tblocks;  // tiles of 128 weight rows, blocks of 128 positions
+  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next two)
+  int sk_tiles, sk_pairs;   // the first sk_tiles tiles are split along K over the first sk_pairs CTA pairs
   int M;                    // positions
+  float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]
+  int* counters;            // [2 * num_sms], zero between launches
   int epi;                  // EPI_STORE, EPI_RESID or EPI_SWIGLU
   float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID)
   int out_ld;
@@ -180,6 +184,7 @@ struct PfGemmParams {
   uint32_t* err;
 };
 cudaError_t prefill_prepare();
+size_t prefill_partials(int num_sms);
 cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 struct RopeKvParams {
   const float* qkv;         // [M][3R]

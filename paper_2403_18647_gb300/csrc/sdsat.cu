@@ -131,6 +131,8 @@ struct sdsat_ctx {
   int* adaptive = nullptr;
   uint32_t* err = nullptr;
   // prefill workspaces (chunks of up to PF_ROWS positions; allocated with the weights)
+  float* pf_partials = nullptr;  // split-K parts and tile counters of the prefill GEMM
+  int* pf_counters = nullptr;
   float* pf_h = nullptr;         // [PF_ROWS][d] residual stream
   float* pf_qkv = nullptr;       // [PF_ROWS][3R] projections before RoPE
   float* pf_q = nullptr;         // [PF_ROWS][R] rotated queries
@@ -423,6 +425,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     g.kc = (K + 63) / 64;
     g.n_tblocks = ntb;
     g.M = M;
+    g.partials = c->pf_partials;
+    g.counters = c->pf_counters;
     g.err = c->err;
     return g;
   };
@@ -645,6 +649,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
             dalloc(c, &c->qbuf, (size_t)rows * R) && dalloc(c, &c->attn, (size_t)rows * R) &&
             dalloc(c, &c->act, (size_t)rows * F) && dalloc(c, &c->partials, (size_t)c->num_sms * 2 * 2 * 64 * 128) &&
             dalloc(c, &c->gemm_counters, MAX_GEMM_TILES) &&
+            dalloc(c, &c->pf_partials, prefill_partials(c->num_sms)) &&
+            dalloc(c, &c->pf_counters, 2 * (size_t)c->num_sms) &&
             dalloc(c, &c->acc_targets, rows) &&
             dalloc(c, &c->acc_counters, rows) && dalloc(c, &c->adaptive, SDSAT_MAX_ADAPTIVE) &&
             dalloc(c, &c->tree_pos, rows) && dalloc(c, &c->tree_anc, rows) &&
@@ -1072,6 +1078,8 @@ sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const
     g.epi = EPI_STORE;
     g.out = y_dev;
     g.out_ld = N;
+    g.partials = c->pf_partials;
+    g.counters = c->pf_counters;
     g.err = c->err;
     if (launch_split(x_dev, M, K, c->xop_hi, c->xop_lo, c->stream, c->pdl) != cudaSuccess) return SDSAT_ECUDA;
     return timed(c, K_GEMM_OP, [&] { return launch_prefill_gemm(g, c->num_sms, c->stream, c->pdl); }) == cudaSuccess
