@@ -163,15 +163,19 @@ struct PfAttnParams {
 cudaError_t launch_prefill_attention(const PfAttnParams& p, cudaStream_t st, bool pdl);
 
 // ---- prefill (prompt chunks of up to PF_ROWS positions) -------------------------
-constexpr int PF_ROWS = 512;
+#ifndef SDSAT_PF_ROWS
+#define SDSAT_PF_ROWS 2048
+#endif
+constexpr int PF_ROWS = SDSAT_PF_ROWS;
 struct PfGemmParams {
   CUtensorMap tmap[3];      // weights, as GemmParams::tmap (map_mode)
-  CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [PF_ROWS][K], boxes of 64 x 128
+  CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [rows][K], boxes of 64 x 128
   int map_mode, rows_per_map;
   int N;                    // output features (MAP_GATEUP: F)
   int kc;                   // 64-column chunks of K
   int n_wtiles, n_tblocks;  // tiles of 128 weight rows, blocks of 128 positions
-  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next two)
+  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next three)
+  int group;                // position blocks numbered together
   int sk_tiles, sk_pairs;   // the first sk_tiles tiles are split along K over the first sk_pairs CTA pairs
   int M;                    // positions
   float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]

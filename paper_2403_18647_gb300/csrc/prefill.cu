@@ -38,6 +38,10 @@ constexpr int PF_XROW = PF_CHUNK / 2 + 1;                // exchange row: half a
 constexpr int PF_STAGING = 2 * 128 * PF_XROW;            // fp32 exchange of the two epilogue groups
 constexpr int PF_NBAR = 2 * PF_STAGES + 5;
 constexpr size_t PF_SMEM = 1024 + (size_t)PF_STAGES * PF_STAGE + PF_STAGING * 4 + PF_NBAR * 8 + 64;
+#ifndef SDSAT_PF_GROUP
+#define SDSAT_PF_GROUP 8
+#endif
+constexpr int PF_GROUP = SDSAT_PF_GROUP;
 constexpr int PF_SK_MIN = 4;                             // chunks of a split-K share, at least
 
 __device__ __forceinline__ void pf_tile_half_src(int map_mode, int rows_per_map, int t, int h, int& map, int& row) {
@@ -85,6 +89,16 @@ struct PfWalk {
     return true;
   }
 };
+
+// Tile -> (pair of weight tiles, position block).  Position blocks go in groups of p.group:
+// within a group the tiles are numbered weight-major, so the pairs working at the same time
+// share a few weight tiles and the group's positions through L2.
+__device__ __forceinline__ void pf_tile(const PfGemmParams& p, int tile, int& wp, int& tb) {
+  const int per = p.n_pairs_w * p.group, g = tile / per, rem = tile - g * per;
+  const int width = min(p.group, p.n_tblocks - g * p.group);
+  wp = rem / width;
+  tb = g * p.group + rem - wp * width;
+}
 
 __device__ __forceinline__ void pf_drain(uint64_t* bar, uint32_t parity) {
   const uint64_t t0 = globaltimer_ns();
@@ -141,9 +155,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
       const uint64_t pol_x = l2_policy_evict_last();    // a position block is read by every weight tile
       PfWalk w(p, pair);
       bool more = w.next();
-      int kc = w.k0, map0, row0, map1, row1;
+      int kc = w.k0, map0, row0, map1, row1, tb = 0;
       auto src = [&] {   // the CTA's weight tile (past the last one: that one, unused)
-        const int wt = min(2 * (w.tile / p.n_tblocks) + rank, p.n_wtiles - 1);
+        int wp;
+        pf_tile(p, w.tile, wp, tb);
+        const int wt = min(2 * wp + rank, p.n_wtiles - 1);
         pf_tile_half_src(p.map_mode, p.rows_per_map, wt, 0, map0, row0);
         pf_tile_half_src(p.map_mode, p.rows_per_map, wt, 1, map1, row1);
       };
@@ -167,7 +183,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
 #pragma unroll
       for (int s = 0; s < PF_STAGES; ++s) {
         xk[s] = kc;
-        xt[s] = w.tile % p.n_tblocks;
+        xt[s] = tb;
         if (!more) continue;
         if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * PF_STAGE);
         load_w(s, mapa_shared(smem_u32(&full[s]), 0));
@@ -180,7 +196,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
         if (s < npre) load_x(s, mapa_shared(smem_u32(&full[s]), 0), xk[s], xt[s]);
       int it = npre, s = it % PF_STAGES;
       uint32_t ph = 0;   // parity of the stage's previous use being consumed
-      int tb = more ? w.tile % p.n_tblocks : 0;
       while (more) {
         if (!mbar_wait_bounded(&empty[s], ph, abort_flag, p.err)) break;
         if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * PF_STAGE);
@@ -192,10 +207,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
           s = 0;
           ph ^= 1u;
         }
-        if (step() && more) {
-          src();
-          tb = w.tile % p.n_tblocks;
-        }
+        if (step() && more) src();
       }
       if (!*abort_flag) {
         // the CTA stays until the tensor cores have released its last stages (the commits of
@@ -266,7 +278,9 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     int seg = 0;
     PfWalk w(p, pair);
     for (; w.next(); ++seg) {
-      const int wt = 2 * (w.tile / p.n_tblocks) + rank, tb = w.tile % p.n_tblocks;
+      int wp, tb;
+      pf_tile(p, w.tile, wp, tb);
+      const int wt = 2 * wp + rank;
       const int buf = seg & 1;
       const int mt = tb * PF_TOK;   // the tile's first position
       const bool got = named_bar_and(1, NE, mbar_wait_bounded(&acc_full[buf], (seg >> 1) & 1, abort_flag, p.err));
@@ -413,6 +427,7 @@ size_t prefill_partials(int num_sms) { return (size_t)(num_sms / 2) * 2 * 2 * PF
 cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl) {
   const int P = std::max(1, std::min(num_sms / 2, g_pf_pairs));
   p.n_pairs_w = (p.n_wtiles + 1) / 2;
+  p.group = std::min(p.n_tblocks, PF_GROUP);
   const int T = p.n_pairs_w * p.n_tblocks, rem = T % P;
   p.sk_tiles = 0;
   p.sk_pairs = 0;

@@ -96,7 +96,8 @@ const char* const KCLASS_NAME[K_COUNT] = {"rmsnorm", "gemm_qkv", "attention", "g
                                           "prefill_rope_kv", "prefill_attention"};
 
 constexpr int MAX_GEMM_TILES = 1 << 16;
-constexpr int OP_MAX_K = 32768;   // K limit of sdsat_op_gemm (its operand scratch is sized at create)
+constexpr int OP_MAX_K = 32768;   // limits of sdsat_op_gemm (its operand scratch is sized at create)
+constexpr int OP_MAX_M = 512;
 
 // the GEMM activation operands (bf16 hi + lo), one pair per producer
 enum XSrc : int { X_NORM = 0, X_ATTN = 1, X_FFN = 2, X_COUNT = 3 };
@@ -402,7 +403,7 @@ sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const 
   return SDSAT_OK;
 }
 
-// one prefill chunk: M (a multiple of SDSAT_MAX_Q, <= PF_ROWS) prompt positions of sequence seq
+// one prefill chunk: M <= PF_ROWS prompt positions of sequence seq
 // through every layer on the tiled GEMM, then committed
 sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* tokens, int M) {
   const sdsat_config& cf = c->cfg;
@@ -655,9 +656,9 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
             dalloc(c, &c->acc_counters, rows) && dalloc(c, &c->adaptive, SDSAT_MAX_ADAPTIVE) &&
             dalloc(c, &c->tree_pos, rows) && dalloc(c, &c->tree_anc, rows) &&
             dalloc(c, &c->tree_ws, (size_t)rows * TREE_WS_STRIDE) &&
-            dalloc(c, &c->err, 1) && dalloc(c, &c->xop_hi, (size_t)PF_ROWS * OP_MAX_K) &&
+            dalloc(c, &c->err, 1) && dalloc(c, &c->xop_hi, (size_t)OP_MAX_M * OP_MAX_K) &&
             dalloc(c, &c->ssq, (size_t)rows * ((d + 127) / 128)) &&
-            dalloc(c, &c->xop_lo, (size_t)PF_ROWS * OP_MAX_K);
+            dalloc(c, &c->xop_lo, (size_t)OP_MAX_M * OP_MAX_K);
   const int xcols[X_COUNT] = {d, R, F};
   for (int xs = 0; ok && xs < X_COUNT; ++xs) {
     ok = dalloc(c, &c->x_hi[xs], (size_t)rows * xcols[xs]) && dalloc(c, &c->x_lo[xs], (size_t)rows * xcols[xs]);
@@ -826,23 +827,21 @@ sdsat_status sdsat_prefill(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
   if (!c || !kv || kv->ctx != c || !c->has_weights || !tokens_dev || seq < 0 || seq >= kv->batch || n < 0)
     return SDSAT_EINVAL;
   if (n > kv->cap) return SDSAT_ECAPACITY;
-  // chunks of up to PF_ROWS positions (a multiple of SDSAT_MAX_Q) on the tiled GEMM; a tail
-  // shorter than SDSAT_MAX_Q runs as one ordinary block
-  for (int i = 0; i < n;) {
-    const int rem = n - i;
-    if (rem >= SDSAT_MAX_Q) {
-      const int M = std::min(PF_ROWS, rem / SDSAT_MAX_Q * SDSAT_MAX_Q);
-      const sdsat_status s = prefill_chunk(c, kv, seq, tokens_dev + i, M);
-      if (s != SDSAT_OK) return s;
-      i += M;
-      continue;
-    }
-    const sdsat_status s = forward(c, kv, seq, 1, rem, tokens_dev + i, nullptr, nullptr);
+  if (n > 0 && n <= SDSAT_MAX_Q) {   // fits one block
+    const sdsat_status s = forward(c, kv, seq, 1, n, tokens_dev, nullptr, nullptr);
     if (s != SDSAT_OK) return s;
-    if (timed(c, K_PREFILL_COMMIT, [&] { return launch_add_len(kv->len, seq, rem, kv->cap, c->err, c->stream, c->pdl); }) !=
-        cudaSuccess)
-      return SDSAT_ECUDA;
-    i += rem;
+    return timed(c, K_PREFILL_COMMIT, [&] { return launch_add_len(kv->len, seq, n, kv->cap, c->err, c->stream, c->pdl); }) ==
+                   cudaSuccess
+               ? SDSAT_OK
+               : SDSAT_ECUDA;
+  }
+  // Chunks of equal size up to the position block: every chunk streams all the weights, so
+  // none is left with a few positions (a 4095-position prompt: 2048 + 2047; 2050: 1152 + 898).
+  const int chunks = (n + PF_ROWS - 1) / PF_ROWS;
+  const int per = chunks ? ((n + chunks - 1) / chunks + 127) / 128 * 128 : 0;
+  for (int i = 0; i < n; i += per) {
+    const sdsat_status s = prefill_chunk(c, kv, seq, tokens_dev + i, std::min(per, n - i));
+    if (s != SDSAT_OK) return s;
   }
   return SDSAT_OK;
 }
@@ -1059,11 +1058,11 @@ sdsat_status sdsat_get_error(sdsat_ctx* c, uint32_t* flags) {
 
 sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const void* w_dev, int N, float* y_dev) {
   if (!c || !x_dev || !y_dev || !aligned16(w_dev) || !aligned16(x_dev)) return SDSAT_EINVAL;
-  if (M < 1 || M > PF_ROWS || K < 8 || K % 8 || K > OP_MAX_K || N < 1 || (N + 127) / 128 > MAX_GEMM_TILES)
+  if (M < 1 || M > OP_MAX_M || K < 8 || K % 8 || K > OP_MAX_K || N < 1 || (N + 127) / 128 > MAX_GEMM_TILES)
     return SDSAT_EINVAL;
   if (M > SDSAT_MAX_ROWS) {
     // the prefill GEMM (tiles of 128 weight rows x 128 positions)
-    const int rows = (M + 127) / 128 * 128;   // <= PF_ROWS rows of the operand scratch
+    const int rows = (M + 127) / 128 * 128;   // <= OP_MAX_M rows of the operand scratch
     PfGemmParams g;
     std::memset(&g, 0, sizeof(g));
     if (!make_wmap(&g.tmap[0], w_dev, N, K) || !make_xmap(&g.tmap_x[0], c->xop_hi, rows, K, 128) ||
