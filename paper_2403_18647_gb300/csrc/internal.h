@@ -169,12 +169,13 @@ cudaError_t launch_prefill_attention(const PfAttnParams& p, cudaStream_t st, boo
 constexpr int PF_ROWS = SDSAT_PF_ROWS;
 struct PfGemmParams {
   CUtensorMap tmap[3];      // weights, as GemmParams::tmap (map_mode)
-  CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [rows][K], boxes of 64 x 128
+  CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [rows][K], boxes of 64 x prefill_tok(M)
   int map_mode, rows_per_map;
   int N;                    // output features (MAP_GATEUP: F)
   int kc;                   // 64-column chunks of K
-  int n_wtiles, n_tblocks;  // tiles of 128 weight rows, blocks of 128 positions
-  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next three)
+  int n_wtiles;             // tiles of 128 weight rows
+  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next four)
+  int n_tblocks;            // blocks of prefill_tok(M) positions
   int group;                // position blocks numbered together
   int sk_tiles, sk_pairs;   // the first sk_tiles tiles are split along K over the first sk_pairs CTA pairs
   int M;                    // positions
@@ -186,8 +187,10 @@ struct PfGemmParams {
   __nv_bfloat16* out_hi;    // EPI_SWIGLU: [M][out_ld] the down projection's operand
   __nv_bfloat16* out_lo;
   uint32_t* err;
+  Trace trace;
 };
 cudaError_t prefill_prepare();
+int prefill_tok(int M);      // positions per tile of the GEMM over M positions: 64 or 128
 size_t prefill_partials(int num_sms);
 cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 struct RopeKvParams {

@@ -120,7 +120,7 @@ struct sdsat_ctx {
   float* qbuf = nullptr;
   float* attn = nullptr;
   float* act = nullptr;
-  float* partials = nullptr;
+  float* partials = nullptr;   // split-K parts and tile counters of the GEMM that runs (decode or prefill)
   int* gemm_counters = nullptr;
   float* ssq = nullptr;        // [SDSAT_MAX_ROWS][ssq_ld] per-tile sums of h^2 (RMSNorm folded into the GEMMs)
   int ssq_ld = 0;
@@ -132,15 +132,13 @@ struct sdsat_ctx {
   int* adaptive = nullptr;
   uint32_t* err = nullptr;
   // prefill workspaces (chunks of up to PF_ROWS positions; allocated with the weights)
-  float* pf_partials = nullptr;  // split-K parts and tile counters of the prefill GEMM
-  int* pf_counters = nullptr;
   float* pf_h = nullptr;         // [PF_ROWS][d] residual stream
   float* pf_qkv = nullptr;       // [PF_ROWS][3R] projections before RoPE
   float* pf_q = nullptr;         // [PF_ROWS][R] rotated queries
   float* pf_attn = nullptr;      // [PF_ROWS][R] attention output
   __nv_bfloat16* pf_hi[X_COUNT] = {};   // GEMM operands [PF_ROWS][K] (normed x, attention, act)
   __nv_bfloat16* pf_lo[X_COUNT] = {};
-  CUtensorMap pf_xmap[X_COUNT][2];      // boxes of 64 x 128
+  CUtensorMap pf_xmap[2][X_COUNT][2];   // boxes of 64 x 128 and 64 x 64
   __nv_bfloat16* x_hi[X_COUNT] = {};
   __nv_bfloat16* x_lo[X_COUNT] = {};
   CUtensorMap xmap[X_COUNT][3][2];     // [source][MPAD 16/32/64][hi/lo]
@@ -410,7 +408,7 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
   const int d = cf.d_model, H = cf.n_heads, hd = cf.head_dim, F = cf.ffn_dim, R = H * hd, L = cf.n_layers;
   cudaStream_t st = c->stream;
   const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
-  const int ntb = (M + 127) / 128;
+  const int xi = prefill_tok(M) == 64;
   auto norm = [&](const int32_t* toks, const void* gain) {
     return timed(c, K_RMSNORM, [&] {
       return launch_rmsnorm(toks, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->pf_h, d, M,
@@ -421,17 +419,17 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
   auto base = [&](int xsrc, int K) {
     PfGemmParams g;
     std::memset(&g, 0, sizeof(g));
-    g.tmap_x[0] = c->pf_xmap[xsrc][0];
-    g.tmap_x[1] = c->pf_xmap[xsrc][1];
+    g.tmap_x[0] = c->pf_xmap[xi][xsrc][0];
+    g.tmap_x[1] = c->pf_xmap[xi][xsrc][1];
     g.kc = (K + 63) / 64;
-    g.n_tblocks = ntb;
     g.M = M;
-    g.partials = c->pf_partials;
-    g.counters = c->pf_counters;
+    g.partials = c->partials;
+    g.counters = c->gemm_counters;
     g.err = c->err;
     return g;
   };
   auto gemm = [&](PfGemmParams& g) {
+    g.trace = next_trace(c, K_PF_GEMM);
     return timed(c, K_PF_GEMM, [&] { return launch_prefill_gemm(g, c->num_sms, st, c->pdl); });
   };
   if (norm(tokens, c->layers[0].attn_norm) != cudaSuccess) return SDSAT_ECUDA;
@@ -648,10 +646,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   c->ssq_ld = (d + 127) / 128;
   bool ok = dalloc(c, &c->rope, rope.size()) && dalloc(c, &c->h, (size_t)rows * d) &&
             dalloc(c, &c->qbuf, (size_t)rows * R) && dalloc(c, &c->attn, (size_t)rows * R) &&
-            dalloc(c, &c->act, (size_t)rows * F) && dalloc(c, &c->partials, (size_t)c->num_sms * 2 * 2 * 64 * 128) &&
+            dalloc(c, &c->act, (size_t)rows * F) && dalloc(c, &c->partials, std::max((size_t)c->num_sms * 2 * 2 * 64 * 128, prefill_partials(c->num_sms))) &&
             dalloc(c, &c->gemm_counters, MAX_GEMM_TILES) &&
-            dalloc(c, &c->pf_partials, prefill_partials(c->num_sms)) &&
-            dalloc(c, &c->pf_counters, 2 * (size_t)c->num_sms) &&
             dalloc(c, &c->acc_targets, rows) &&
             dalloc(c, &c->acc_counters, rows) && dalloc(c, &c->adaptive, SDSAT_MAX_ADAPTIVE) &&
             dalloc(c, &c->tree_pos, rows) && dalloc(c, &c->tree_anc, rows) &&
@@ -672,8 +668,10 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
          dalloc(c, &c->pf_q, (size_t)pr * R) && dalloc(c, &c->pf_attn, (size_t)pr * R);
     for (int xs = 0; ok && xs < X_COUNT; ++xs)
       ok = dalloc(c, &c->pf_hi[xs], (size_t)pr * xcols[xs]) && dalloc(c, &c->pf_lo[xs], (size_t)pr * xcols[xs]) &&
-           make_xmap(&c->pf_xmap[xs][0], c->pf_hi[xs], pr, xcols[xs], 128) &&
-           make_xmap(&c->pf_xmap[xs][1], c->pf_lo[xs], pr, xcols[xs], 128);
+           make_xmap(&c->pf_xmap[0][xs][0], c->pf_hi[xs], pr, xcols[xs], 128) &&
+           make_xmap(&c->pf_xmap[0][xs][1], c->pf_lo[xs], pr, xcols[xs], 128) &&
+           make_xmap(&c->pf_xmap[1][xs][0], c->pf_hi[xs], pr, xcols[xs], 64) &&
+           make_xmap(&c->pf_xmap[1][xs][1], c->pf_lo[xs], pr, xcols[xs], 64);
   }
   if (!ok) {
     sdsat_destroy(c);
@@ -1065,21 +1063,21 @@ sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const
     const int rows = (M + 127) / 128 * 128;   // <= OP_MAX_M rows of the operand scratch
     PfGemmParams g;
     std::memset(&g, 0, sizeof(g));
-    if (!make_wmap(&g.tmap[0], w_dev, N, K) || !make_xmap(&g.tmap_x[0], c->xop_hi, rows, K, 128) ||
-        !make_xmap(&g.tmap_x[1], c->xop_lo, rows, K, 128))
+    if (!make_wmap(&g.tmap[0], w_dev, N, K) || !make_xmap(&g.tmap_x[0], c->xop_hi, rows, K, prefill_tok(M)) ||
+        !make_xmap(&g.tmap_x[1], c->xop_lo, rows, K, prefill_tok(M)))
       return SDSAT_ECUDA;
     g.map_mode = MAP_PLAIN;
     g.N = N;
     g.kc = (K + 63) / 64;
     g.n_wtiles = (N + 127) / 128;
-    g.n_tblocks = rows / 128;
     g.M = M;
     g.epi = EPI_STORE;
     g.out = y_dev;
     g.out_ld = N;
-    g.partials = c->pf_partials;
-    g.counters = c->pf_counters;
+    g.partials = c->partials;
+    g.counters = c->gemm_counters;
     g.err = c->err;
+    g.trace = next_trace(c, K_GEMM_OP);
     if (launch_split(x_dev, M, K, c->xop_hi, c->xop_lo, c->stream, c->pdl) != cudaSuccess) return SDSAT_ECUDA;
     return timed(c, K_GEMM_OP, [&] { return launch_prefill_gemm(g, c->num_sms, c->stream, c->pdl); }) == cudaSuccess
                ? SDSAT_OK
