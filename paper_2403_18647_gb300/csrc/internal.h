@@ -181,21 +181,18 @@ struct PfGemmParams {
   int M;                    // positions
   float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]
   int* counters;            // [2 * num_sms], zero between launches
-  int epi;                  // EPI_STORE, EPI_RESID or EPI_SWIGLU
-  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID)
+  int epi;                  // EPI_STORE, EPI_RESID, EPI_QKV or EPI_SWIGLU
+  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID; EPI_QKV: the rotated queries)
   int out_ld;
-  __nv_bfloat16* out_hi;    // EPI_SWIGLU: [M][out_ld] the down projection's operand
+  __nv_bfloat16* out_hi;    // [M][out_ld] the next GEMM's operand (EPI_SWIGLU; EPI_RESID with gain_next)
   __nv_bfloat16* out_lo;
-  uint32_t* err;
-  Trace trace;
-};
-cudaError_t prefill_prepare();
-int prefill_tok(int M);      // positions per tile of the GEMM over M positions: 64 or 128
-size_t prefill_partials(int num_sms);
-cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl);
-struct RopeKvParams {
-  const float* qkv;         // [M][3R]
-  float* qout;              // [M][R]
+  // RMSNorm folded into the GEMMs, as in GemmParams
+  const float* ssq_in;      // [M][ssq_ld] sums of h^2 per weight tile, or null (operand already normalised)
+  float* ssq_out;           // with gain_next: this GEMM's sums
+  const __nv_bfloat16* gain_next;
+  int ssq_ld, norm_dim;
+  float norm_eps;
+  // EPI_QKV
   __nv_bfloat16* k_layer;   // this layer's caches [B][H][cap][hd]
   __nv_bfloat16* v_layer;
   const int* len;
@@ -203,8 +200,12 @@ struct RopeKvParams {
   const float2* rope;
   int rope_len;
   uint32_t* err;
+  Trace trace;
 };
-cudaError_t launch_rope_kv(const RopeKvParams& p, int M, cudaStream_t st, bool pdl);
+cudaError_t prefill_prepare();
+int prefill_tok(int M);      // positions per tile of the GEMM over M positions: 64 or 128
+size_t prefill_partials(int num_sms);
+cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 
 // ---- embedding, acceptance, block building ------------------------------------
 // x = h * rsqrt(mean h^2 + eps) * g, stored as bf16 hi + lo (tokens != null: h = E[tokens] first)

@@ -24,10 +24,12 @@
 // their reduction overlaps the whole tiles that follow.
 // TOK = 64 for at most 64 positions: half the position traffic and half the split parts.
 //
-// Epilogues: store (q, k, v before RoPE), residual add (O and down projections), and
-// SiLU(gate) * up written as the down projection's bf16 hi + lo operand.  RMSNorm and
-// RoPE + the KV append are small row kernels here (the decode path folds them into the
-// GEMMs); attention is the causal flash-attention kernel at the end of attention.cu.
+// Epilogues: store; RoPE and the KV append (QKV); residual add (O and down projections), which
+// also emits the next RMSNorm's operand h * g and per-tile sums of h^2, as the decode GEMM
+// does, so that the consuming GEMM only scales its result by each position's factor; SiLU(gate)
+// * up as the down projection's bf16 hi + lo operand.  RMSNorm and RoPE as row kernels of their
+// own cost two more passes over the chunk's rows each (2047 positions: 34 us per RMSNorm, 59
+// us per RoPE + append).  Attention is the causal flash-attention kernel of attention.cu.
 #include <algorithm>
 
 #include "common.cuh"
@@ -39,8 +41,7 @@ constexpr int PF_W_BYTES = 128 * 128;                    // a CTA's 128 weight r
 constexpr int PF_CHUNK = 32;                             // positions per epilogue round
 constexpr int PF_EPI_WARPS = 8;                          // two per TMEM lane quarter
 constexpr int PF_THREADS = 64 + 32 * PF_EPI_WARPS;
-constexpr int PF_XROW = PF_CHUNK / 2 + 1;                // exchange row: half a round's positions, padded
-constexpr int PF_STAGING = 2 * 128 * PF_XROW;            // fp32 exchange of the two epilogue groups
+constexpr int PF_STAGING = 2 * 128 * PF_CHUNK;           // fp32 exchange of the two epilogue groups
 #ifndef SDSAT_PF_GROUP
 #define SDSAT_PF_GROUP 8
 #endif
@@ -58,7 +59,8 @@ struct PfCfg {
   static constexpr int ACC = 2 * TOK;                    // TMEM columns of one accumulator (hi, lo)
   static constexpr int ROUNDS = TOK / (2 * PF_CHUNK);    // epilogue rounds of each of the two warp groups
   static constexpr int NBAR = 2 * STAGES + 6;
-  static constexpr size_t SMEM = 1024 + (size_t)RING + PF_STAGING * 4 + NBAR * 8 + 64;
+  static constexpr size_t SMEM = 1024 + (size_t)RING + PF_STAGING * 4 + 2 * TOK * 4 + NBAR * 8 + 64;
+  static_assert(SMEM <= 232448, "shared memory of one CTA");
 };
 
 __device__ __forceinline__ void pf_tile_half_src(int map_mode, int rows_per_map, int t, int h, int& map, int& row) {
@@ -134,7 +136,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* stages = smem;
   float* staging = reinterpret_cast<float*>(smem + C::RING);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + PF_STAGING);
+  float* s_inv = staging + PF_STAGING;    // [2][TOK] RMSNorm factors of a tile's positions
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_inv + 2 * TOK);
   uint64_t* full = bars;                  // rank 0: both CTAs' weights and positions landed (TMA)
   uint64_t* empty = bars + S;     // the stage was consumed by the tensor cores
   uint64_t* acc_full = bars + 2 * S;   // [2] accumulator ready
@@ -300,11 +303,15 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     const int r = e * 32 + lane;         // the CTA's weight row
     const int tid = threadIdx.x - 64;
     constexpr int NE = 32 * PF_EPI_WARPS;
-    float* xch = staging + grp * 128 * PF_XROW;
+    // exchange between the group's 128 rows: element (row, j) at row * 32 + (j ^ lane of the
+    // row), so that a warp's rows fall on different banks
+    float* xch = staging + grp * 128 * PF_CHUNK;
+    int round = 0;
     const uint32_t acc_empty0 = mapa_shared(smem_u32(acc_empty), 0);
     const int U = p.sk_tiles * p.kc;
     pdl_wait();   // residual rows and outputs belong to the previous kernels' results
     if (p.trace.rec) t_wait = globaltimer_ns();
+    const int len0 = p.epi == EPI_QKV ? __ldcg(p.len + p.seq) : 0;
     int seg = 0;
     PfWalk w(p, pair);
     for (; w.next(); ++seg) {
@@ -313,6 +320,19 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
       const int wt = 2 * wp + rank;
       const int buf = seg & 1;
       const int mt = tb * TOK;   // the tile's first position
+      const float* inv = s_inv + (seg & 1) * TOK;
+      if (p.ssq_in) {
+        // RMSNorm factors of the tile's positions while the tensor cores work: eight lanes sum a
+        // position's parts, in a fixed order (read after the barrier below)
+        for (int c = tid >> 3; c < TOK; c += NE / 8) {
+          const float* src = p.ssq_in + (size_t)min(mt + c, p.M - 1) * p.ssq_ld;
+          float q = 0.f;
+          for (int t = tid & 7; t < p.ssq_ld; t += 8) q += __ldcg(src + t);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+          if ((tid & 7) == 0) s_inv[(seg & 1) * TOK + c] = 1.0f / sqrtf(q / (float)p.norm_dim + p.norm_eps);
+        }
+      }
       const bool got = named_bar_and(1, NE, mbar_wait_bounded(&acc_full[buf], (seg >> 1) & 1, abort_flag, p.err));
       if (!got) break;
       tc_fence_after();
@@ -426,21 +446,26 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             }
           }
         }
+        if (p.ssq_in) {
+#pragma unroll
+          for (int j = 0; j < PF_CHUNK; ++j) y[j] *= inv[c0 + j];
+        }
         if (p.epi == EPI_SWIGLU) {
           // tile rows 0-63: gate features 64*wt + r, rows 64-127: the matching up features; the
           // gate thread takes the round's first 16 positions, the up thread the other 16
           const int f = 64 * wt + (r & 63);
           const bool gate = r < 64;
 #pragma unroll
-          for (int j = 0; j < PF_CHUNK / 2; ++j) xch[r * PF_XROW + j] = gate ? y[16 + j] : y[j];
+          for (int j = 0; j < PF_CHUNK / 2; ++j) xch[r * PF_CHUNK + (j ^ lane)] = gate ? y[16 + j] : y[j];
           named_bar_sync(2 + grp, 128);
-          const float* other = xch + (r ^ 64) * PF_XROW;
+          const float* other = xch + (r ^ 64) * PF_CHUNK;
           if (wt < p.n_wtiles && f < p.N) {
 #pragma unroll
             for (int j = 0; j < PF_CHUNK / 2; ++j) {
               const int m = m0 + (gate ? j : 16 + j);
               if (m < p.M) {
-                const float g = gate ? y[j] : other[j], up = gate ? other[j] : y[16 + j];
+                const float x = other[j ^ lane];
+                const float g = gate ? y[j] : x, up = gate ? x : y[16 + j];
                 const float a = g / (1.0f + expf(-g)) * up;
                 const __nv_bfloat16 h = __float2bfloat16_rn(a);
                 p.out_hi[(size_t)m * p.out_ld + f] = h;
@@ -449,20 +474,91 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             }
           }
           named_bar_sync(2 + grp, 128);
-        } else {
-          const int n = 128 * wt + r;
-          if (n < p.N) {
-            if (p.epi == EPI_RESID) {
-              float hv[PF_CHUNK];
+        } else if (p.epi == EPI_QKV) {
+          // The tile lies in one of q, k, v and holds whole heads.  RoPE (rotate-half) pairs row
+          // r with row r ^ hd/2; position m0 + j sits at slot (and position) len + m0 + j.
+          const int R = p.rows_per_map, g = 128 * wt;
+          const int which = (g >= R) + (g >= 2 * R);
+          const int f = g - which * R + r, half = p.hd >> 1, i = f & (p.hd - 1);
+          const int slot0 = len0 + m0;
+          if (which < 2 && wt < p.n_wtiles) {
+#pragma unroll
+            for (int j = 0; j < PF_CHUNK; ++j) xch[r * PF_CHUNK + (j ^ lane)] = y[j];
+            named_bar_sync(2 + grp, 128);
+            const float* other = xch + (r ^ half) * PF_CHUNK;
+            const float sgn = i < half ? -1.f : 1.f;
+            const float2* cs = p.rope + (i & (half - 1));
+#pragma unroll
+            for (int j = 0; j < PF_CHUNK; ++j) {
+              const float2 t = __ldg(cs + (size_t)min(slot0 + j, p.rope_len - 1) * half);
+              y[j] = y[j] * t.x + sgn * (other[j ^ lane] * t.y);
+            }
+            named_bar_sync(2 + grp, 128);
+          }
+          if (wt < p.n_wtiles) {
+            const int valid = min(PF_CHUNK, p.M - m0);
+            if (which == 0) {
+              float* dst = p.out + (size_t)m0 * p.out_ld + f;
 #pragma unroll
               for (int j = 0; j < PF_CHUNK; ++j)
-                hv[j] = (m0 + j < p.M) ? __ldcg(p.out + (size_t)(m0 + j) * p.out_ld + n) : 0.f;
+                if (j < valid) dst[(size_t)j * p.out_ld] = y[j];
+            } else {
+              const int fits = min(valid, p.cap - slot0);
+              __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
+                                   ((size_t)(p.seq * p.H + f / p.hd) * p.cap + slot0) * p.hd + i;
 #pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j) y[j] += hv[j];
+              for (int j = 0; j < PF_CHUNK; ++j)
+                if (j < fits) dst[j * p.hd] = __float2bfloat16_rn(y[j]);
+              if (r == 0 && fits < valid) set_error(p.err, ERR_CAPACITY);
+              if (r == 0 && slot0 + valid > p.rope_len) set_error(p.err, ERR_POSITION);
+            }
+          }
+        } else {
+          const int n = 128 * wt + r;
+          const bool in = n < p.N;
+          float* dst = p.out + (size_t)m0 * p.out_ld + n;
+          const int valid = in ? min(PF_CHUNK, p.M - m0) : 0;
+          if (p.epi == EPI_RESID) {
+            float hv[PF_CHUNK];
+#pragma unroll
+            for (int j = 0; j < PF_CHUNK; ++j) hv[j] = j < valid ? __ldcg(dst + (size_t)j * p.out_ld) : 0.f;
+#pragma unroll
+            for (int j = 0; j < PF_CHUNK; ++j) y[j] += hv[j];
+          }
+#pragma unroll
+          for (int j = 0; j < PF_CHUNK; ++j)
+            if (j < valid) dst[(size_t)j * p.out_ld] = y[j];
+          if (p.gain_next) {
+            // the next RMSNorm's operand h * g, and this weight tile's sum of h^2 per position:
+            // halving exchanges leave position j's sum over the warp's rows on lane j, the
+            // group's four warps add up through shared memory (two buffers, one barrier)
+            const float gn = in ? __bfloat162float(p.gain_next[n]) : 0.f;
+            const size_t o = (size_t)m0 * p.out_ld + n;
+#pragma unroll
+            for (int j = 0; j < PF_CHUNK; ++j) {
+              const float x = y[j] * gn;
+              const __nv_bfloat16 h = __float2bfloat16_rn(x);
+              if (j < valid) {
+                p.out_hi[o + (size_t)j * p.out_ld] = h;
+                p.out_lo[o + (size_t)j * p.out_ld] = __float2bfloat16_rn(x - __bfloat162float(h));
+              }
+              y[j] = j < valid ? y[j] * y[j] : 0.f;
             }
 #pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j)
-              if (m0 + j < p.M) p.out[(size_t)(m0 + j) * p.out_ld + n] = y[j];
+            for (int o2 = 16; o2 > 0; o2 >>= 1) {
+              const bool up = lane & o2;
+#pragma unroll
+              for (int j = 0; j < o2; ++j) {
+                const float send = up ? y[j] : y[j + o2], keep = up ? y[j + o2] : y[j];
+                y[j] = keep + __shfl_xor_sync(0xffffffffu, send, o2);
+              }
+            }
+            float* part = xch + (round++ & 1) * 128;
+            part[e * 32 + lane] = y[0];
+            named_bar_sync(2 + grp, 128);
+            if (e == 0 && m0 + lane < p.M && wt < p.n_wtiles)
+              p.ssq_out[(size_t)(m0 + lane) * p.ssq_ld + wt] =
+                  (part[lane] + part[32 + lane]) + (part[64 + lane] + part[96 + lane]);
           }
         }
       }
@@ -537,51 +633,6 @@ cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, b
       pf_config(tok, std::min(P, std::max(p.sk_pairs, T - p.sk_tiles)), st, pdl, attr);
   return tok == 64 ? cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<64>, p)
                    : cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<128>, p);
-}
-
-// ---- RoPE + KV append of a prefill chunk ------------------------------------------------
-// qkv [M][3R] (q | k | v, head-major columns) -> q rotated into qout [M][R]; k rotated and v
-// into the cache slots len[seq] + m at position len[seq] + m (rotate-half pairing (i, i + hd/2)).
-__global__ void __launch_bounds__(256) rope_kv_kernel(RopeKvParams p) {
-  pdl_wait();
-  pdl_trigger();
-  const int m = blockIdx.x;
-  const int R = p.H * p.hd, half = p.hd >> 1;
-  const int slot = __ldcg(p.len + p.seq) + m;
-  int pos = slot;
-  if (pos >= p.rope_len) {
-    if (threadIdx.x == 0) set_error(p.err, ERR_POSITION);
-    pos = p.rope_len - 1;
-  }
-  const bool fits = slot < p.cap;
-  if (!fits && threadIdx.x == 0) set_error(p.err, ERR_CAPACITY);
-  const float* row = p.qkv + (size_t)m * 3 * R;
-  for (int idx = threadIdx.x; idx < R; idx += blockDim.x) {
-    const int h = idx / p.hd, i = idx % p.hd;
-    const int partner = i < half ? idx + half : idx - half;
-    const float2 cs = p.rope[(size_t)pos * half + (i % half)];
-    const float qa = row[idx], qp = row[partner];
-    const float ka = row[R + idx], kp = row[R + partner];
-    p.qout[(size_t)m * R + idx] = i < half ? qa * cs.x - qp * cs.y : qa * cs.x + qp * cs.y;
-    if (fits) {
-      const size_t o = (((size_t)p.seq * p.H + h) * p.cap + slot) * p.hd + i;
-      p.k_layer[o] = __float2bfloat16_rn(i < half ? ka * cs.x - kp * cs.y : ka * cs.x + kp * cs.y);
-      p.v_layer[o] = __float2bfloat16_rn(row[2 * R + idx]);
-    }
-  }
-}
-
-cudaError_t launch_rope_kv(const RopeKvParams& p, int M, cudaStream_t st, bool pdl) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(M);
-  cfg.blockDim = dim3(256);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, rope_kv_kernel, p);
 }
 
 }  // namespace sdsat

@@ -14,6 +14,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "sdsat.h"
@@ -88,12 +89,12 @@ struct LayerMaps {
 enum KClass : int {
   K_RMSNORM = 0, K_GEMM_QKV, K_ATTENTION, K_GEMM_O, K_GEMM_GATEUP, K_GEMM_DOWN, K_GEMM_LM_HEAD, K_ACCEPT,
   K_BUILD_BLOCK, K_KV_COMMIT, K_PREFILL_COMMIT, K_GEMM_OP, K_ATTENTION_OP, K_TREE_PREP, K_TREE_COMPACT,
-  K_PF_GEMM, K_PF_ROPE_KV, K_PF_ATTENTION, K_COUNT
+  K_PF_GEMM, K_PF_ATTENTION, K_COUNT
 };
 const char* const KCLASS_NAME[K_COUNT] = {"rmsnorm", "gemm_qkv", "attention", "gemm_o", "gemm_gateup", "gemm_down",
                                           "gemm_lm_head", "accept", "build_block", "kv_commit", "prefill_commit",
                                           "gemm_op", "attention_op", "tree_prep", "tree_compact", "prefill_gemm",
-                                          "prefill_rope_kv", "prefill_attention"};
+                                          "prefill_attention"};
 
 constexpr int MAX_GEMM_TILES = 1 << 16;
 constexpr int OP_MAX_K = 32768;   // limits of sdsat_op_gemm (its operand scratch is sized at create)
@@ -133,7 +134,7 @@ struct sdsat_ctx {
   uint32_t* err = nullptr;
   // prefill workspaces (chunks of up to PF_ROWS positions; allocated with the weights)
   float* pf_h = nullptr;         // [PF_ROWS][d] residual stream
-  float* pf_qkv = nullptr;       // [PF_ROWS][3R] projections before RoPE
+  float* pf_ssq = nullptr;       // [PF_ROWS][ssq_ld] per-tile sums of h^2
   float* pf_q = nullptr;         // [PF_ROWS][R] rotated queries
   float* pf_attn = nullptr;      // [PF_ROWS][R] attention output
   __nv_bfloat16* pf_hi[X_COUNT] = {};   // GEMM operands [PF_ROWS][K] (normed x, attention, act)
@@ -409,12 +410,20 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
   cudaStream_t st = c->stream;
   const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
   const int xi = prefill_tok(M) == 64;
-  auto norm = [&](const int32_t* toks, const void* gain) {
-    return timed(c, K_RMSNORM, [&] {
-      return launch_rmsnorm(toks, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->pf_h, d, M,
-                            static_cast<const __nv_bfloat16*>(gain), cf.rms_eps, c->pf_hi[X_NORM], c->pf_lo[X_NORM],
-                            c->err, st, c->pdl);
-    });
+  // RMSNorm folded into the GEMMs as in forward(): O and down emit the next operand and the
+  // sums of squares, gate/up and the next QKV scale by the factor
+  auto fold_in = [&](PfGemmParams& g) {
+    g.ssq_in = c->pf_ssq;
+    g.ssq_ld = c->ssq_ld;
+    g.norm_dim = d;
+    g.norm_eps = cf.rms_eps;
+  };
+  auto fold_out = [&](PfGemmParams& g, const void* gain) {
+    g.gain_next = static_cast<const __nv_bfloat16*>(gain);
+    g.out_hi = c->pf_hi[X_NORM];
+    g.out_lo = c->pf_lo[X_NORM];
+    g.ssq_out = c->pf_ssq;
+    g.ssq_ld = c->ssq_ld;
   };
   auto base = [&](int xsrc, int K) {
     PfGemmParams g;
@@ -432,7 +441,12 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     g.trace = next_trace(c, K_PF_GEMM);
     return timed(c, K_PF_GEMM, [&] { return launch_prefill_gemm(g, c->num_sms, st, c->pdl); });
   };
-  if (norm(tokens, c->layers[0].attn_norm) != cudaSuccess) return SDSAT_ECUDA;
+  if (timed(c, K_RMSNORM, [&] {
+        return launch_rmsnorm(tokens, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->pf_h, d, M,
+                              static_cast<const __nv_bfloat16*>(c->layers[0].attn_norm), cf.rms_eps,
+                              c->pf_hi[X_NORM], c->pf_lo[X_NORM], c->err, st, c->pdl);
+      }) != cudaSuccess)
+    return SDSAT_ECUDA;
   for (int l = 0; l < L; ++l) {
     const LayerMaps& mp = c->maps[l];
     PfGemmParams gq = base(X_NORM, d);
@@ -443,13 +457,20 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gq.rows_per_map = R;
     gq.N = 3 * R;
     gq.n_wtiles = 3 * R / 128;
-    gq.epi = EPI_STORE;
-    gq.out = c->pf_qkv;
-    gq.out_ld = 3 * R;
+    gq.epi = EPI_QKV;
+    gq.out = c->pf_q;
+    gq.out_ld = R;
+    gq.k_layer = kv->k + l * layer_elems;
+    gq.v_layer = kv->v + l * layer_elems;
+    gq.len = kv->len;
+    gq.seq = seq;
+    gq.H = H;
+    gq.hd = hd;
+    gq.cap = kv->cap;
+    gq.rope = c->rope;
+    gq.rope_len = cf.max_position;
+    if (l > 0) fold_in(gq);
     if (gemm(gq) != cudaSuccess) return SDSAT_ECUDA;
-    RopeKvParams rp{c->pf_qkv, c->pf_q, kv->k + l * layer_elems, kv->v + l * layer_elems, kv->len, seq, H, hd,
-                    kv->cap, c->rope, cf.max_position, c->err};
-    if (timed(c, K_PF_ROPE_KV, [&] { return launch_rope_kv(rp, M, st, c->pdl); }) != cudaSuccess) return SDSAT_ECUDA;
     // causal attention of the chunk's positions over the cache
     PfAttnParams a;
     std::memset(&a, 0, sizeof(a));
@@ -479,8 +500,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     go.epi = EPI_RESID;
     go.out = c->pf_h;
     go.out_ld = d;
+    fold_out(go, c->layers[l].ffn_norm);
     if (gemm(go) != cudaSuccess) return SDSAT_ECUDA;
-    if (norm(nullptr, c->layers[l].ffn_norm) != cudaSuccess) return SDSAT_ECUDA;
     PfGemmParams gg = base(X_NORM, d);
     gg.tmap[0] = mp.gate;
     gg.tmap[1] = mp.up;
@@ -491,6 +512,7 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gg.out_hi = c->pf_hi[X_FFN];
     gg.out_lo = c->pf_lo[X_FFN];
     gg.out_ld = F;
+    fold_in(gg);
     if (gemm(gg) != cudaSuccess) return SDSAT_ECUDA;
     PfGemmParams gd = base(X_FFN, F);
     gd.tmap[0] = mp.down;
@@ -500,8 +522,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gd.epi = EPI_RESID;
     gd.out = c->pf_h;
     gd.out_ld = d;
+    if (l + 1 < L) fold_out(gd, c->layers[l + 1].attn_norm);
     if (gemm(gd) != cudaSuccess) return SDSAT_ECUDA;
-    if (l + 1 < L && norm(nullptr, c->layers[l + 1].attn_norm) != cudaSuccess) return SDSAT_ECUDA;
   }
   return timed(c, K_PREFILL_COMMIT, [&] { return launch_add_len(kv->len, seq, M, kv->cap, c->err, st, c->pdl); }) ==
                  cudaSuccess
@@ -646,7 +668,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   c->ssq_ld = (d + 127) / 128;
   bool ok = dalloc(c, &c->rope, rope.size()) && dalloc(c, &c->h, (size_t)rows * d) &&
             dalloc(c, &c->qbuf, (size_t)rows * R) && dalloc(c, &c->attn, (size_t)rows * R) &&
-            dalloc(c, &c->act, (size_t)rows * F) && dalloc(c, &c->partials, std::max((size_t)c->num_sms * 2 * 2 * 64 * 128, prefill_partials(c->num_sms))) &&
+            dalloc(c, &c->act, (size_t)rows * F) &&
+            dalloc(c, &c->partials, std::max((size_t)c->num_sms * 2 * 2 * 64 * 128, prefill_partials(c->num_sms))) &&
             dalloc(c, &c->gemm_counters, MAX_GEMM_TILES) &&
             dalloc(c, &c->acc_targets, rows) &&
             dalloc(c, &c->acc_counters, rows) && dalloc(c, &c->adaptive, SDSAT_MAX_ADAPTIVE) &&
@@ -663,15 +686,30 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
            make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], 16 << mi);
   }
   if (ok && c->has_weights) {
-    const int pr = PF_ROWS;
-    ok = dalloc(c, &c->pf_h, (size_t)pr * d) && dalloc(c, &c->pf_qkv, (size_t)pr * 3 * R) &&
-         dalloc(c, &c->pf_q, (size_t)pr * R) && dalloc(c, &c->pf_attn, (size_t)pr * R);
+    // the prefill workspaces in one allocation (a cudaMalloc each cost 30-50 us of sdsat_create)
+    const size_t pr = PF_ROWS;
+    uint8_t* arena = nullptr;
+    size_t used = 0;
+    for (int pass = 0; ok && pass < 2; ++pass) {
+      if (pass) ok = dalloc(c, &arena, used);
+      used = 0;
+      auto take = [&](auto** p, size_t count) {
+        if (arena) *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(arena + used);
+        used += (count * sizeof(**p) + 255) / 256 * 256;
+      };
+      take(&c->pf_h, pr * d);
+      take(&c->pf_ssq, pr * c->ssq_ld);
+      take(&c->pf_q, pr * R);
+      take(&c->pf_attn, pr * R);
+      for (int xs = 0; xs < X_COUNT; ++xs) {
+        take(&c->pf_hi[xs], pr * xcols[xs]);
+        take(&c->pf_lo[xs], pr * xcols[xs]);
+      }
+    }
     for (int xs = 0; ok && xs < X_COUNT; ++xs)
-      ok = dalloc(c, &c->pf_hi[xs], (size_t)pr * xcols[xs]) && dalloc(c, &c->pf_lo[xs], (size_t)pr * xcols[xs]) &&
-           make_xmap(&c->pf_xmap[0][xs][0], c->pf_hi[xs], pr, xcols[xs], 128) &&
-           make_xmap(&c->pf_xmap[0][xs][1], c->pf_lo[xs], pr, xcols[xs], 128) &&
-           make_xmap(&c->pf_xmap[1][xs][0], c->pf_hi[xs], pr, xcols[xs], 64) &&
-           make_xmap(&c->pf_xmap[1][xs][1], c->pf_lo[xs], pr, xcols[xs], 64);
+      for (int i = 0; ok && i < 2; ++i)
+        ok = make_xmap(&c->pf_xmap[i][xs][0], c->pf_hi[xs], PF_ROWS, xcols[xs], 128 >> i) &&
+             make_xmap(&c->pf_xmap[i][xs][1], c->pf_lo[xs], PF_ROWS, xcols[xs], 128 >> i);
   }
   if (!ok) {
     sdsat_destroy(c);
