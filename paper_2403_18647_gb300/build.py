@@ -16,7 +16,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsdsat.so")
-SOURCES = ["gemm.cu", "attention.cu", "accept.cu", "prefill.cu", "sdsat.cu", "noalloc.cu"]
+SOURCES = ["gemm.cu", "attention.cu", "accept.cu", "prefill.cu", "prefill_attention.cu", "sdsat.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include")]

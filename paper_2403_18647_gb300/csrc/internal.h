@@ -146,21 +146,21 @@ void attention_grid(int pairs, const int* maxc, int cs_cap, int num_sms, int* cs
 
 // Causal attention of M consecutive prompt positions of sequence seq (a prefill chunk at
 // slots len[seq] .. len[seq]+M-1, already in the cache) over the cache: position i sees
-// slots [0, len + i].  One CTA per (head, 64-position block).
+// slots [0, len + i].
 struct PfAttnParams {
   CUtensorMap kmap, vmap;   // the caches, as AttnParams
+  CUtensorMap qmap[2];      // rotated queries, bf16 hi / lo [rows][H*hd], boxes of 64 x 128
   int row0;                 // first cache row of this layer
-  const float* Q;           // [M][q_ld] rotated queries, head h at column h*hd
-  int q_ld;
   const int* len;
   int seq, M, H, hd, cap;
-  float* out;               // [M][out_ld] fp32
+  int tiles;                // set by launch_prefill_attention: tiles of 128 positions per CTA (1 or 2)
   int out_ld;
-  __nv_bfloat16* out_hi;    // the same as bf16 hi + lo (the O projection's operand)
+  __nv_bfloat16* out_hi;    // [M][out_ld] the O projection's operand
   __nv_bfloat16* out_lo;
   uint32_t* err;
 };
-cudaError_t launch_prefill_attention(const PfAttnParams& p, cudaStream_t st, bool pdl);
+cudaError_t prefill_attention_prepare();
+cudaError_t launch_prefill_attention(PfAttnParams& p, int num_sms, cudaStream_t st, bool pdl);
 
 // ---- prefill (prompt chunks of up to PF_ROWS positions) -------------------------
 #ifndef SDSAT_PF_ROWS
@@ -182,9 +182,10 @@ struct PfGemmParams {
   float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]
   int* counters;            // [2 * num_sms], zero between launches
   int epi;                  // EPI_STORE, EPI_RESID, EPI_QKV or EPI_SWIGLU
-  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID; EPI_QKV: the rotated queries)
+  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID)
   int out_ld;
-  __nv_bfloat16* out_hi;    // [M][out_ld] the next GEMM's operand (EPI_SWIGLU; EPI_RESID with gain_next)
+  __nv_bfloat16* out_hi;    // [M][out_ld] bf16 hi + lo: the next GEMM's operand (EPI_SWIGLU; EPI_RESID
+                            // with gain_next), the rotated queries (EPI_QKV)
   __nv_bfloat16* out_lo;
   // RMSNorm folded into the GEMMs, as in GemmParams
   const float* ssq_in;      // [M][ssq_ld] sums of h^2 per weight tile, or null (operand already normalised)

@@ -29,7 +29,7 @@
 // does, so that the consuming GEMM only scales its result by each position's factor; SiLU(gate)
 // * up as the down projection's bf16 hi + lo operand.  RMSNorm and RoPE as row kernels of their
 // own cost two more passes over the chunk's rows each (2047 positions: 34 us per RMSNorm, 59
-// us per RoPE + append).  Attention is the causal flash-attention kernel of attention.cu.
+// us per RoPE + append).  Attention is prefill_attention.cu.
 #include <algorithm>
 
 #include "common.cuh"
@@ -498,10 +498,14 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
           if (wt < p.n_wtiles) {
             const int valid = min(PF_CHUNK, p.M - m0);
             if (which == 0) {
-              float* dst = p.out + (size_t)m0 * p.out_ld + f;
+              const size_t o = (size_t)m0 * p.out_ld + f;
 #pragma unroll
               for (int j = 0; j < PF_CHUNK; ++j)
-                if (j < valid) dst[(size_t)j * p.out_ld] = y[j];
+                if (j < valid) {
+                  const __nv_bfloat16 h = __float2bfloat16_rn(y[j]);
+                  p.out_hi[o + (size_t)j * p.out_ld] = h;
+                  p.out_lo[o + (size_t)j * p.out_ld] = __float2bfloat16_rn(y[j] - __bfloat162float(h));
+                }
             } else {
               const int fits = min(valid, p.cap - slot0);
               __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +

@@ -135,8 +135,8 @@ struct sdsat_ctx {
   // prefill workspaces (chunks of up to PF_ROWS positions; allocated with the weights)
   float* pf_h = nullptr;         // [PF_ROWS][d] residual stream
   float* pf_ssq = nullptr;       // [PF_ROWS][ssq_ld] per-tile sums of h^2
-  float* pf_q = nullptr;         // [PF_ROWS][R] rotated queries
-  float* pf_attn = nullptr;      // [PF_ROWS][R] attention output
+  __nv_bfloat16 *pf_qhi = nullptr, *pf_qlo = nullptr;   // [PF_ROWS][R] rotated queries
+  CUtensorMap pf_qmap[2];               // boxes of 64 x 128
   __nv_bfloat16* pf_hi[X_COUNT] = {};   // GEMM operands [PF_ROWS][K] (normed x, attention, act)
   __nv_bfloat16* pf_lo[X_COUNT] = {};
   CUtensorMap pf_xmap[2][X_COUNT][2];   // boxes of 64 x 128 and 64 x 64
@@ -458,7 +458,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gq.N = 3 * R;
     gq.n_wtiles = 3 * R / 128;
     gq.epi = EPI_QKV;
-    gq.out = c->pf_q;
+    gq.out_hi = c->pf_qhi;
+    gq.out_lo = c->pf_qlo;
     gq.out_ld = R;
     gq.k_layer = kv->k + l * layer_elems;
     gq.v_layer = kv->v + l * layer_elems;
@@ -476,21 +477,20 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     std::memset(&a, 0, sizeof(a));
     a.kmap = kv->kmap;
     a.vmap = kv->vmap;
+    a.qmap[0] = c->pf_qmap[0];
+    a.qmap[1] = c->pf_qmap[1];
     a.row0 = l * kv->batch * H * kv->cap;
-    a.Q = c->pf_q;
-    a.q_ld = R;
     a.len = kv->len;
     a.seq = seq;
     a.M = M;
     a.H = H;
     a.hd = hd;
     a.cap = kv->cap;
-    a.out = c->pf_attn;
     a.out_ld = R;
     a.out_hi = c->pf_hi[X_ATTN];
     a.out_lo = c->pf_lo[X_ATTN];
     a.err = c->err;
-    if (timed(c, K_PF_ATTENTION, [&] { return launch_prefill_attention(a, st, c->pdl); }) != cudaSuccess)
+    if (timed(c, K_PF_ATTENTION, [&] { return launch_prefill_attention(a, c->num_sms, st, c->pdl); }) != cudaSuccess)
       return SDSAT_ECUDA;
     PfGemmParams go = base(X_ATTN, R);
     go.tmap[0] = mp.o;
@@ -621,7 +621,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   }
   if (cudaGetDevice(&c->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
-      gemm_prepare() != cudaSuccess || attention_prepare() != cudaSuccess || prefill_prepare() != cudaSuccess) {
+      gemm_prepare() != cudaSuccess || attention_prepare() != cudaSuccess || prefill_prepare() != cudaSuccess ||
+      prefill_attention_prepare() != cudaSuccess) {
     delete c;
     return SDSAT_ECUDA;
   }
@@ -686,7 +687,7 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
            make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], 16 << mi);
   }
   if (ok && c->has_weights) {
-    // the prefill workspaces in one allocation (a cudaMalloc each cost 30-50 us of sdsat_create)
+    // the prefill workspaces in one allocation
     const size_t pr = PF_ROWS;
     uint8_t* arena = nullptr;
     size_t used = 0;
@@ -699,13 +700,15 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
       };
       take(&c->pf_h, pr * d);
       take(&c->pf_ssq, pr * c->ssq_ld);
-      take(&c->pf_q, pr * R);
-      take(&c->pf_attn, pr * R);
+      take(&c->pf_qhi, pr * R);
+      take(&c->pf_qlo, pr * R);
       for (int xs = 0; xs < X_COUNT; ++xs) {
         take(&c->pf_hi[xs], pr * xcols[xs]);
         take(&c->pf_lo[xs], pr * xcols[xs]);
       }
     }
+    ok = ok && make_xmap(&c->pf_qmap[0], c->pf_qhi, PF_ROWS, R, 128) &&
+         make_xmap(&c->pf_qmap[1], c->pf_qlo, PF_ROWS, R, 128);
     for (int xs = 0; ok && xs < X_COUNT; ++xs)
       for (int i = 0; ok && i < 2; ++i)
         ok = make_xmap(&c->pf_xmap[i][xs][0], c->pf_hi[xs], PF_ROWS, xcols[xs], 128 >> i) &&
