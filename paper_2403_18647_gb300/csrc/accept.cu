@@ -8,8 +8,8 @@
 // 1 + m (the rejected rows, and in draft step 1 the adaptive-token rows, are
 // rolled back by not being committed).
 //
-// One CTA per block row selects that row's target; the last CTA of a sequence
-// (per-sequence counter, no waiting) runs the prefix scan and the commit.
+// One thread-block cluster per block row selects that row's target; the last row of a
+// sequence (per-sequence counter, no waiting) runs the prefix scan and the commit.
 //
 // Tree blocks (Sec. 2.1.2): the rows are the nodes of a draft tree in
 // topological order (parent[j] < j, row 0 the root).  Row j sits at position
@@ -18,6 +18,8 @@
 // deep ones) ends the accepted path n_0 = 0, ..., n_m.  Its targets are
 // emitted, and a compaction kernel moves the path's K and V rows to the slots
 // len + 1 .. len + m before len advances by 1 + m.
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -70,37 +72,122 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32
   }
 }
 
-// ---- block-wide reductions (1024 threads) -----------------------------------------
-constexpr int ACC_THREADS = 1024;
-constexpr int ACC_EPT = 32;   // logits per thread in the nucleus kernel (vocab <= 32768)
+// ---- the row's cluster -------------------------------------------------------------------
+// One thread-block cluster per row: p.cs CTAs of ACC_THREADS threads; thread t of rank r owns
+// the ids [ACC_SPAN r + ACC_EPT t, + ACC_EPT) (ascending id order is rank, thread, slot order).
+// One CTA per row (1024 threads of 32 ids) left most SMs idle and ran its chain of dependent
+// steps on four times the work per thread.  us per call, 32016 logits a row, one CTA per row ->
+// a cluster: 24 rows, top-p 0.95, T 0.2: 48.4 -> 22.5; with top-k 10: 34.5 -> 16.7; T 1 (row-wide
+// searches): 101 -> 47; greedy 7.1 -> 5.0; 64 rows (512 CTAs, more than one wave): 48 -> 36, T 1:
+// 101 -> 93, greedy 7.35 -> 7.4.  What is left is the chain of barriers, not bytes (3 MB).
+// A sum over the row: the warps' totals meet in shared
+// memory, warp 0 writes the CTA's total into every CTA of the cluster (distributed shared
+// memory), and after one cluster barrier each warp reads the cluster's totals locally.  (Every
+// warp reading every warp's total remotely was 15 us a sum with 24 rows.)  Two buffers
+// alternate: one is written again only after the next barrier, which no CTA passes before
+// every CTA has read it.
+constexpr int ACC_THREADS = 512;
+constexpr int ACC_EPT = 8;
+constexpr int ACC_SPAN = ACC_THREADS * ACC_EPT;   // 4096 ids per CTA, vocab <= 32768
+constexpr int ACC_WARPS = ACC_THREADS / 32;
+constexpr int ACC_CS = 8;                         // most CTAs of a row
+constexpr int ACC_WORDS = 5;                      // 64-bit words of one warp's slot
 
-__device__ __forceinline__ uint64_t block_sum_u64(uint64_t v, uint64_t* red) {
+struct AccSlots {
+  unsigned long long w[2][ACC_WARPS * ACC_WORDS];   // this CTA's warps
+  unsigned long long c[2][ACC_CS * ACC_WORDS];      // the cluster's CTAs, written by each of them
+};
+
+__device__ __forceinline__ void st_dsmem_u64(uint32_t addr, uint64_t v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// a warp's total of per-thread sums below 2^29
+__device__ __forceinline__ uint64_t warp_total(uint32_t v) {
+  const uint64_t hi = __reduce_add_sync(0xffffffffu, v >> 12);
+  return (hi << 12) + __reduce_add_sync(0xffffffffu, v & 4095u);
+}
+
+struct Row {   // the row's cluster, seen from one thread
+  AccSlots* slots;
+  int cs, rank, ph;
+  // v[n]: this warp's values (every lane); afterwards combine() of them over the row, and with
+  // `before` the sum of word 0 over the warps that come before this one in id order
+  template <int N, typename F>
+  __device__ void reduce(uint64_t (&v)[N], uint64_t identity, F combine, uint64_t* before = nullptr) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned long long* mine = slots->w[ph & 1];
+    unsigned long long* all = slots->c[ph & 1];
+    ++ph;
+    if (lane == 0)
+#pragma unroll
+      for (int n = 0; n < N; ++n) mine[w * N + n] = v[n];
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        uint64_t t = lane < ACC_WARPS ? mine[lane * N + n] : identity;
+#pragma unroll
+        for (int o = ACC_WARPS / 2; o > 0; o >>= 1) t = combine(t, (uint64_t)__shfl_xor_sync(0xffffffffu, t, o));
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (lane < cs) st_dsmem_u64(mapa_shared(smem_u32(&all[rank * N + n]), lane), t);
+      }
+    }
+    cluster_sync_all();
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      uint64_t t = lane < cs ? all[lane * N + n] : identity;
+      if (n == 0 && before)   // earlier CTAs, then earlier warps of this one
+        *before = warp_sum_u64((lane < rank ? t : 0) + (lane < w ? mine[lane * N] : 0));
+#pragma unroll
+      for (int o = ACC_CS / 2; o > 0; o >>= 1) t = combine(t, (uint64_t)__shfl_xor_sync(0xffffffffu, t, o));
+      v[n] = __shfl_sync(0xffffffffu, t, 0);
+    }
+  }
+  template <int N>
+  __device__ void sum(uint64_t (&v)[N], uint64_t* before = nullptr) {
+    reduce<N>(v, 0, [](uint64_t a, uint64_t b) { return a + b; }, before);
+  }
+  __device__ uint64_t largest(uint64_t warp_value) {
+    uint64_t v[1] = {warp_value};
+    reduce<1>(v, 0, [](uint64_t a, uint64_t b) { return a > b ? a : b; });
+    return v[0];
+  }
+  __device__ uint64_t sum(uint64_t warp_value) {
+    uint64_t v[1] = {warp_value};
+    sum<1>(v);
+    return v[0];
+  }
+  // exclusive prefix over the row's threads, in id order, of v < 2^29
+  __device__ uint64_t exscan(uint32_t v) {
+    const int lane = threadIdx.x & 31;
+    uint64_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    uint64_t t[1] = {__shfl_sync(0xffffffffu, x, 31)}, before;
+    sum<1>(t, &before);
+    return before + x - v;
+  }
+};
+
+// ---- block-wide sums (the list runs in one CTA) --------------------------------------------
+__device__ __forceinline__ uint64_t block_sum_u64(uint64_t v, uint64_t* red) {
+  v = warp_sum_u64(v);
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   __syncthreads();
   if (l == 0) red[w] = v;
   __syncthreads();
-  uint64_t t = (l < (int)(blockDim.x >> 5)) ? red[l] : 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+  return warp_sum_u64(l < ACC_WARPS ? red[l] : 0);
 }
 
-__device__ __forceinline__ float block_max_f(float v, float* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float t = (l < (int)(blockDim.x >> 5)) ? red[l] : -INFINITY;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, o));
-  return t;
-}
-
-// exclusive prefix sum over threads (in thread order) of v; returns this thread's offset
+// exclusive prefix sum over threads (in thread order) of v
 __device__ __forceinline__ uint64_t block_exscan_u64(uint64_t v, uint64_t* red) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   uint64_t x = v;
@@ -112,49 +199,48 @@ __device__ __forceinline__ uint64_t block_exscan_u64(uint64_t v, uint64_t* red) 
   __syncthreads();
   if (l == 31) red[w] = x;
   __syncthreads();
-  if (w == 0) {
-    uint64_t t = (l < (int)(blockDim.x >> 5)) ? red[l] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t y = __shfl_up_sync(0xffffffffu, t, o);
-      if (l >= o) t += y;
-    }
-    red[l] = t;   // inclusive prefix of warp sums
-  }
-  __syncthreads();
-  return (w > 0 ? red[w - 1] : 0) + x - v;
+  return warp_sum_u64(l < w ? red[l] : 0) + x - v;
 }
 
 // ---- greedy: argmax with the lowest id on ties, NaN as -inf ----------------------------
-__device__ int row_argmax(const float* row, int V, uint32_t* err, float* redf, int* redi) {
+// (float value ordered as an unsigned word, inverted id): larger is heavier, then lower id
+__device__ __forceinline__ uint64_t arg_key(float x, int id) {
+  const uint32_t b = __float_as_uint(x);
+  return ((uint64_t)((b & 0x80000000u) ? ~b : b | 0x80000000u) << 32) | (uint32_t)(0x7FFFFFFF - id);
+}
+
+__device__ int row_argmax(const float* row, int V, uint32_t* err, Row& rw) {
   float best = -INFINITY;
-  int bi = 0x7FFFFFFF;
-  bool nan = false;
+  int bi = 0;   // (a thread without ids, or with NaN alone, loses to any other: see the key)
+  bool nan = false, any = false;
   auto take = [&](float x, int i) {
     if (x != x) {
       nan = true;
       x = -INFINITY;
     }
-    if (x > best || (x == best && i < bi)) {
+    x += 0.f;   // -0 counts as +0
+    if (!any || x > best) {
+      any = true;
       best = x;
       bi = i;
     }
   };
-  // float4 loads, a round of RN per thread issued before any is compared (the row is one
-  // L2 round trip per round, not one per element); a thread visits its ids in increasing order
-  constexpr int RN = 8;
+  // float4 loads, a round of RN per thread issued before any is compared; the row's CTAs take
+  // its rounds in turn, a thread visits its ids in increasing order
+  constexpr int RN = 2;
+  const int nthr = rw.cs * ACC_THREADS, tid = rw.rank * ACC_THREADS + threadIdx.x;
   const bool vec = (reinterpret_cast<uintptr_t>(row) & 15u) == 0;
   const int V4 = vec ? V / 4 : 0;
-  for (int i0 = 0; i0 < V4; i0 += RN * (int)blockDim.x) {
+  for (int i0 = 0; i0 < V4; i0 += RN * nthr) {
     float4 v[RN];
 #pragma unroll
     for (int u = 0; u < RN; ++u) {
-      const int i = i0 + u * (int)blockDim.x + threadIdx.x;
+      const int i = i0 + u * nthr + tid;
       if (i < V4) v[u] = __ldcg(reinterpret_cast<const float4*>(row) + i);
     }
 #pragma unroll
     for (int u = 0; u < RN; ++u) {
-      const int i = i0 + u * (int)blockDim.x + threadIdx.x;
+      const int i = i0 + u * nthr + tid;
       if (i < V4) {
         take(v[u].x, 4 * i);
         take(v[u].y, 4 * i + 1);
@@ -163,47 +249,18 @@ __device__ int row_argmax(const float* row, int V, uint32_t* err, float* redf, i
       }
     }
   }
-  for (int i = 4 * V4 + threadIdx.x; i < V; i += blockDim.x) take(__ldcg(row + i), i);
+  for (int i = 4 * V4 + tid; i < V; i += nthr) take(__ldcg(row + i), i);
   if (nan) set_error(err, ERR_NAN_LOGITS);
+  uint64_t key = any ? arg_key(best, bi) : 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ob > best || (ob == best && oi < bi)) {
-      best = ob;
-      bi = oi;
-    }
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) {
-    redf[w] = best;
-    redi[w] = bi;
-  }
-  __syncthreads();
-  if (w == 0) {
-    const int nw = blockDim.x >> 5;
-    best = l < nw ? redf[l] : -INFINITY;
-    bi = l < nw ? redi[l] : 0x7FFFFFFF;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) {
-        best = ob;
-        bi = oi;
-      }
-    }
-    if (l == 0) redi[0] = (bi == 0x7FFFFFFF) ? 0 : bi;
-  }
-  __syncthreads();
-  return redi[0];
+  for (int o = 16; o > 0; o >>= 1) key = max(key, (uint64_t)__shfl_xor_sync(0xffffffffu, key, o));
+  key = rw.largest(key);
+  return 0x7FFFFFFF - (int)(uint32_t)key;
 }
 
 // ---- nucleus: the fixed-point top-k / top-p sampler ------------------------------------
-// Thread t owns ids [32t, 32t+32) (ascending id order is thread order, then
-// slot) and keeps their weights W (uint32, <= 2^24) in registers.  Selections
-// are predicates on (W, id); per-thread sums fit 32 bits, block sums 64.
+// A thread keeps the weights W (uint32, <= 2^24) of its ids in registers.  Selections are
+// predicates on (W, id); per-thread sums fit 32 bits, row sums 64.
 struct Cut {
   uint32_t xk;  // top-k: candidates are W > xk, or W == xk and id <= idk
   int idk;
@@ -236,7 +293,7 @@ __device__ __forceinline__ bool pred(uint32_t W, int id, const Cut& c, uint32_t 
   }
 }
 
-// per-thread sum of W (COUNT: number of ids) over the owned ids selected by P
+// per-thread sum of W (COUNT: number of ids) over the owned ids selected by P (< 2^28)
 template <int P, bool COUNT>
 __device__ __forceinline__ uint32_t lsum(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x) {
   uint32_t s = 0;
@@ -245,16 +302,32 @@ __device__ __forceinline__ uint32_t lsum(const uint32_t (&W)[ACC_EPT], int base,
     if (pred<P>(W[e], base + e, c, x)) s += COUNT ? 1u : W[e];
   return s;
 }
+template <int P, bool COUNT>
+__device__ __forceinline__ uint64_t row_sum(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x, Row& rw) {
+  return rw.sum(warp_total(lsum<P, COUNT>(W, base, c, x)));
+}
 
-// largest x in [0, 2^24] whose block total of lsum<P, COUNT>(x) is >= need (monotone in x)
+// largest x in [0, 2^24] whose row total of lsum<P, COUNT>(x) is >= need (monotone in x); three
+// thresholds a step: a step is one cluster barrier, whose latency outweighs the sums
 template <int P, bool COUNT>
 __device__ __forceinline__ uint32_t search_threshold(const uint32_t (&W)[ACC_EPT], int base, const Cut& c,
-                                                     uint64_t need, uint64_t* red) {
+                                                     uint64_t need, Row& rw) {
   uint32_t lo = 0, hi = 1u << 24;
   while (lo < hi) {
-    const uint32_t mid = lo + (hi - lo + 1) / 2;
-    if (block_sum_u64(lsum<P, COUNT>(W, base, c, mid), red) >= need) lo = mid;
-    else hi = mid - 1;
+    const uint32_t d = (hi - lo + 3) / 4;
+    const uint32_t x[3] = {min(lo + d, hi), min(lo + 2 * d, hi), min(lo + 3 * d, hi)};
+    uint64_t t[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) t[i] = warp_total(lsum<P, COUNT>(W, base, c, x[i]));
+    rw.sum<3>(t);
+    uint32_t nlo = lo, nhi = hi;
+#pragma unroll
+    for (int i = 2; i >= 0; --i) {
+      if (t[i] >= need) nlo = max(nlo, x[i]);
+      else nhi = x[i] - 1;   // (the last assignment is the lowest failing threshold's)
+    }
+    lo = nlo;
+    hi = nhi;
   }
   return lo;
 }
@@ -262,37 +335,29 @@ __device__ __forceinline__ uint32_t search_threshold(const uint32_t (&W)[ACC_EPT
 // the n-th (n >= 1) smallest id selected by P, or INT_MAX if there are fewer
 template <int P>
 __device__ __forceinline__ int nth_id(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x,
-                                      uint64_t n, uint64_t* red, int* redi) {
-  const uint64_t mine = lsum<P, true>(W, base, c, x);
-  const uint64_t before = block_exscan_u64(mine, red);
-  if (threadIdx.x == 0) redi[0] = 0x7FFFFFFF;
-  __syncthreads();
-  if (before < n && before + mine >= n) {
-    uint64_t k = before;
-    int hit = 0x7FFFFFFF;
+                                      uint64_t n, Row& rw) {
+  const uint32_t mine = lsum<P, true>(W, base, c, x);
+  uint64_t k = rw.exscan(mine);
+  uint32_t hit = 0;   // id + 1 in the one thread that holds it
+  if (k < n && k + mine >= n) {
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e)
-      if (pred<P>(W[e], base + e, c, x) && ++k == n) hit = base + e;
-    redi[0] = hit;
+      if (pred<P>(W[e], base + e, c, x) && ++k == n) hit = base + e + 1;
   }
-  __syncthreads();
-  const int out = redi[0];
-  __syncthreads();
-  return out;
+  const uint64_t id = rw.sum(warp_total(hit));
+  return id ? (int)id - 1 : 0x7FFFFFFF;
 }
 
 // ---- the sampler on a compacted list ----------------------------------------------------
 // The kept set is a prefix of the order (W desc, id asc), so it lies among the heaviest
 // weights.  With a floor F such that the elements with W >= F provably contain it (top-k:
 // at least k of them, or all non-zero weights; top-p alone: their mass reaches the top-p
-// threshold), those elements are copied in ascending id order into shared memory and one
-// warp runs the same selection on them: searches cost O(list / 32) per step and no block
-// barrier.  Otherwise the block-wide searches over all ids run.
+// threshold), those elements go in ascending id order into rank 0's shared memory, and that
+// CTA finishes the row.  Otherwise the row-wide searches over all ids run.
 constexpr int NUC_LIST_MAX = 4096;
 constexpr int NUC_FLOORS = 7;
 // floor f: 2^24 (the largest weight), 2^22, 2^20, 2^18, 2^16 (ratio 2^-8), 2^8 (2^-16), then 1
 // (every non-zero weight).  Weights of bucket b (nuc_bucket) are >= the floors f >= b.
-__device__ __forceinline__ uint32_t nuc_floor(int f) { return f < 5 ? 1u << (24 - 2 * f) : (f == 5 ? 256u : 1u); }
 __device__ __forceinline__ int nuc_bucket(uint32_t w) {
   if (w == 0) return NUC_FLOORS;
   const int e = 31 - __clz(w);
@@ -300,11 +365,9 @@ __device__ __forceinline__ int nuc_bucket(uint32_t w) {
 }
 
 struct NucList {
-  uint32_t w[NUC_LIST_MAX];
-  int id[NUC_LIST_MAX];
-  uint32_t cnt[NUC_FLOORS];                 // block totals: weights >= floor f
-  unsigned long long mhi[3], mlo[3];        // masses >= floors 4, 5, 6: sum(w >> 12), sum(w & 4095)
-  unsigned long long kstar, sk;             // the kept prefix's last key and its mass
+  unsigned long long key[NUC_LIST_MAX];      // nuc_key of the list's elements, ascending id
+  unsigned long long sorted[NUC_LIST_MAX];   // the same in descending order
+  unsigned long long kstar, sk;              // the kept prefix's last key and its mass
   int pick;
 };
 
@@ -330,7 +393,7 @@ __device__ int list_small(const AcceptParams& p, const NucList& L, int n, uint64
   for (int r = 0; r < rounds && !(nc > 0 && !topk && C >= thr); ++r) {
     uint64_t best = 0;
     for (int i = lane; i < n; i += 32) {
-      const uint64_t k = nuc_key(L.w[i], L.id[i]);
+      const uint64_t k = L.key[i];
       if (k < prev && k > best) best = k;
     }
     const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32));
@@ -372,53 +435,69 @@ __device__ int list_small(const AcceptParams& p, const NucList& L, int n, uint64
   return __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
 }
 
-// Steps 4-7 on the list with the whole block.  The list holds the first n elements of the
-// order (W desc, id asc) in ascending id; its keys are sorted once (bitonic, descending, over
-// the list's own storage), so the candidates (the first min(k, n)), their mass, the kept
-// prefix (the shortest one whose mass reaches ceil(P S / 2^24)) and its mass are prefix sums
-// of the sorted weights.  The pick then scans every id's weight, still in registers, in
-// ascending id with "kept" = key >= the kept prefix's last key.
-__device__ int list_sorted_select(const AcceptParams& p, NucList& L, int n, uint64_t S_all, uint64_t rnd,
-                                  const uint32_t (&W)[ACC_EPT], int base, uint64_t* red, int* redi) {
-  constexpr int PER = NUC_LIST_MAX / ACC_THREADS;   // list elements per thread
-  uint64_t* K = reinterpret_cast<uint64_t*>(L.w);    // NUC_LIST_MAX keys over w[] and id[]
-  int n2 = 32;
-  while (n2 < n) n2 <<= 1;
-  uint64_t kk[PER];
-#pragma unroll
+// L.sorted = the n2 (a power of two >= 32, the list's n keys and zeros) keys in descending
+// order: bitonic; distances below 32 stay in the warp (element i is on lane i & 31), so 1024
+// keys take 15 block barriers and not 55.
+__device__ void list_sort(NucList& L, int n, int n2) {
+  constexpr int PER = NUC_LIST_MAX / ACC_THREADS;
+  auto in_warp = [&](uint64_t x, int i, int k, int j) {   // distances j .. 1 of the merge of size k
+    for (; j > 0; j >>= 1) {
+      const uint64_t y = __shfl_xor_sync(0xffffffffu, x, j);
+      // descending blocks where bit k of i is clear: the lower element keeps the larger key
+      const bool keep_max = ((i & k) == 0) == ((i & j) == 0);
+      x = keep_max ? max(x, y) : min(x, y);
+    }
+    return x;
+  };
+#pragma unroll 1
   for (int r = 0; r < PER; ++r) {
     const int i = threadIdx.x + r * ACC_THREADS;
-    kk[r] = i < n ? nuc_key(L.w[i], L.id[i]) : 0ull;   // padding sorts last (every list W >= 1)
+    if (i >= n2) break;   // (whole warps)
+    uint64_t x = i < n ? L.key[i] : 0ull;   // padding sorts last (every list W >= 1)
+    for (int k = 2; k <= 32; k <<= 1) x = in_warp(x, i, k, k >> 1);
+    L.sorted[i] = x;
   }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < PER; ++r) {
-    const int i = threadIdx.x + r * ACC_THREADS;
-    if (i < n2) K[i] = kk[r];
-  }
-  __syncthreads();
-  for (int k = 2; k <= n2; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
+  for (int k = 64; k <= n2; k <<= 1) {
+    for (int j = k >> 1; j >= 32; j >>= 1) {
+      __syncthreads();
       for (int i = threadIdx.x; i < n2; i += ACC_THREADS) {
         const int l = i ^ j;
         if (l > i) {
-          const uint64_t a = K[i], b = K[l];
-          if (((i & k) == 0) == (a < b)) {   // descending blocks where bit k of i is clear
-            K[i] = b;
-            K[l] = a;
+          const uint64_t a = L.sorted[i], b = L.sorted[l];
+          if (((i & k) == 0) == (a < b)) {
+            L.sorted[i] = b;
+            L.sorted[l] = a;
           }
         }
       }
-      __syncthreads();
     }
-  // candidates and the kept prefix: thread t holds sorted elements PER*t .. PER*t + PER - 1
+    __syncthreads();
+#pragma unroll 1
+    for (int r = 0; r < PER; ++r) {
+      const int i = threadIdx.x + r * ACC_THREADS;
+      if (i >= n2) break;
+      L.sorted[i] = in_warp(L.sorted[i], i, k, 16);
+    }
+  }
+  __syncthreads();
+}
+
+// Steps 4-7 on the list with the whole CTA.  The list holds the first n elements of the order
+// (W desc, id asc), in ascending id.  Its keys are sorted once, so the candidates (the first
+// min(k, n)), their mass, the kept prefix (the shortest one whose mass reaches
+// ceil(P S / 2^24)) and its mass are prefix sums of the sorted weights.  The pick then scans
+// the list itself in ascending id with "kept" = key >= the kept prefix's last key.
+__device__ int list_sorted_select(const AcceptParams& p, NucList& L, int n, uint64_t S_all, uint64_t rnd,
+                                  uint64_t* red) {
+  int n2 = 32;
+  while (n2 < n) n2 <<= 1;
+  list_sort(L, n, n2);
+  // candidates and the kept prefix: thread t holds `per` consecutive sorted elements
+  const int per = (n + ACC_THREADS - 1) / ACC_THREADS, i0 = threadIdx.x * per, i1 = min(i0 + per, n);
   const bool topk = p.top_k > 0 && p.top_k < p.V;
   const int nc = topk ? min(p.top_k, n) : n;
-  const int i0 = threadIdx.x * PER;
   uint64_t wsum = 0;
-#pragma unroll
-  for (int e = 0; e < PER; ++e)
-    if (i0 + e < nc) wsum += K[i0 + e] >> 32;
+  for (int i = i0; i < min(i1, nc); ++i) wsum += L.sorted[i] >> 32;
   const uint64_t S = topk ? block_sum_u64(wsum, red) : S_all;
   const uint64_t prod = (uint64_t)p.p_fixed * S;
   const uint64_t thr = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
@@ -427,11 +506,10 @@ __device__ int list_sorted_select(const AcceptParams& p, NucList& L, int n, uint
   // provably holds it
   if (thr == 0 ? threadIdx.x == 0 : (before < thr && before + wsum >= thr)) {
     uint64_t cum = before;
-#pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      cum += K[i0 + e] >> 32;
+    for (int i = i0; i < i1; ++i) {
+      cum += L.sorted[i] >> 32;
       if (cum >= thr) {
-        L.kstar = K[i0 + e];
+        L.kstar = L.sorted[i];
         L.sk = cum;
         break;
       }
@@ -442,54 +520,47 @@ __device__ int list_sorted_select(const AcceptParams& p, NucList& L, int n, uint
   const uint64_t tau = __umul64hi(rnd, Sk);
   // 7. the first kept id (ascending) whose inclusive cumulative weight exceeds tau
   uint64_t mine = 0;
-#pragma unroll
-  for (int e = 0; e < ACC_EPT; ++e)
-    if (nuc_key(W[e], base + e) >= kstar) mine += W[e];
+  for (int i = i0; i < i1; ++i)
+    if (L.key[i] >= kstar) mine += L.key[i] >> 32;
   const uint64_t below = block_exscan_u64(mine, red);
-  if (threadIdx.x == 0) redi[0] = 0x7FFFFFFF;
-  __syncthreads();
   if (below <= tau && below + mine > tau) {
     uint64_t cum = below;
-    int pick = 0x7FFFFFFF;
-#pragma unroll
-    for (int e = 0; e < ACC_EPT; ++e) {
-      if (nuc_key(W[e], base + e) >= kstar) {
-        cum += W[e];
-        if (cum > tau && pick == 0x7FFFFFFF) pick = base + e;
+    for (int i = i0; i < i1; ++i)
+      if (L.key[i] >= kstar) {
+        cum += L.key[i] >> 32;
+        if (cum > tau) {
+          L.pick = 0x7FFFFFFF - (int)(uint32_t)L.key[i];
+          break;
+        }
       }
-    }
-    redi[0] = pick;
   }
   __syncthreads();
-  const int out = redi[0];
-  __syncthreads();
-  return out;
+  return L.pick;
 }
 
+// The row's sampled id (valid in rank 0).  Every CTA of the cluster passes the same barriers:
+// every branch is taken on values that the whole row shares.
 __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* row, int position, int seq,
-                                           float* redf, uint64_t* red, int* redi, NucList& L) {
+                                           uint64_t* red, Row& rw, NucList& L) {
   const int V = p.V;
-  const int base = threadIdx.x * ACC_EPT;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int base = rw.rank * ACC_SPAN + threadIdx.x * ACC_EPT;
   uint32_t W[ACC_EPT];
-  float mx = -INFINITY;
-  bool nan = false;
-  if (threadIdx.x < NUC_FLOORS) L.cnt[threadIdx.x] = 0;   // published by block_max_f's barriers
-  if (threadIdx.x < 3) L.mhi[threadIdx.x] = L.mlo[threadIdx.x] = 0;
   {
     // 1. logits (NaN -> -inf; ids >= V are -inf, hence W = 0) and the row maximum
     float l[ACC_EPT];
+    if ((reinterpret_cast<uintptr_t>(row) & 15u) == 0 && base + ACC_EPT <= V) {
 #pragma unroll
-    for (int e = 0; e < ACC_EPT; e += 4) {
-      float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-      if (base + e + 3 < V) {
-        v = __ldcg(reinterpret_cast<const float4*>(row + base + e));
-      } else {
-        if (base + e < V) v.x = __ldcg(row + base + e);
-        if (base + e + 1 < V) v.y = __ldcg(row + base + e + 1);
-        if (base + e + 2 < V) v.z = __ldcg(row + base + e + 2);
+      for (int e = 0; e < ACC_EPT; e += 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(row + base + e));
+        l[e] = v.x; l[e + 1] = v.y; l[e + 2] = v.z; l[e + 3] = v.w;
       }
-      l[e] = v.x; l[e + 1] = v.y; l[e + 2] = v.z; l[e + 3] = v.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < ACC_EPT; ++e) l[e] = base + e < V ? __ldcg(row + base + e) : -INFINITY;
     }
+    bool nan = false;
+    float mx = -INFINITY;
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e) {
       if (l[e] != l[e]) {
@@ -499,7 +570,11 @@ __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* r
       mx = fmaxf(mx, l[e]);
     }
     if (nan) set_error(p.err, ERR_NAN_LOGITS);
-    mx = block_max_f(mx, redf);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    // (ordered as in arg_key, with id bits that do not matter)
+    const uint32_t ord = (uint32_t)(rw.largest(arg_key(mx, 0)) >> 32);
+    mx = __uint_as_float((ord & 0x80000000u) ? ord & 0x7FFFFFFFu : ~ord);
     // 2-3. W_i = floor(exp((l_i - max) / T) * 2^24)
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e) W[e] = fixed24(exp_sd(__fdiv_rn(__fsub_rn(l[e], mx), p.temperature)));
@@ -510,60 +585,35 @@ __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* r
   const uint64_t rnd = ((uint64_t)ctr[0] << 32) | ctr[1];
 
   // ---- the list path: counts (and, without top-k, masses) of the weights above each floor
+  const bool topk = p.top_k > 0 && p.top_k < V;
   {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool topk = p.top_k > 0 && p.top_k < V;
-    uint32_t c01 = 0, c23 = 0, c45 = 0, c6 = 0;   // per-thread counts, two 11-bit fields per word
-    uint32_t m4 = 0, m5 = 0, m6 = 0;              // per-thread masses >= floors 4, 5, 6 (< 2^29)
+    // per-thread counts (<= 8) of the floors in 16-bit fields: floors 0-3 and 4-6
+    uint64_t c03 = 0, c46 = 0;
+    uint32_t m4 = 0, m5 = 0, m6 = 0;   // masses >= floors 4, 5, 6 (< 2^28)
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e) {
       const int b = nuc_bucket(W[e]);
-      c01 += (b <= 0 ? 1u : 0u) + (b <= 1 ? 1u << 11 : 0u);
-      c23 += (b <= 2 ? 1u : 0u) + (b <= 3 ? 1u << 11 : 0u);
-      c45 += (b <= 4 ? 1u : 0u) + (b <= 5 ? 1u << 11 : 0u);
-      c6 += b <= 6 ? 1u : 0u;
-      if (!topk) {
-        m4 += b <= 4 ? W[e] : 0u;
-        m5 += b <= 5 ? W[e] : 0u;
-        m6 += W[e];
-      }
-    }
-    c01 = __reduce_add_sync(0xffffffffu, c01);   // warp totals <= 1024 per field
-    c23 = __reduce_add_sync(0xffffffffu, c23);
-    c45 = __reduce_add_sync(0xffffffffu, c45);
-    c6 = __reduce_add_sync(0xffffffffu, c6);
-    uint32_t mh[3] = {0, 0, 0}, ml[3] = {0, 0, 0};
-    if (!topk) {
-      const uint32_t m[3] = {m4, m5, m6};
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        mh[i] = __reduce_add_sync(0xffffffffu, m[i] >> 12);
-        ml[i] = __reduce_add_sync(0xffffffffu, m[i] & 4095u);
-      }
-    }
-    if (lane == 0) {
-      atomicAdd(&L.cnt[0], c01 & 2047u);
-      atomicAdd(&L.cnt[1], c01 >> 11);
-      atomicAdd(&L.cnt[2], c23 & 2047u);
-      atomicAdd(&L.cnt[3], c23 >> 11);
-      atomicAdd(&L.cnt[4], c45 & 2047u);
-      atomicAdd(&L.cnt[5], c45 >> 11);
-      atomicAdd(&L.cnt[6], c6);
-      if (!topk)
+      for (int f = 0; f < 4; ++f) c03 += b <= f ? 1ull << (16 * f) : 0ull;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          atomicAdd(&L.mhi[i], (unsigned long long)mh[i]);
-          atomicAdd(&L.mlo[i], (unsigned long long)ml[i]);
-        }
+      for (int f = 4; f < NUC_FLOORS; ++f) c46 += b <= f ? 1ull << (16 * (f - 4)) : 0ull;
+      m4 += b <= 4 ? W[e] : 0u;
+      m5 += b <= 5 ? W[e] : 0u;
+      m6 += W[e];
     }
-    __syncthreads();
+    // (warp totals of a field <= 256, row totals <= 32768)
+    auto add16 = [&](uint64_t v) {
+      return ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 32)) << 32) |
+             __reduce_add_sync(0xffffffffu, (uint32_t)v);
+    };
+    uint64_t t[ACC_WORDS] = {add16(c03), add16(c46), warp_total(m4), warp_total(m5), warp_total(m6)};
+    const int buf = rw.ph & 1;
+    rw.sum<ACC_WORDS>(t);
+    const unsigned long long *warps = rw.slots->w[buf], *ctas = rw.slots->c[buf];
     int N[NUC_FLOORS];
 #pragma unroll
-    for (int f = 0; f < NUC_FLOORS; ++f) N[f] = (int)L.cnt[f];
-    if (N[6] == 0) return 0;   // every weight 0 (all-NaN row): the lowest candidate, id 0
-    uint64_t Sf[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) Sf[i] = (L.mhi[i] << 12) + L.mlo[i];
+    for (int f = 0; f < NUC_FLOORS; ++f) N[f] = (int)(((f < 4 ? t[0] : t[1]) >> (16 * (f & 3))) & 0xFFFF);
+    const uint64_t Sf[3] = {t[2], t[3], t[4]};
     const uint64_t S_all = Sf[2];
     uint64_t thr_all = 0;
     if (!topk) {
@@ -577,80 +627,92 @@ __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* r
       const bool holds = topk ? (N[i] >= p.top_k || N[i] == N[6]) : (i >= 4 && Sf[i - 4] >= thr_all);
       if (f < 0 && N[i] <= NUC_LIST_MAX && holds) f = i;
     }
+    if (N[6] == 0) return 0;   // every weight 0 (all-NaN row): the lowest candidate, id 0
     if (f >= 0) {
+      int nf = 0;
+#pragma unroll
+      for (int i = 0; i < NUC_FLOORS; ++i) nf = i == f ? N[i] : nf;
+      // this thread's place in the list: the CTAs and warps before (from the totals just
+      // summed), then the lanes before
+      const int word = f >> 2, sh = 16 * (f & 3);
+      uint64_t at = 0;
+      if (lane < rw.rank) at += (ctas[lane * ACC_WORDS + word] >> sh) & 0xFFFF;
+      if (lane < w) at += (warps[lane * ACC_WORDS + word] >> sh) & 0xFFFF;
+      at = warp_sum_u64(at);
       uint32_t mine = 0;
 #pragma unroll
       for (int e = 0; e < ACC_EPT; ++e) mine += nuc_bucket(W[e]) <= f;
-      uint32_t at = (uint32_t)block_exscan_u64(mine, red);
+      uint32_t x = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      uint32_t dst = mapa_shared(smem_u32(&L.key[0]), 0) + ((uint32_t)at + x - mine) * 8;
 #pragma unroll
       for (int e = 0; e < ACC_EPT; ++e)
         if (nuc_bucket(W[e]) <= f) {
-          L.w[at] = W[e];
-          L.id[at] = base + e;
-          ++at;
+          st_dsmem_u64(dst, nuc_key(W[e], base + e));
+          dst += 8;
         }
-      __syncthreads();
+      cluster_sync_all();   // the list is complete
+      if (rw.rank) return 0;
       // a kept set (or top-k) of at most 32 on the lanes of one warp when that is cheap: a
       // small top-k, or a short list; otherwise, or when it does not apply, the sorted list
-      if ((topk && p.top_k <= 32) || N[f] <= 64) {
+      if ((topk && p.top_k <= 32) || nf <= 64) {
         if (w == 0) {
-          const int pick = list_small(p, L, N[f], S_all, topk, rnd);
+          const int pick = list_small(p, L, nf, S_all, topk, rnd);
           if (lane == 0) L.pick = pick;
         }
         __syncthreads();
         const int pick = L.pick;
         if (pick >= 0) return pick;
+        __syncthreads();   // L.pick is written again
       }
-      return list_sorted_select(p, L, N[f], S_all, rnd, W, base, red, redi);
+      return list_sorted_select(p, L, nf, S_all, rnd, red);
     }
   }
 
-  // ---- the block-wide path over all ids
+  // ---- the row-wide path over all ids
   Cut c;
   c.xk = 0;
   c.idk = 0x7FFFFFFF;
   c.xp = 0;
   c.idp = 0x7FFFFFFF;
   // 4. top-k candidates
-  if (p.top_k > 0 && p.top_k < V) {
-    c.xk = search_threshold<P_GE, true>(W, base, c, (uint64_t)p.top_k, red);
-    const uint64_t above = block_sum_u64(lsum<P_GT, true>(W, base, c, c.xk), red);
-    c.idk = nth_id<P_EQ>(W, base, c, c.xk, (uint64_t)p.top_k - above, red, redi);
+  if (topk) {
+    c.xk = search_threshold<P_GE, true>(W, base, c, (uint64_t)p.top_k, rw);
+    const uint64_t above = row_sum<P_GT, true>(W, base, c, c.xk, rw);
+    c.idk = nth_id<P_EQ>(W, base, c, c.xk, (uint64_t)p.top_k - above, rw);
   }
   // 5. top-p over the candidates: thr = ceil(P * S / 2^24), P <= 2^24, S < 2^40
-  const uint64_t S = block_sum_u64(lsum<P_CAND, false>(W, base, c, 0), red);
-  if (S == 0) return nth_id<P_CAND>(W, base, c, 0, 1, red, redi);   // all-NaN row: lowest candidate
+  const uint64_t S = row_sum<P_CAND, false>(W, base, c, 0, rw);
   const uint64_t prod = (uint64_t)p.p_fixed * S;
   const uint64_t thr = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-  c.xp = search_threshold<P_CAND_GE, false>(W, base, c, thr, red);
-  const uint64_t above = block_sum_u64(lsum<P_CAND_GT, false>(W, base, c, c.xp), red);
-  const uint64_t n_above = block_sum_u64(lsum<P_CAND_GT, true>(W, base, c, c.xp), red);
-  uint64_t ties = thr > above ? (thr - above + c.xp - 1) / c.xp : 0;
-  if (n_above == 0 && ties == 0) ties = 1;
-  c.idp = ties == 0 ? -1 : nth_id<P_CAND_EQ>(W, base, c, c.xp, ties, red, redi);
-  const uint64_t Sk = block_sum_u64(lsum<P_KEPT, false>(W, base, c, 0), red);
-  const uint64_t tau = __umul64hi(rnd, Sk);
+  c.xp = search_threshold<P_CAND_GE, false>(W, base, c, thr, rw);
+  uint64_t ab[2] = {warp_total(lsum<P_CAND_GT, false>(W, base, c, c.xp)),
+                    warp_total(lsum<P_CAND_GT, true>(W, base, c, c.xp))};
+  rw.sum<2>(ab);
+  uint64_t ties = thr > ab[0] ? (thr - ab[0] + c.xp - 1) / c.xp : 0;
+  if (ab[1] == 0 && ties == 0) ties = 1;
+  c.idp = ties == 0 ? -1 : nth_id<P_CAND_EQ>(W, base, c, c.xp, ties, rw);
   // 7. the first kept id (ascending) whose inclusive cumulative weight exceeds tau
-  const uint64_t mine = lsum<P_KEPT, false>(W, base, c, 0);
-  const uint64_t before = block_exscan_u64(mine, red);
-  if (threadIdx.x == 0) redi[0] = 0x7FFFFFFF;
-  __syncthreads();
+  const uint32_t mine = lsum<P_KEPT, false>(W, base, c, 0);
+  const uint64_t Sk = rw.sum(warp_total(mine));
+  const uint64_t tau = __umul64hi(rnd, Sk);
+  const uint64_t before = rw.exscan(mine);
+  uint32_t hit = 0;   // id + 1 in the one thread that holds it
   if (before <= tau && before + mine > tau) {
     uint64_t cum = before;
-    int pick = 0x7FFFFFFF;
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e) {
       if (pred<P_KEPT>(W[e], base + e, c, 0)) {
         cum += W[e];
-        if (cum > tau && pick == 0x7FFFFFFF) pick = base + e;
+        if (cum > tau && !hit) hit = base + e + 1;
       }
     }
-    redi[0] = pick;
   }
-  __syncthreads();
-  const int out = redi[0];
-  __syncthreads();
-  return out;
+  return (int)rw.sum(warp_total(hit)) - 1;
 }
 
 // parent of tree row i (0 < i < q): an earlier row; anything else is flagged and read as the root
@@ -671,30 +733,28 @@ __device__ __forceinline__ int tree_depth(const int* par, int j, uint32_t* err) 
 }
 
 __global__ void __launch_bounds__(ACC_THREADS) accept_kernel(const AcceptParams p) {
-  __shared__ float redf[32];
-  __shared__ uint64_t red[32];
-  __shared__ int redi[32];
-  __shared__ int s_last;
-  __shared__ NucList nl;
+  extern __shared__ __align__(16) uint8_t acc_smem[];   // NucList (nucleus only)
+  __shared__ AccSlots slots;
+  __shared__ uint64_t red[ACC_WARPS];
+  cluster_arrive_thread();
   pdl_wait();
   pdl_trigger();
-  const int j = blockIdx.x, sl = blockIdx.y, s = p.seq0 + sl;
+  cluster_wait_thread();   // every CTA of the row has started: its shared memory may be written
+  Row rw{&slots, p.cs, (int)cluster_ctarank(), 0};
+  const int j = blockIdx.x / p.cs, sl = blockIdx.y, s = p.seq0 + sl;
   const float* row = p.logits + (size_t)(sl * p.q + j) * p.V;
   int t;
   if (p.temperature <= 0.f) {
-    t = row_argmax(row, p.V, p.err, redf, redi);
+    t = row_argmax(row, p.V, p.err, rw);
   } else {
     // the produced token's position: one past the row's own (len + j, or len + depth(j))
     const int position = __ldcg(p.len + s) + (p.parent ? tree_depth(p.parent + sl * p.q, j, nullptr) : j) + 1;
-    t = row_nucleus(p, row, position, s, redf, red, redi, nl);
+    t = row_nucleus(p, row, position, s, red, rw, *reinterpret_cast<NucList*>(acc_smem));
   }
-  if (threadIdx.x == 0) p.targets[sl * p.q + j] = t;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = (atomicAdd(p.counters + sl, 1) == p.q - 1);
-  __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
-  __threadfence();
+  // the last row of a sequence (per-sequence counter) verifies and commits
+  if (rw.rank || threadIdx.x) return;
+  p.targets[sl * p.q + j] = t;
+  if (atomic_add_acq_rel_gpu(p.counters + sl, 1) != p.q - 1) return;
   int tg[SDSAT_ATT_MAXQ];
   for (int i = 0; i < p.q; ++i) tg[i] = __ldcg(p.targets + sl * p.q + i);
   int m = 0;
@@ -757,9 +817,21 @@ static cudaLaunchConfig_t make_cfg(dim3 grid, dim3 block, cudaStream_t st, bool 
   return cfg;
 }
 
-cudaError_t launch_accept(const AcceptParams& p, cudaStream_t st, bool pdl) {
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = make_cfg(dim3(p.q, p.nb), dim3(ACC_THREADS), st, pdl, attr);
+cudaError_t accept_prepare() {
+  return cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NucList));
+}
+
+cudaError_t launch_accept(const AcceptParams& p0, cudaStream_t st, bool pdl) {
+  AcceptParams p = p0;
+  p.cs = std::min(ACC_CS, (p.V + ACC_SPAN - 1) / ACC_SPAN);   // (a larger vocabulary is greedy only)
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = make_cfg(dim3(p.q * p.cs, p.nb), dim3(ACC_THREADS), st, pdl, attr);
+  cfg.dynamicSmemBytes = p.temperature > 0.f ? sizeof(NucList) : 0;
+  attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+  attr[cfg.numAttrs].val.clusterDim.x = p.cs;
+  attr[cfg.numAttrs].val.clusterDim.y = 1;
+  attr[cfg.numAttrs].val.clusterDim.z = 1;
+  ++cfg.numAttrs;
   return cudaLaunchKernelEx(&cfg, accept_kernel, p);
 }
 

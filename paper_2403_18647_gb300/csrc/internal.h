@@ -237,8 +237,10 @@ struct AcceptParams {
   const int* parent;        // tree blocks: [nb*q] parent row of every row (row 0: -1); null = chain
   int* path;                // tree blocks: [nb*q] accepted path rows, -1 past its end (optional)
   int* tree_ws;             // tree blocks: [nb][TREE_WS_STRIDE] len before the step, m, path rows
+  int cs;                   // CTAs per row (set by launch_accept)
   uint32_t* err;
 };
+cudaError_t accept_prepare();
 constexpr int TREE_WS_STRIDE = SDSAT_ATT_MAXQ + 2;
 constexpr int TREE_MAX_ROWS = 64;   // rows of one block forward (the tree kernels run one thread per row)
 cudaError_t launch_accept(const AcceptParams& p, cudaStream_t st, bool pdl);

@@ -622,7 +622,7 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   if (cudaGetDevice(&c->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
       gemm_prepare() != cudaSuccess || attention_prepare() != cudaSuccess || prefill_prepare() != cudaSuccess ||
-      prefill_attention_prepare() != cudaSuccess) {
+      prefill_attention_prepare() != cudaSuccess || accept_prepare() != cudaSuccess) {
     delete c;
     return SDSAT_ECUDA;
   }

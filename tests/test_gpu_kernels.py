@@ -175,7 +175,7 @@ def accept_env(sd):
 
 
 def _run_accept(ctx, logits, drafts, b, q, n_verify, lens, temperature=0.0, top_p=1.0, seed=0, top_k=0):
-    kv = ctx.kv(b, 4000)
+    kv = ctx.kv(b, min(4000, ctx.cfg.max_position))
     ln = torch.tensor(lens, dtype=torch.int32, device="cuda")
     ctx.kv_commit(kv, ln, b)
     acc = torch.empty(b, dtype=torch.int32, device="cuda")
@@ -400,3 +400,35 @@ def test_attention_40_heads_sampled(big_ctx):
                       [n + j + 1 for j in range(q)])
         err = np.abs(out.cpu().double().numpy().reshape(q, H, hd)[:, h] - o[:, 0]).max()
         assert err <= 2e-5, (h, err)
+
+
+@pytest.mark.parametrize("V", [2, 33, 1001, 4095, 4096, 4097, 8195, 20481, 32767, 32768])
+def test_accept_vocabulary_edges(sd, V):
+    """One to eight CTAs per row, ids that end inside a thread's eight, rows that are not 16-byte
+    aligned (odd vocabularies): bit-exact against the oracle, each selection."""
+    shape = synth.ModelShape("v%d" % V, 1, 128, 1, 128, 256, V, 0)
+    ctx = sd.Context(shape, None, max_position=4096)
+    b, q = 2, 3
+    lg = _logits(V, b * q, V)
+    lg[0, V - 1] = lg[0, 0] = lg[0].max() + 0.5   # a tie between the first and the last id
+    lg[1] = -lg[1].abs()
+    lg[1, V // 2] = float("-inf")
+    lgc = lg.cpu().numpy()
+    drafts = [0] * (b * q)
+    dr = torch.zeros(b * q, dtype=torch.int32, device="cuda")
+    for T, top_p, top_k in [(0.0, 1.0, 0), (1.0, 0.95, 0), (1.0, 1.0, 0), (0.2, 0.95, 10), (3.0, 0.9, 40)]:
+        acc, out, flags, _ = _run_accept(ctx, lg, dr, b, q, q - 1, [7, 9], T, top_p, 3, top_k)
+        racc, rout = _oracle_accept(lgc, drafts, b, q, q - 1, [7, 9], T, top_p, 3, top_k)
+        assert (out, acc, flags) == (rout, racc, 0), (T, top_p, top_k)
+
+
+def test_argmax_signed_zero_and_minus_infinity(sd):
+    """-0 ties with +0 (the lowest id wins), rows of -inf or NaN alone give id 0."""
+    shape = synth.ModelShape("v9000", 1, 128, 1, 128, 256, 9000, 0)
+    ctx = sd.Context(shape, None, max_position=64)
+    lg = torch.full((3, 9000), -1.0, device="cuda")
+    lg[0, 8000], lg[0, 5000] = 0.0, -0.0
+    lg[1] = float("-inf")
+    lg[2] = float("nan")
+    acc, out, flags, _ = _run_accept(ctx, lg, torch.zeros(3, dtype=torch.int32, device="cuda"), 1, 3, 0, [0])
+    assert out[0] == [5000, 0, 0] and flags == 0x1
