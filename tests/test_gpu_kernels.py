@@ -432,3 +432,17 @@ def test_argmax_signed_zero_and_minus_infinity(sd):
     lg[2] = float("nan")
     acc, out, flags, _ = _run_accept(ctx, lg, torch.zeros(3, dtype=torch.int32, device="cuda"), 1, 3, 0, [0])
     assert out[0] == [5000, 0, 0] and flags == 0x1
+
+
+@pytest.mark.parametrize("M,K,N", [(6, 1024, 300), (6, 1032, 300), (6, 1000, 38912), (6, 1024, 38913),
+                                   (24, 1024, 4097), (48, 1024, 19456), (48, 1024, 19457), (64, 1032, 130)])
+def test_gemm_whole_and_split_tiles(tiny_ctx, M, K, N):
+    """Both sides of the rule that leaves tiles whole: 16 and 17 chunks, as many tiles as CTAs
+    and one more (two CTAs per SM up to 32 rows, one beyond)."""
+    x = synth.normal_f32(11, M, (M, K), 1.0, device="cuda")
+    w = synth.normal_bf16(11, N, (N, K), 0.02, device="cuda")
+    y = torch.full((M, N), float("nan"), device="cuda")
+    tiny_ctx.op_gemm(x, w, y)
+    ref = x.double() @ w.double().t()
+    tol = 5e-5 * math.sqrt(K) * 0.02 + 1e-6 * ref.abs().max().item()   # as test_gemm_parity
+    assert (y.double() - ref).abs().max().item() <= tol
