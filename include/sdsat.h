@@ -393,7 +393,8 @@ SDSAT_API sdsat_status sdsat_debug_workspace(sdsat_ctx* ctx, int which, int rows
  * at once, else 2 * num_sms); otherwise *cs = 1 and *nclusters = min(pairs, resident),
  * each CTA taking several pairs.  max_clusters[c] (c = 1..16, host array of 17 entries,
  * [0] unused) = the most clusters of c CTAs the device holds at once, as
- * cudaOccupancyMaxActiveClusters reports it for the attention kernel.  Errors: EINVAL. */
+ * cudaOccupancyMaxActiveClusters reports it for the attention kernel.  The launches also cap
+ * cs at the cache's 64-slot units.  Errors: EINVAL. */
 SDSAT_API sdsat_status sdsat_attention_grid(int pairs, const int32_t* max_clusters, int cs_cap, int num_sms,
                                             int* cs, int* nclusters);
 

@@ -623,7 +623,10 @@ void attention_grid(int pairs, const int* maxc, int cs_cap, int num_sms, int* cs
 
 cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st, bool pdl) {
   AttnParams p = p0;
-  attention_grid(p.nb * p.H, g_att_clusters[p.hd == 128][p.q > 8], g_att_cs_cap, num_sms, &p.cs, &p.nclusters);
+  // No more CTAs per pair than the cache has units: the others only widened the merge (one
+  // sequence, 32 heads, us per launch: capacity 106 6.64 -> 5.28, 506 6.72 -> 6.41).
+  attention_grid(p.nb * p.H, g_att_clusters[p.hd == 128][p.q > 8],
+                 std::min(g_att_cs_cap, (p.cap + ATT_UNIT - 1) / ATT_UNIT), num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
