@@ -817,10 +817,6 @@ static cudaLaunchConfig_t make_cfg(dim3 grid, dim3 block, cudaStream_t st, bool 
   return cfg;
 }
 
-cudaError_t accept_prepare() {
-  return cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NucList));
-}
-
 cudaError_t launch_accept(const AcceptParams& p0, cudaStream_t st, bool pdl) {
   AcceptParams p = p0;
   p.cs = std::min(ACC_CS, (p.V + ACC_SPAN - 1) / ACC_SPAN);   // (a larger vocabulary is greedy only)
@@ -1093,6 +1089,19 @@ cudaError_t launch_add_len(int* len, int seq, int n, int cap, uint32_t* err, cud
 __global__ void exp_kernel(const float* in, float* out, int n) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = exp_sd(in[i]);
+}
+
+cudaError_t accept_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NucList));
+  if (e == cudaSuccess) e = prefer_shared(accept_kernel);
+  if (e == cudaSuccess) e = prefer_shared(rmsnorm_kernel);
+  if (e == cudaSuccess) e = prefer_shared(split_kernel);
+  if (e == cudaSuccess) e = prefer_shared(build_block_kernel);
+  if (e == cudaSuccess) e = prefer_shared(tree_prep_kernel);
+  if (e == cudaSuccess) e = prefer_shared(tree_compact_kernel);
+  if (e == cudaSuccess) e = prefer_shared(commit_kernel);
+  if (e == cudaSuccess) e = prefer_shared(add_len_kernel);
+  return e;
 }
 
 cudaError_t launch_exp(const float* in, float* out, int n, cudaStream_t st) {

@@ -562,6 +562,7 @@ int g_att_cs_cap = ATT_CS_MAX;   // SDSAT_ATT_CLUSTER_MAX: the largest cluster s
 template <int HD, int QT>
 cudaError_t prepare_decode_kernel(int (&maxc)[ATT_CS_MAX + 1]) {
   cudaError_t e;
+  if ((e = prefer_shared(attention_kernel<HD, QT>)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attention_kernel<HD, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)AttCfg<HD, QT>::SMEM)) != cudaSuccess)
     return e;

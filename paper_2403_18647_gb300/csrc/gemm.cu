@@ -67,9 +67,12 @@ struct GemmCfg {
   static constexpr int W_BYTES = 128 * 128;      // 128 rows x 64 bf16
   static constexpr int X_BYTES = MPAD * 128;     // MPAD rows x 64 bf16 (hi or lo)
   static constexpr int STAGE_BYTES = W_BYTES + 2 * X_BYTES;
-  static constexpr int STAGING = 128 * (MPAD + 1) + 128;   // [128][MPAD+1] exchange + [128/MPAD][MPAD] sums
+  static constexpr int STAGING = 128 * (MPAD + 1) + 128;   // [128][MPAD+1] exchange + [PARTS][MPAD] sums
   static constexpr int ACC_COLS = 2 * MPAD;     // hi and lo products side by side
-  static constexpr int TMEM_COLS = 2 * ACC_COLS;  // two accumulators
+  // two accumulators (an allocation is a power of two, at least 32 columns)
+  static constexpr int TMEM_COLS = MPAD <= 8 ? 32 : (MPAD <= 16 ? 64 : (MPAD <= 32 ? 128 : 256));
+  // parts of a tile's 128 rows that the sums of h^2 are first added up in
+  static constexpr int PARTS = MPAD <= 8 ? 16 : (MPAD <= 16 ? 8 : (MPAD <= 32 ? 4 : 2));
   static constexpr int NBAR = 2 * STAGES + 6;
   static constexpr int CS = MPAD * 64;           // EPI_QKV: RoPE (cos, sin) of every row and frequency
   // residual rows loaded before the accumulator wait: every row up to 32 (MPAD 64 keeps
@@ -157,9 +160,10 @@ __device__ __forceinline__ void epilogue_final(const GemmParams& p, int tile, in
     }
     named_bar_sync(1, 128);
     // pass 1: thread (part, m) sums lanes part*RPP .. part*RPP+RPP-1 of row m
-    constexpr int PARTS = 128 / MPAD, RPP = 128 / PARTS;   // parts of the 128 lanes, lanes per part
+    constexpr int PARTS = GemmCfg<MPAD>::PARTS, RPP = 128 / PARTS;
+    static_assert(PARTS * MPAD <= 128, "one thread per (part, row)");
     float* part_sum = staging + 128 * (MPAD + 1);          // [PARTS][MPAD], beyond the [128][MPAD+1] block
-    {
+    if (r < PARTS * MPAD) {
       const int m = r % MPAD, part = r / MPAD;
       float sq = 0.f;
       if (m < M) {
@@ -605,21 +609,53 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
     trace_write(p.trace, (unsigned)s_mark[3], t_entry, t_wait, s_mark[0], s_mark[1], s_mark[2], globaltimer_ns());
 }
 
-int gemm_mpad(int M) { return M <= 16 ? 16 : (M <= 32 ? 32 : 64); }
+// Rows are padded to a multiple of 8 up to 32 (16 is the smallest N of the MMA: 8 rows, hi and
+// lo), then to 64: the operand's padding costs L2 -> SM traffic, shared memory and epilogue time.
+// us per launch, 6 rows padded to 16 -> 8: QKV 21.6 -> 20.9, O 12.4 -> 11.4, gate/up 34.7 -> 33.4,
+// down 20.8 -> 19.6, LM head 46.5 -> 44.6; 24 rows, 32 -> 24: 24.7 -> 23.6, 16.3 -> 15.2, 39.5 -> 37.8,
+// 25.5 -> 24.1, 52.0 -> 49.9.  A fifth stage in the room that 8 rows leave was slower (386.9 against
+// 383.5 us for four layers and LM head); so were 48 rows with two CTAs per SM (gate/up 44.3 -> 47.4).
+int gemm_mpad(int M) { return M <= 32 ? (M + 7) / 8 * 8 : 64; }
 
-size_t gemm_smem_bytes(int mpad) {
-  return mpad == 16 ? GemmCfg<16>::SMEM : (mpad == 32 ? GemmCfg<32>::SMEM : GemmCfg<64>::SMEM);
+namespace {
+template <typename F>
+cudaError_t with_mpad(int mpad, F&& f) {   // f.operator()<MPAD>()
+  switch (mpad) {
+    case 8: return f.template operator()<8>();
+    case 16: return f.template operator()<16>();
+    case 24: return f.template operator()<24>();
+    case 32: return f.template operator()<32>();
+    default: return f.template operator()<64>();
+  }
 }
+struct PrepareGemm {
+  template <int MPAD>
+  cudaError_t operator()() const {
+    static_assert(GemmCfg<MPAD>::SMEM <= (MPAD <= 32 ? 115712 : 232448), "CTAs per SM");
+    // (MPAD 64 runs one CTA per SM and leaves no room for the next kernel's: it keeps its L1)
+    const cudaError_t e = MPAD <= 32 ? prefer_shared(gemm_kernel<MPAD>) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(gemm_kernel<MPAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)GemmCfg<MPAD>::SMEM);
+  }
+};
+struct LaunchGemm {
+  const GemmParams& p;
+  cudaLaunchConfig_t& cfg;
+  template <int MPAD>
+  cudaError_t operator()() const {
+    cfg.dynamicSmemBytes = GemmCfg<MPAD>::SMEM;
+    return cudaLaunchKernelEx(&cfg, gemm_kernel<MPAD>, p);
+  }
+};
+}  // namespace
 
 cudaError_t gemm_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)GemmCfg<16>::SMEM);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)GemmCfg<32>::SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)GemmCfg<64>::SMEM);
+  for (int mpad : GEMM_MPADS) {
+    const cudaError_t e = with_mpad(mpad, PrepareGemm{});
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Tiles of at most this many chunks are not split when each can have a CTA of its own: a chunk
@@ -636,7 +672,6 @@ static int gemm_grid(const GemmParams& p, int num_sms) {
 }
 
 cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl) {
-  const int mpad = gemm_mpad(p.M);
   p.P = gemm_grid(p, num_sms);
   if ((long long)p.n_tiles * p.kc * p.P >= (1LL << 31)) return cudaErrorInvalidValue;   // 32-bit split math
   // Snapping costs the next CTA up to `snap` units, so it is used only where a CTA's share
@@ -646,16 +681,13 @@ cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.P);
   cfg.blockDim = dim3(192);
-  cfg.dynamicSmemBytes = gemm_smem_bytes(mpad);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (mpad == 16) return cudaLaunchKernelEx(&cfg, gemm_kernel<16>, p);
-  if (mpad == 32) return cudaLaunchKernelEx(&cfg, gemm_kernel<32>, p);
-  return cudaLaunchKernelEx(&cfg, gemm_kernel<64>, p);
+  return with_mpad(gemm_mpad(p.M), LaunchGemm{p, cfg});
 }
 
 }  // namespace sdsat

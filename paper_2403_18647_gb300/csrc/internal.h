@@ -40,8 +40,18 @@ __device__ __forceinline__ void trace_write(const Trace& t, unsigned int flags, 
   r[7] = t1;
 }
 
+// Every kernel of a step asks for the largest shared-memory carve-out.  An SM whose L1 / shared
+// split differs from what the next kernel asks for has to drain before it changes it, so with
+// mixed carve-outs no CTA of the next kernel starts beside the last ones of the previous.  (7B
+// layers, 6 rows, four layers and LM head: GEMM CTAs of 82 KB took 412 us beside attention's,
+// which fill the SM, and 389 us when padded to 98 KB or with this attribute.)
+template <typename K>
+cudaError_t prefer_shared(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 // ---- skinny weight-streaming GEMM --------------------------------------------
-// CTAs per SM of the skinny GEMM's grid for M <= 32 (compile-time tuning; one for M > 32).
+// CTAs per SM of the skinny GEMM's grid for M <= 32 (compile-time tuning; one beyond).
 // Every user of the grid size (the split-K partials, the fixed scratch of the
 // scratch-free entry point) sizes its buffers from this constant.
 #ifndef SDSAT_GEMM_CTAS_PER_SM
@@ -108,8 +118,8 @@ struct GemmParams {
   Trace trace;
 };
 
-int gemm_mpad(int M);                 // 16, 32 or 64
-size_t gemm_smem_bytes(int mpad);
+int gemm_mpad(int M);                 // rows of the operand boxes: 8, 16, 24, 32 or 64
+constexpr int GEMM_MPADS[] = {8, 16, 24, 32, 64};
 cudaError_t gemm_prepare();           // set smem attributes (idempotent)
 cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 
@@ -240,7 +250,7 @@ struct AcceptParams {
   int cs;                   // CTAs per row (set by launch_accept)
   uint32_t* err;
 };
-cudaError_t accept_prepare();
+cudaError_t accept_prepare();   // attributes of every kernel of accept.cu
 constexpr int TREE_WS_STRIDE = SDSAT_ATT_MAXQ + 2;
 constexpr int TREE_MAX_ROWS = 64;   // rows of one block forward (the tree kernels run one thread per row)
 cudaError_t launch_accept(const AcceptParams& p, cudaStream_t st, bool pdl);

@@ -141,9 +141,9 @@ extern "C" sdsat_status sdsat_gemm_static(const float* x_dev, int M, int K, cons
   int* counters = reinterpret_cast<int*>(s->scratch + SA_OFF_CNT);
   GemmParams g;
   std::memset(&g, 0, sizeof(g));
-  // the operand buffers hold SA_MAX_M rows of K columns; the kernel reads 16-row boxes
-  if (!encode(&g.tmap[0], w_dev, N, K, 64) || !encode(&g.tmap_x[0], xhi, SA_MAX_M, K, 16) ||
-      !encode(&g.tmap_x[1], xlo, SA_MAX_M, K, 16))
+  // the operand buffers hold SA_MAX_M rows of K columns; the kernel reads boxes of 8 or 16 rows
+  if (!encode(&g.tmap[0], w_dev, N, K, 64) || !encode(&g.tmap_x[0], xhi, SA_MAX_M, K, gemm_mpad(M)) ||
+      !encode(&g.tmap_x[1], xlo, SA_MAX_M, K, gemm_mpad(M)))
     return SDSAT_ECUDA;
   g.map_mode = MAP_PLAIN;
   g.N = N;

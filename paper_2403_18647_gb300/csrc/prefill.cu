@@ -606,6 +606,8 @@ cudaError_t prefill_prepare() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(prefill_gemm_kernel<128>, a, (int)PfCfg<128>::SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<64>, a, (int)PfCfg<64>::SMEM);
+  if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<128>);
+  if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<64>);
   if (e != cudaSuccess || g_pf_pairs > 0) return e;
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = pf_config(128, 1, nullptr, false, attr);

@@ -353,8 +353,10 @@ __global__ void __launch_bounds__(PA_THREADS, 1) prefill_attention_kernel(const 
 cudaError_t prefill_attention_prepare() {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(prefill_attention_kernel<64>, a, (int)PaCfg<64>::SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(prefill_attention_kernel<128>, a, (int)PaCfg<128>::SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_attention_kernel<128>, a, (int)PaCfg<128>::SMEM);
+  if (e == cudaSuccess) e = prefer_shared(prefill_attention_kernel<64>);
+  if (e == cudaSuccess) e = prefer_shared(prefill_attention_kernel<128>);
+  return e;
 }
 
 cudaError_t launch_prefill_attention(PfAttnParams& p, int num_sms, cudaStream_t st, bool pdl) {

@@ -77,7 +77,8 @@ bool make_kvmap(CUtensorMap* map, const void* ptr, long long rows, int hd) {
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int mpad_index(int M) { return M <= 16 ? 0 : (M <= 32 ? 1 : 2); }
+constexpr int N_MPADS = sizeof(GEMM_MPADS) / sizeof(GEMM_MPADS[0]);
+int mpad_index(int M) { return (int)(std::find(GEMM_MPADS, GEMM_MPADS + N_MPADS, gemm_mpad(M)) - GEMM_MPADS); }
 
 bool aligned16(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -142,7 +143,7 @@ struct sdsat_ctx {
   CUtensorMap pf_xmap[2][X_COUNT][2];   // boxes of 64 x 128 and 64 x 64
   __nv_bfloat16* x_hi[X_COUNT] = {};
   __nv_bfloat16* x_lo[X_COUNT] = {};
-  CUtensorMap xmap[X_COUNT][3][2];     // [source][MPAD 16/32/64][hi/lo]
+  CUtensorMap xmap[X_COUNT][N_MPADS][2];   // [source][GEMM_MPADS][hi/lo]
   __nv_bfloat16* xop_hi = nullptr;     // operand scratch of sdsat_op_gemm
   __nv_bfloat16* xop_lo = nullptr;
   std::vector<void*> allocs;
@@ -682,9 +683,9 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   const int xcols[X_COUNT] = {d, R, F};
   for (int xs = 0; ok && xs < X_COUNT; ++xs) {
     ok = dalloc(c, &c->x_hi[xs], (size_t)rows * xcols[xs]) && dalloc(c, &c->x_lo[xs], (size_t)rows * xcols[xs]);
-    for (int mi = 0; ok && mi < 3; ++mi)
-      ok = make_xmap(&c->xmap[xs][mi][0], c->x_hi[xs], rows, xcols[xs], 16 << mi) &&
-           make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], 16 << mi);
+    for (int mi = 0; ok && mi < N_MPADS; ++mi)
+      ok = make_xmap(&c->xmap[xs][mi][0], c->x_hi[xs], rows, xcols[xs], GEMM_MPADS[mi]) &&
+           make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], GEMM_MPADS[mi]);
   }
   if (ok && c->has_weights) {
     // the prefill workspaces in one allocation
@@ -1126,8 +1127,8 @@ sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const
   }
   GemmParams g = gemm_base(c, M, -1);
   CUtensorMap m;
-  if (!make_wmap(&m, w_dev, N, K) || !make_xmap(&g.tmap_x[0], c->xop_hi, SDSAT_MAX_ROWS, K, 16 << mpad_index(M)) ||
-      !make_xmap(&g.tmap_x[1], c->xop_lo, SDSAT_MAX_ROWS, K, 16 << mpad_index(M)))
+  if (!make_wmap(&m, w_dev, N, K) || !make_xmap(&g.tmap_x[0], c->xop_hi, SDSAT_MAX_ROWS, K, gemm_mpad(M)) ||
+      !make_xmap(&g.tmap_x[1], c->xop_lo, SDSAT_MAX_ROWS, K, gemm_mpad(M)))
     return SDSAT_ECUDA;
   set_plain(g, m, N, K);
   if (launch_split(x_dev, M, K, c->xop_hi, c->xop_lo, c->stream, c->pdl) != cudaSuccess) return SDSAT_ECUDA;
