@@ -31,7 +31,7 @@
 // Each CTA's run over its units of a pair ends in a partial result (row max,
 // exp-sum, unnormalised output) that it leaves in its own shared memory; after
 // a cluster barrier every CTA merges its share of the pair's output elements
-// from the cs partials through distributed shared memory, in rank order with
+// from the cs partials through distributed shared memory, in a fixed order with
 // the usual log-sum-exp rescaling (deterministic), and writes them in fp32 and
 // as the O projection's bf16 hi + lo operand.  A second cluster barrier keeps
 // the partials in place until every CTA of the cluster has read them.
@@ -477,45 +477,61 @@ __global__ void __launch_bounds__(128, QT == 1 ? 3 : 1) attention_kernel(const _
     if (p.trace.rec) t_part = globaltimer_ns();
     cluster_sync_all();   // the cluster's cs partials of the pair are complete
     // ---- merge this CTA's share of the pair's (row, 4 dimensions) outputs over the cs
-    // partials, read in rank order from the cluster's shared memory: w_r = exp(m_r - max m),
+    // partials, read from the cluster's shared memory: w_r = exp(m_r - max m),
     // L = sum_r w_r l_r, O = (sum_r w_r o_r) / L.  The second cluster barrier only keeps the
     // partials in place until every CTA has read them, so each thread arrives at it right
     // after its last remote loads and waits only at the end: the barrier's round trip
     // overlaps the merge arithmetic and the output stores.
+    // Few threads have an item (18 of 128 with 11 CTAs), and this code runs once per launch and is
+    // fetched cold, so G lanes share an item, each with at most four of the cs partials: one
+    // thread with an unrolled loop over 16 took 1.5 us from the loads to the stores with 11 CTAs.
     bool arrived = false;
     {
+      const int G = CS <= 4 ? 1 : (CS <= 8 ? 2 : 4), gl = tid & (G - 1), per = 128 / G;
       const int items = q * D4, i0 = items * rank / CS, i1 = items * (rank + 1) / CS;
-      for (int it = i0 + tid; it < i1; it += 128) {
+      const int passes = (i1 - i0 + per - 1) / per;
+#pragma unroll 1
+      for (int pass = 0; pass < passes; ++pass) {
+        const int mine = i0 + pass * per + tid / G, it = min(mine, i1 - 1);   // (every lane shuffles)
         const int j = it / D4, d4 = it - j * D4;
         const uint32_t a_ml = smem_u32(pml + 2 * j), a_o = smem_u32(po + j * HD + 4 * d4);
-        float2 ml[ATT_CS_MAX];
-        float4 ov[ATT_CS_MAX];
+        float2 ml[4];
+        float4 ov[4];
 #pragma unroll
-        for (int r = 0; r < ATT_CS_MAX; ++r)
+        for (int u = 0; u < 4; ++u) {
+          const int r = gl + u * G;
+          ml[u] = make_float2(-INFINITY, 0.f);
+          ov[u] = make_float4(0.f, 0.f, 0.f, 0.f);
           if (r < CS) {
-            ml[r] = ld_dsmem_f2(mapa_shared(a_ml, r));
-            ov[r] = ld_dsmem_f4(mapa_shared(a_o, r));
+            ml[u] = ld_dsmem_f2(mapa_shared(a_ml, r));
+            ov[u] = ld_dsmem_f4(mapa_shared(a_o, r));
           }
-        if (it + 128 >= i1) {   // this thread's last item: its reads of the partials are done
+        }
+        if (pass + 1 == passes) {   // this thread's reads of the partials are done
           cluster_arrive_thread();
           arrived = true;
         }
-        float mx = -INFINITY;
-#pragma unroll
-        for (int r = 0; r < ATT_CS_MAX; ++r)
-          if (r < CS) mx = fmaxf(mx, ml[r].x);
+        float mx = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
+        for (int o = 1; o < G; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float L = 0.f;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int r = 0; r < ATT_CS_MAX; ++r)
-          if (r < CS) {
-            const float w = (ml[r].x == -INFINITY) ? 0.f : __expf(ml[r].x - mx);
-            L += w * ml[r].y;
-            a.x += w * ov[r].x;
-            a.y += w * ov[r].y;
-            a.z += w * ov[r].z;
-            a.w += w * ov[r].w;
-          }
+        for (int u = 0; u < 4; ++u) {
+          const float w = (ml[u].x == -INFINITY) ? 0.f : __expf(ml[u].x - mx);
+          L += w * ml[u].y;
+          a.x += w * ov[u].x;
+          a.y += w * ov[u].y;
+          a.z += w * ov[u].z;
+          a.w += w * ov[u].w;
+        }
+        for (int o = 1; o < G; o <<= 1) {
+          L += __shfl_xor_sync(0xffffffffu, L, o);
+          a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+          a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+          a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
+          a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
+        }
+        if (gl || mine >= i1) continue;
         const float iv = 1.0f / L;
         const float4 o = make_float4(a.x * iv, a.y * iv, a.z * iv, a.w * iv);
         const size_t idx = (size_t)(sl * q + j) * p.out_ld + h * HD + 4 * d4;
@@ -626,8 +642,12 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   AttnParams p = p0;
   // No more CTAs per pair than the cache has units: the others only widened the merge (one
   // sequence, 32 heads, us per launch: capacity 106 6.64 -> 5.28, 506 6.72 -> 6.41).
-  attention_grid(p.nb * p.H, g_att_clusters[p.hd == 128][p.q > 8],
-                 std::min(g_att_cs_cap, (p.cap + ATT_UNIT - 1) / ATT_UNIT), num_sms, &p.cs, &p.nclusters);
+  // With head dimension 64 two more spare clusters (32 heads, context 8192: 11 CTAs 20.3 us, 10
+  // CTAs 18.4; context 2000 10.1 and 8.5; 40 heads keep 9).
+  const int* maxc = g_att_clusters[p.hd == 128][p.q > 8];
+  int cap = std::min(g_att_cs_cap, (p.cap + ATT_UNIT - 1) / ATT_UNIT);
+  if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (p.nb * p.H + ATT_SPARE_CLUSTERS + 2)));
+  attention_grid(p.nb * p.H, maxc, cap, num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
