@@ -12,8 +12,7 @@
 // Work: the grid is nclusters thread-block clusters of cs CTAs, all resident
 // at once (launch_attention picks the largest cs <= ATT_CS_MAX for which one
 // cluster per (sequence, head) pair fits on the GPU with room to spare; else
-// cs = 1 and each CTA takes several pairs).  Three CTAs fit on an SM for q <= 8
-// (two for q <= 16).  Cluster c takes the pairs c, c + nclusters, ...; the
+// cs = 1 and each CTA takes several pairs).  Three CTAs fit on an SM.  Cluster c takes the pairs c, c + nclusters, ...; the
 // nu units of ATT_UNIT = 64 consecutive slots of a pair are split over the
 // cluster's CTAs as [r*nu/cs, (r+1)*nu/cs) for CTA rank r.  One thread keeps a
 // two-stage ring of K and V tiles (TMA, boxes of 64 dims x 64 rows, 128-byte
@@ -52,6 +51,7 @@ constexpr int ATT_PREFETCH = 4;   // units past the ring requested into L2 ahead
 // 5.303 -> 5.256 ms), while shorter slices (batch 4 at context 1024: 5-6 units) lose more from
 // the later units' missed L2 hits than they gain (attention 13.7 -> 15.1 us with 1)
 constexpr int ATT_LONG_SLICE = 7;
+constexpr size_t ATT_TWO_PER_SM = 96 * 1024;   // dynamic shared memory of which only two fit on an SM
 constexpr int ATT_SPARE_CLUSTERS = 8;   // room left for this many more clusters (measured: 7B/13B shapes, b = 1, 4)
 
 template <int HD, int QT = 2>
@@ -63,13 +63,16 @@ struct AttCfg {
   static constexpr int STAGE = 2 * TILE;                 // K then V
   static constexpr int QSTRIDE = HD * 2 + 16;            // bytes per row of the bf16 Q tiles (padded)
   static constexpr int PSTRIDE = ATT_UNIT * 2 + 16;      // bytes per row of the bf16 P tiles (padded)
-  static constexpr int RED = 17;                         // floats per row of the row-reduction scratch
   // Q hi + lo tiles; once the CTA's units of a pair are done, its partial output [ROWS][HD] fp32
   static constexpr size_t OFF_Q = (size_t)ATT_STAGES * STAGE;
-  // P hi + lo tiles
+  // P hi + lo tiles in their own area; with two query tiles of 128 dimensions over the unit's K
+  // tile, whose last reader has passed the barrier before P is written, so that three CTAs fit
+  // on an SM (75.9 KB instead of 81.5): 32 heads, 11 rows, context 16384 66.7 -> 55.9 us, three
+  // sequences of 16 rows, context 8000 110 -> 73, context 2048 13.3 -> 13.2
+  static constexpr bool P_OVER_K = QT == 2 && HD == 128;
   static constexpr size_t OFF_P = OFF_Q + 2 * ROWS * QSTRIDE;
-  static constexpr size_t OFF_RED = OFF_P + 2 * ROWS * PSTRIDE;   // [16][RED]: unit row max, sums; partial stats
-  static constexpr size_t OFF_SEQ = OFF_RED + 16 * RED * 4;                         // len, units [64]
+  static constexpr size_t OFF_RED = OFF_P + (P_OVER_K ? 0 : 2 * ROWS * PSTRIDE);   // unit row max, sums; partial stats
+  static constexpr size_t OFF_SEQ = OFF_RED + (128 + 2 * 16) * 4;                   // len, units [64]
   static constexpr size_t OFF_ANC = OFF_SEQ + (64 + 64) * 4;                        // [16] visible block rows per row
   static constexpr size_t OFF_BAR = (OFF_ANC + 16 * 4 + 7) / 8 * 8;
   static constexpr size_t SMEM = 1024 + OFF_BAR + ATT_STAGES * 8 + 16;
@@ -102,7 +105,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo_elem, float hi_elem) {
 
 // QT: tiles of 8 query rows (1 for q <= 8, 2 for q <= 16)
 template <int HD, int QT>
-__global__ void __launch_bounds__(128, QT == 1 ? 3 : 1) attention_kernel(const __grid_constant__ AttnParams p) {
+__global__ void __launch_bounds__(128, 3) attention_kernel(const __grid_constant__ AttnParams p) {
   using C = AttCfg<HD, QT>;
   constexpr int KSTEPS = HD / 16;          // MMA k-steps over the head dimension
   constexpr int MT = HD / 64;              // 16-dimension tiles per warp in V^T P^T
@@ -113,8 +116,6 @@ __global__ void __launch_bounds__(128, QT == 1 ? 3 : 1) attention_kernel(const _
   uint8_t* Qh = smem + C::OFF_Q;                    // bf16 [ROWS][HD] (scaled q, hi part), padded rows
   uint8_t* Ql = Qh + C::ROWS * C::QSTRIDE;          // lo part
   float* po = reinterpret_cast<float*>(smem + C::OFF_Q);        // [ROWS][HD] partial output (after the units)
-  uint8_t* Ph = smem + C::OFF_P;                    // bf16 [ROWS][ATT_UNIT] softmax numerators, hi part
-  uint8_t* Pl = Ph + C::ROWS * C::PSTRIDE;
   float* red = reinterpret_cast<float*>(smem + C::OFF_RED);     // row-reduction scratch [4][16] max, [4][16] sums
   float* pml = red + 128;                                       // [ROWS][2] partial row max, exp-sum (after the units)
   int* len_seq = reinterpret_cast<int*>(smem + C::OFF_SEQ);     // [64] committed length of each sequence
@@ -294,6 +295,8 @@ __global__ void __launch_bounds__(128, QT == 1 ? 3 : 1) attention_kernel(const _
       const int c0 = c * ATT_UNIT;                  // slot of the unit's first key
       const uint8_t* Kt = smem + (size_t)(k % ATT_STAGES) * C::STAGE;
       const uint8_t* Vt = Kt + C::TILE;
+      uint8_t* Ph = C::P_OVER_K ? const_cast<uint8_t*>(Kt) : smem + C::OFF_P;
+      uint8_t* Pl = Ph + C::ROWS * C::PSTRIDE;
       // one decision per warp (mma.sync needs every lane; a wait can run out for some only)
       const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[k % ATT_STAGES], (k / ATT_STAGES) & 1,
                                                               abort_flag, p.err));
@@ -364,6 +367,7 @@ __global__ void __launch_bounds__(128, QT == 1 ? 3 : 1) attention_kernel(const _
       __syncthreads();   // every warp is also done with the previous unit (its stage, P, red)
       if (tid == 0 && k >= 1 && isu.pi < npairs && !*abort_flag) {
         // refill the previous unit's stage with unit k + 1, extend the L2 window
+        if (C::P_OVER_K) fence_proxy_async_smem();   // the load overwrites P, written by every thread
         bool committed;
         issue(issued, unit_row(isu, committed));
         advance(isu);
@@ -580,7 +584,7 @@ cudaError_t prepare_decode_kernel(int (&maxc)[ATT_CS_MAX + 1]) {
   cudaError_t e;
   if ((e = prefer_shared(attention_kernel<HD, QT>)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(attention_kernel<HD, QT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)AttCfg<HD, QT>::SMEM)) != cudaSuccess)
+                                (int)std::max<size_t>(AttCfg<HD, QT>::SMEM, ATT_TWO_PER_SM))) != cudaSuccess)
     return e;
   if ((e = cudaFuncSetAttribute(attention_kernel<HD, QT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
       cudaSuccess)
@@ -651,7 +655,11 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
+  // Single CTAs that fit two to an SM: room for no third, or some SMs get three and others one
+  // (240 pairs, 10 rows, context 1000: 39.2 us against 32.9; 7 sequences of 4 rows, 32 heads, context 3000: 82 against 65).
   cfg.dynamicSmemBytes = attention_smem_bytes(p.hd, p.q);
+  if (p.cs == 1 && p.nclusters <= 2 * num_sms)
+    cfg.dynamicSmemBytes = std::max<size_t>(cfg.dynamicSmemBytes, ATT_TWO_PER_SM);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -446,3 +446,28 @@ def test_gemm_whole_and_split_tiles(tiny_ctx, M, K, N):
     ref = x.double() @ w.double().t()
     tol = 5e-5 * math.sqrt(K) * 0.02 + 1e-6 * ref.abs().max().item()   # as test_gemm_parity
     assert (y.double() - ref).abs().max().item() <= tol
+
+
+@pytest.mark.parametrize("b,q,H,hd", [(6, 10, 40, 128), (4, 16, 40, 64), (8, 8, 38, 128), (8, 8, 40, 128),
+                                      (5, 9, 32, 128), (1, 16, 1, 128), (1, 11, 32, 64), (7, 3, 44, 64)])
+def test_attention_grids(sd, b, q, H, hd):
+    """One to sixteen CTAs per (sequence, head), single CTAs that fit two to an SM and more of
+    them, both query-tile counts and head dimensions, ragged lengths down to an empty cache and
+    a cache filled to its last slot; against the explicit softmax in fp64."""
+    cap = 700
+    lens = [0, cap - q, 63, 64, 65, 300, 511, 129][:b]
+    shape = synth.ModelShape("att", 1, H * hd, H, hd, 256, 256, 0)
+    ctx = sd.Context(shape, None, max_position=64) if (H * hd) % 128 == 0 and H * hd <= 8192 else None
+    x = synth.normal_f32(21, b, (b * q, H * hd), 1.0, device="cuda")
+    k = synth.normal_bf16(21, 1, (b * H * cap, hd), 1.0, device="cuda").view(b, H, cap, hd)
+    v = synth.normal_bf16(21, 2, (b * H * cap, hd), 1.0, device="cuda").view(b, H, cap, hd)
+    out = torch.full((b * q, H * hd), float("nan"), device="cuda")
+    ctx.op_attention(x, k, v, torch.tensor(lens, dtype=torch.int32, device="cuda"), b, q, H, hd, cap, out)
+    assert ctx.get_error() == 0
+    for s, n in enumerate(lens):
+        qs = x[s * q:(s + 1) * q].double().view(q, H, hd)
+        sc = torch.einsum("qhd,hkd->hqk", qs, k[s, :, :n + q].double()) / math.sqrt(hd)
+        seen = torch.ones(q, n + q, dtype=torch.bool, device="cuda").tril(n)
+        ref = torch.einsum("hqk,hkd->qhd", sc.masked_fill(~seen, float("-inf")).softmax(-1), v[s, :, :n + q].double())
+        # operands as bf16 hi + lo (2^-16 relative), fp32 sums, outputs of order one
+        assert (out[s * q:(s + 1) * q].double().view(q, H, hd) - ref).abs().max().item() <= 2e-5
