@@ -173,10 +173,7 @@ cudaError_t prefill_attention_prepare();
 cudaError_t launch_prefill_attention(PfAttnParams& p, int num_sms, cudaStream_t st, bool pdl);
 
 // ---- prefill (prompt chunks of up to PF_ROWS positions) -------------------------
-#ifndef SDSAT_PF_ROWS
-#define SDSAT_PF_ROWS 2048
-#endif
-constexpr int PF_ROWS = SDSAT_PF_ROWS;
+constexpr int PF_ROWS = 4096;   // 4095 positions, two 7B layers: 4.53 ms in one chunk, 4.64 in two
 struct PfGemmParams {
   CUtensorMap tmap[3];      // weights, as GemmParams::tmap (map_mode)
   CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [rows][K], boxes of 64 x prefill_tok(M)

@@ -133,12 +133,13 @@ struct sdsat_ctx {
   int* tree_ws = nullptr;      // [SDSAT_MAX_ROWS][TREE_WS_STRIDE] tree commit: len, m, path
   int* adaptive = nullptr;
   uint32_t* err = nullptr;
-  // prefill workspaces (chunks of up to PF_ROWS positions; allocated with the weights)
-  float* pf_h = nullptr;         // [PF_ROWS][d] residual stream
-  float* pf_ssq = nullptr;       // [PF_ROWS][ssq_ld] per-tile sums of h^2
-  __nv_bfloat16 *pf_qhi = nullptr, *pf_qlo = nullptr;   // [PF_ROWS][R] rotated queries
+  // prefill workspaces (chunks of up to pf_rows positions; allocated with the weights)
+  int pf_rows = 0;
+  float* pf_h = nullptr;         // [pf_rows][d] residual stream
+  float* pf_ssq = nullptr;       // [pf_rows][ssq_ld] per-tile sums of h^2
+  __nv_bfloat16 *pf_qhi = nullptr, *pf_qlo = nullptr;   // [pf_rows][R] rotated queries
   CUtensorMap pf_qmap[2];               // boxes of 64 x 128
-  __nv_bfloat16* pf_hi[X_COUNT] = {};   // GEMM operands [PF_ROWS][K] (normed x, attention, act)
+  __nv_bfloat16* pf_hi[X_COUNT] = {};   // GEMM operands [pf_rows][K] (normed x, attention, act)
   __nv_bfloat16* pf_lo[X_COUNT] = {};
   CUtensorMap pf_xmap[2][X_COUNT][2];   // boxes of 64 x 128 and 64 x 64
   __nv_bfloat16* x_hi[X_COUNT] = {};
@@ -403,7 +404,7 @@ sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const 
   return SDSAT_OK;
 }
 
-// one prefill chunk: M <= PF_ROWS prompt positions of sequence seq
+// one prefill chunk: M <= pf_rows prompt positions of sequence seq
 // through every layer on the tiled GEMM, then committed
 sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* tokens, int M) {
   const sdsat_config& cf = c->cfg;
@@ -688,8 +689,9 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
            make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], GEMM_MPADS[mi]);
   }
   if (ok && c->has_weights) {
-    // the prefill workspaces in one allocation
-    const size_t pr = PF_ROWS;
+    // the prefill workspaces in one allocation; a prompt is no longer than max_position
+    c->pf_rows = (int)std::min<long long>(PF_ROWS, ((long long)cfg->max_position + 127) / 128 * 128);
+    const size_t pr = c->pf_rows;
     uint8_t* arena = nullptr;
     size_t used = 0;
     for (int pass = 0; ok && pass < 2; ++pass) {
@@ -708,12 +710,12 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
         take(&c->pf_lo[xs], pr * xcols[xs]);
       }
     }
-    ok = ok && make_xmap(&c->pf_qmap[0], c->pf_qhi, PF_ROWS, R, 128) &&
-         make_xmap(&c->pf_qmap[1], c->pf_qlo, PF_ROWS, R, 128);
+    ok = ok && make_xmap(&c->pf_qmap[0], c->pf_qhi, c->pf_rows, R, 128) &&
+         make_xmap(&c->pf_qmap[1], c->pf_qlo, c->pf_rows, R, 128);
     for (int xs = 0; ok && xs < X_COUNT; ++xs)
       for (int i = 0; ok && i < 2; ++i)
-        ok = make_xmap(&c->pf_xmap[i][xs][0], c->pf_hi[xs], PF_ROWS, xcols[xs], 128 >> i) &&
-             make_xmap(&c->pf_xmap[i][xs][1], c->pf_lo[xs], PF_ROWS, xcols[xs], 128 >> i);
+        ok = make_xmap(&c->pf_xmap[i][xs][0], c->pf_hi[xs], c->pf_rows, xcols[xs], 128 >> i) &&
+             make_xmap(&c->pf_xmap[i][xs][1], c->pf_lo[xs], c->pf_rows, xcols[xs], 128 >> i);
   }
   if (!ok) {
     sdsat_destroy(c);
@@ -876,8 +878,8 @@ sdsat_status sdsat_prefill(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
                : SDSAT_ECUDA;
   }
   // Chunks of equal size up to the position block: every chunk streams all the weights, so
-  // none is left with a few positions (a 4095-position prompt: 2048 + 2047; 2050: 1152 + 898).
-  const int chunks = (n + PF_ROWS - 1) / PF_ROWS;
+  // none is left with a few positions (8191: 4096 + 4095; 4100: 2176 + 1924).
+  const int chunks = (n + c->pf_rows - 1) / c->pf_rows;
   const int per = chunks ? ((n + chunks - 1) / chunks + 127) / 128 * 128 : 0;
   for (int i = 0; i < n; i += per) {
     const sdsat_status s = prefill_chunk(c, kv, seq, tokens_dev + i, std::min(per, n - i));

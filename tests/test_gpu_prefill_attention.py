@@ -21,7 +21,7 @@ def model(request):
     H, hd = request.param
     shape = dataclasses.replace(synth.SHAPES["7b"], name="edge", n_layers=2, d_model=512, n_heads=H, head_dim=hd,
                                 ffn_dim=384, vocab=1000, adaptive_id=999)
-    return shape, sd.Context(shape, synth.make_model(shape, seed=5, device="cuda", gain_std=0.1), max_position=4096)
+    return shape, sd.Context(shape, synth.make_model(shape, seed=5, device="cuda", gain_std=0.1), max_position=8192)
 
 
 def _blocks(ctx, kv, ids, start):
@@ -33,7 +33,7 @@ def _blocks(ctx, kv, ids, start):
 
 
 @pytest.mark.parametrize("start", [0, 37])
-@pytest.mark.parametrize("n", [17, 64, 65, 127, 128, 129, 256, 257, 700, 1000, 2200])
+@pytest.mark.parametrize("n", [17, 64, 65, 127, 128, 129, 256, 257, 700, 1000, 2200, 4200])
 def test_prefill_attention_edges(model, n, start):
     shape, ctx = model
     ids = synth.prompt_ids(7, n, n + start, 900).cuda()
