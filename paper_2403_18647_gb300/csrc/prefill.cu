@@ -41,7 +41,7 @@ constexpr int PF_W_BYTES = 128 * 128;                    // a CTA's 128 weight r
 constexpr int PF_CHUNK = 32;                             // positions per epilogue round
 constexpr int PF_EPI_WARPS = 8;                          // two per TMEM lane quarter
 constexpr int PF_THREADS = 64 + 32 * PF_EPI_WARPS;
-constexpr int PF_STAGING = 2 * 128 * PF_CHUNK;           // fp32 exchange of the two epilogue groups
+constexpr int PF_STAGING = 2 * 128 * PF_CHUNK;           // fp32 slabs of the two epilogue groups
 constexpr int PF_GROUP = 8;                              // position blocks numbered together (16: no better, 32: 4 % slower)
 constexpr int PF_TOK = 128;                              // positions per tile, at most
 constexpr int PF_SK_MIN = 4;                             // chunks of a split-K share, at least
@@ -55,7 +55,7 @@ struct PfCfg {
   static constexpr int RING = STAGES * STAGE;
   static constexpr int ACC = 2 * TOK;                    // TMEM columns of one accumulator (hi, lo)
   static constexpr int ROUNDS = TOK / (2 * PF_CHUNK);    // epilogue rounds of each of the two warp groups
-  static constexpr int NBAR = 2 * STAGES + 6;
+  static constexpr int NBAR = 2 * STAGES + 7;
   static constexpr size_t SMEM = 1024 + (size_t)RING + PF_STAGING * 4 + 2 * TOK * 4 + NBAR * 8 + 64;
   static_assert(SMEM <= 232448, "shared memory of one CTA");
 };
@@ -119,6 +119,20 @@ __device__ __forceinline__ void pf_tile(const PfGemmParams& p, int tile, int& wp
   tb = g * p.group + rem - wp * width;
 }
 
+// two bf16 in a word (a in the low half); four values as bf16 hi + lo at element o (8-byte aligned)
+__device__ __forceinline__ uint32_t pf_pack(float a, float b) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
+         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+}
+__device__ __forceinline__ void pf_store4(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t o, float a, float b, float c,
+                                          float d) {
+  const uint32_t h0 = pf_pack(a, b), h1 = pf_pack(c, d);
+  *reinterpret_cast<uint2*>(hi + o) = make_uint2(h0, h1);
+  *reinterpret_cast<uint2*>(lo + o) =
+      make_uint2(pf_pack(a - __uint_as_float(h0 << 16), b - __uint_as_float(h0 & 0xFFFF0000u)),
+                 pf_pack(c - __uint_as_float(h1 << 16), d - __uint_as_float(h1 & 0xFFFF0000u)));
+}
+
 __device__ __forceinline__ void pf_drain(uint64_t* bar, uint32_t parity) {
   const uint64_t t0 = globaltimer_ns();
   while (!mbar_try_wait(bar, parity))
@@ -141,7 +155,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
   uint64_t* acc_empty = acc_full + 2;          // [2] rank 0: accumulator drained in both CTAs
   uint64_t* drain = acc_empty + 2;
   uint64_t* red_bar = drain + 1;               // parts of the tile being reduced landed (bulk copies)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(red_bar + 1);
+  uint64_t* res_bar = red_bar + 1;             // a round's residual rows landed in the slabs
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* s_last = reinterpret_cast<int*>(tmem_slot + 2);
   // trace marks of the epilogue: after the dependency wait, first and last accumulator, last tile summed
@@ -162,6 +177,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     }
     mbar_init(drain, 1);
     mbar_init(red_bar, 1);
+    mbar_init(res_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -300,12 +316,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     const int r = e * 32 + lane;         // the CTA's weight row
     const int tid = threadIdx.x - 64;
     constexpr int NE = 32 * PF_EPI_WARPS;
-    // exchange between the group's 128 rows: element (row, j) at row * 32 + (j ^ lane of the
-    // row), so that a warp's rows fall on different banks
-    float* xch = staging + grp * 128 * PF_CHUNK;
-    int round = 0;
+    float* slab = staging + grp * 128 * PF_CHUNK;   // [32 positions][128 rows] of the group's round
+    const int w8 = ((warp - 2) & 3) * 8;            // this warp finishes the round's positions w8 .. w8 + 7
     const uint32_t acc_empty0 = mapa_shared(smem_u32(acc_empty), 0);
     const int U = p.sk_tiles * p.kc;
+    uint32_t res_ph = 0;
     pdl_wait();   // residual rows and outputs belong to the previous kernels' results
     if (p.trace.rec) t_wait = globaltimer_ns();
     const int len0 = p.epi == EPI_QKV ? __ldcg(p.len + p.seq) : 0;
@@ -317,6 +332,22 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
       const int wt = 2 * wp + rank;
       const int buf = seg & 1;
       const int mt = tb * TOK;   // the tile's first position
+      const int vr = min(TOK, p.M - mt);   // the tile's positions
+      const bool shared = w.k1 - w.k0 < p.kc;
+      // EPI_RESID: a round's residual rows (512 bytes a position) go into the slabs by bulk
+      // copies, for the first round of a whole tile while the tensor cores work; the values are
+      // then added to them there.  Loading them when the sums were ready took 5 us per tile.
+      const uint32_t res_bytes = p.epi == EPI_RESID ? 4u * max(0, min(128, p.N - 128 * wt)) : 0u;
+      auto load_resid = [&](int b0) {
+        const int cnt = min(2 * PF_CHUNK, vr - b0);
+        if (tid == 0) mbar_arrive_expect_tx(res_bar, cnt * res_bytes);
+        named_bar_sync(1, NE);   // every read of the slabs is done; the bytes are announced
+        if (tid < cnt && res_bytes) {
+          fence_proxy_async_smem();
+          bulk_load_g2s(staging + tid * 128, p.out + (size_t)(mt + b0 + tid) * p.out_ld + 128 * wt, res_bytes, res_bar);
+        }
+      };
+      if (p.epi == EPI_RESID && !shared) load_resid(0);
       const float* inv = s_inv + (seg & 1) * TOK;
       if (p.ssq_in) {
         // RMSNorm factors of the tile's positions while the tensor cores work: eight lanes sum a
@@ -331,7 +362,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
         }
       }
       const bool got = named_bar_and(1, NE, mbar_wait_bounded(&acc_full[buf], (seg >> 1) & 1, abort_flag, p.err));
-      if (!got) break;
+      if (!got) {
+        if (p.epi == EPI_RESID && !shared && tid == 0) pf_drain(res_bar, res_ph);   // copies in flight land
+        break;
+      }
       tc_fence_after();
       if (p.trace.rec) {
         t_acc1 = globaltimer_ns();
@@ -357,8 +391,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc_empty0 + buf * 8);
       };
-      const bool shared = w.k1 - w.k0 < p.kc;
-      const int vr = min(TOK, p.M - mt);   // the tile's positions
       int lo = 0, hi = 0, batch = 0;
       if (shared) {
         // a split tile: publish this pair's part; the last contributor sums the parts in pair
@@ -391,13 +423,17 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
         t_sum = globaltimer_ns();
         t_flags += shared ? 0x101 : 0x100;
       }
-      // Rounds of 2 x 32 positions.  This code runs a few times per launch and is fetched cold,
-      // so it stays rolled: with the rounds unrolled the epilogue took twice as long.
+      // Rounds of 2 x 32 positions.  This code runs a few times per launch and is fetched cold, so
+      // it stays small: rolled rounds, and the values go through shared memory so that a few
+      // vector instructions finish a position (a row per thread, 32 positions unrolled, took 16.6 us
+      // from the last MMA to the end of the O projection at 99 positions, 12.5 now; QKV 12.1, 8.7).
       bool ok = true;
 #pragma unroll 1
       for (int b0 = 0; b0 < vr; b0 += 2 * PF_CHUNK) {
         const int c0 = b0 + grp * PF_CHUNK, m0 = mt + c0;
-        if (batch && b0 % batch == 0) {
+        const bool fetch = batch && b0 % batch == 0;
+        if (p.epi == EPI_RESID && (shared || b0 > 0)) load_resid(b0);
+        if (fetch) {
           const uint32_t bytes = (uint32_t)min(batch, vr - b0) * 512;
           const int cnt = hi - lo + 1;
           if (tid == 0) mbar_arrive_expect_tx(red_bar, cnt * bytes);
@@ -408,158 +444,189 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
                           p.partials + ((size_t)((lo + tid) * 2 + (tid == 0)) * 2 + rank) * PF_TOK * 128 + b0 * 128,
                           bytes, red_bar);
           }
-          const uint32_t ph = (b0 / batch) & 1;
-          ok = named_bar_and(1, NE, mbar_wait_bounded(red_bar, ph, abort_flag, p.err));
+        }
+        if (fetch || p.epi == EPI_RESID) {
+          const uint32_t ph = batch ? (b0 / batch) & 1 : 0;
+          bool in = !fetch || mbar_wait_bounded(red_bar, ph, abort_flag, p.err);
+          if (p.epi == EPI_RESID) in = in && mbar_wait_bounded(res_bar, res_ph, abort_flag, p.err);
+          ok = named_bar_and(1, NE, in);
           if (!ok) {
-            if (tid == 0) pf_drain(red_bar, ph);   // copies in flight land before the CTA exits
+            if (tid == 0) {   // copies in flight land before the CTA exits
+              if (fetch) pf_drain(red_bar, ph);
+              if (p.epi == EPI_RESID) pf_drain(res_bar, res_ph);
+            }
             break;
           }
+          if (p.epi == EPI_RESID) res_ph ^= 1u;
         }
         if (c0 >= vr) break;   // the second group, in the tile's last round
-        float y[PF_CHUNK];
+        // The round's values, position-major, into the slab: from the accumulator each thread
+        // writes its row (all positions), from the parts of a split tile each warp sums its own
+        // eight positions.
         if (!shared) {
+          float y[PF_CHUNK];
           load_acc(c0, y);
           if (b0 + 2 * PF_CHUNK >= TOK || c0 + 2 * PF_CHUNK >= vr) drained();
-        } else {
+          if (p.epi == EPI_STORE) {   // nothing to combine: straight to memory, a row per thread
+            const int n = 128 * wt + r;
+            float* dst = p.out + (size_t)m0 * p.out_ld + n;
+            const int cnt = n < p.N ? vr - c0 : 0;
 #pragma unroll
-          for (int j = 0; j < PF_CHUNK; ++j) y[j] = 0.f;
-          if (batch) {
-            const int rows = min(batch, vr - b0 / batch * batch);
-            const float* src = reinterpret_cast<const float*>(stages) + (c0 - b0 / batch * batch) * 128 + r;
-#pragma unroll 1
-            for (int q = lo; q <= hi; ++q, src += rows * 128)
+            for (int j = 0; j < PF_CHUNK; ++j)
+              if (j < cnt) dst[(size_t)j * p.out_ld] = y[j];
+            continue;
+          }
+          if (p.epi == EPI_RESID) {
 #pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j) y[j] += src[j * 128];
+            for (int j = 0; j < PF_CHUNK; ++j) y[j] += slab[j * 128 + r];
           } else {
-            // (positions past the tile's last read rows of the part that are not used)
+            named_bar_sync(2 + grp, 128);   // the last round's reads of the slab are done
+          }
+#pragma unroll
+          for (int j = 0; j < PF_CHUNK; ++j) slab[j * 128 + r] = y[j];
+          named_bar_sync(2 + grp, 128);
+        } else {
+          // (positions past the tile's last read rows that are not used)
+          float4 v[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            v[k] = p.epi == EPI_RESID ? reinterpret_cast<const float4*>(slab + (w8 + k) * 128)[lane]
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+          const int base = batch ? b0 / batch * batch : 0;
+          const int rows = min(batch, vr - base);
 #pragma unroll 1
-            for (int q = lo; q <= hi; ++q) {
-              const float* src = p.partials + ((size_t)(q * 2 + (q == lo)) * 2 + rank) * PF_TOK * 128 + c0 * 128 + r;
-              float v[PF_CHUNK];
+          for (int q = lo; q <= hi; ++q) {
+            const float* src = batch ? reinterpret_cast<const float*>(stages) + ((q - lo) * rows + c0 - base + w8) * 128
+                                     : p.partials + (((size_t)(q * 2 + (q == lo)) * 2 + rank) * PF_TOK + c0 + w8) * 128;
+            float4 t[8];
 #pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j) v[j] = __ldcg(src + j * 128);
-#pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j) y[j] += v[j];
+            for (int k = 0; k < 8; ++k) {
+              const float4* a = reinterpret_cast<const float4*>(src + k * 128) + lane;
+              t[k] = batch ? *a : __ldcg(a);
             }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k].x += t[k].x, v[k].y += t[k].y, v[k].z += t[k].z, v[k].w += t[k].w;
           }
-        }
-        if (p.ssq_in) {
+          if (p.epi == EPI_STORE) {
+            const int n = 128 * wt + 4 * lane, cnt = vr - c0 - w8;
+            float* dst = p.out + (size_t)(m0 + w8) * p.out_ld + n;
+            const bool vec = (p.out_ld & 3) == 0 && (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0 && n + 4 <= p.N;
 #pragma unroll
-          for (int j = 0; j < PF_CHUNK; ++j) y[j] *= inv[c0 + j];
-        }
-        if (p.epi == EPI_SWIGLU) {
-          // tile rows 0-63: gate features 64*wt + r, rows 64-127: the matching up features; the
-          // gate thread takes the round's first 16 positions, the up thread the other 16
-          const int f = 64 * wt + (r & 63);
-          const bool gate = r < 64;
-#pragma unroll
-          for (int j = 0; j < PF_CHUNK / 2; ++j) xch[r * PF_CHUNK + (j ^ lane)] = gate ? y[16 + j] : y[j];
-          named_bar_sync(2 + grp, 128);
-          const float* other = xch + (r ^ 64) * PF_CHUNK;
-          if (wt < p.n_wtiles && f < p.N) {
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK / 2; ++j) {
-              const int m = m0 + (gate ? j : 16 + j);
-              if (m < p.M) {
-                const float x = other[j ^ lane];
-                const float g = gate ? y[j] : x, up = gate ? x : y[16 + j];
-                const float a = g / (1.0f + expf(-g)) * up;
-                const __nv_bfloat16 h = __float2bfloat16_rn(a);
-                p.out_hi[(size_t)m * p.out_ld + f] = h;
-                p.out_lo[(size_t)m * p.out_ld + f] = __float2bfloat16_rn(a - __bfloat162float(h));
+            for (int k = 0; k < 8; ++k)
+              if (k < cnt) {
+                float* d = dst + (size_t)k * p.out_ld;
+                if (vec) {
+                  *reinterpret_cast<float4*>(d) = v[k];
+                } else {
+                  if (n < p.N) d[0] = v[k].x;
+                  if (n + 1 < p.N) d[1] = v[k].y;
+                  if (n + 2 < p.N) d[2] = v[k].z;
+                  if (n + 3 < p.N) d[3] = v[k].w;
+                }
               }
-            }
+            continue;
           }
-          named_bar_sync(2 + grp, 128);
+          __syncwarp();
+#pragma unroll
+          for (int k = 0; k < 8; ++k) reinterpret_cast<float4*>(slab + (w8 + k) * 128)[lane] = v[k];
+          __syncwarp();
+        }
+        // Each warp finishes its eight positions, lanes along the rows (features): vector loads
+        // and stores, and little code (see above).
+        const int left = min(8, vr - c0 - w8);   // (may be <= 0)
+        if (p.epi == EPI_SWIGLU) {
+          // rows 0-63: gate features 64*wt + .., rows 64-127: the matching up features; half a
+          // warp per position
+          const int i = 4 * (lane & 15), f = 64 * wt + i;
+#pragma unroll 2
+          for (int k = lane >> 4; k < left; k += 2) {
+            const float* row = slab + (w8 + k) * 128 + i;
+            const float4 g = *reinterpret_cast<const float4*>(row), u = *reinterpret_cast<const float4*>(row + 64);
+            const float s = p.ssq_in ? inv[c0 + w8 + k] : 1.f;
+            auto act = [&](float x, float up) { return x * s / (1.0f + expf(-(x * s))) * (up * s); };
+            if (wt < p.n_wtiles && f < p.N)
+              pf_store4(p.out_hi, p.out_lo, (size_t)(m0 + w8 + k) * p.out_ld + f, act(g.x, u.x), act(g.y, u.y),
+                        act(g.z, u.z), act(g.w, u.w));
+          }
         } else if (p.epi == EPI_QKV) {
           // The tile lies in one of q, k, v and holds whole heads.  RoPE (rotate-half) pairs row
-          // r with row r ^ hd/2; position m0 + j sits at slot (and position) len + m0 + j.
-          const int R = p.rows_per_map, g = 128 * wt;
-          const int which = (g >= R) + (g >= 2 * R);
-          const int f = g - which * R + r, half = p.hd >> 1, i = f & (p.hd - 1);
-          const int slot0 = len0 + m0;
-          if (which < 2 && wt < p.n_wtiles) {
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j) xch[r * PF_CHUNK + (j ^ lane)] = y[j];
-            named_bar_sync(2 + grp, 128);
-            const float* other = xch + (r ^ half) * PF_CHUNK;
-            const float sgn = i < half ? -1.f : 1.f;
-            const float2* cs = p.rope + (i & (half - 1));
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j) {
-              const float2 t = __ldg(cs + (size_t)min(slot0 + j, p.rope_len - 1) * half);
-              y[j] = y[j] * t.x + sgn * (other[j ^ lane] * t.y);
-            }
-            named_bar_sync(2 + grp, 128);
-          }
+          // i of a head with row i + hd/2; position m sits at slot (and position) len + m.  Half
+          // a warp per position, four pairs of rows a lane.
+          const int R = p.rows_per_map, g0 = 128 * wt, half = p.hd >> 1;
+          const int which = (g0 >= R) + (g0 >= 2 * R);
+          const int x = 4 * (lane & 15), i = x & (half - 1), r1 = (x - i) * 2 + i;   // rows r1 .. and r1 + half ..
+          const int f = g0 - which * R + r1;   // feature of row r1 within its matrix
           if (wt < p.n_wtiles) {
-            const int valid = min(PF_CHUNK, p.M - m0);
-            if (which == 0) {
-              const size_t o = (size_t)m0 * p.out_ld + f;
-#pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j)
-                if (j < valid) {
-                  const __nv_bfloat16 h = __float2bfloat16_rn(y[j]);
-                  p.out_hi[o + (size_t)j * p.out_ld] = h;
-                  p.out_lo[o + (size_t)j * p.out_ld] = __float2bfloat16_rn(y[j] - __bfloat162float(h));
-                }
-            } else {
-              const int fits = min(valid, p.cap - slot0);
-              __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
-                                   ((size_t)(p.seq * p.H + f / p.hd) * p.cap + slot0) * p.hd + i;
-#pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j)
-                if (j < fits) dst[j * p.hd] = __float2bfloat16_rn(y[j]);
-              if (r == 0 && fits < valid) set_error(p.err, ERR_CAPACITY);
-              if (r == 0 && slot0 + valid > p.rope_len) set_error(p.err, ERR_POSITION);
+#pragma unroll 2
+            for (int k = lane >> 4; k < left; k += 2) {
+              const float* row = slab + (w8 + k) * 128 + r1;
+              float4 a = *reinterpret_cast<const float4*>(row), b = *reinterpret_cast<const float4*>(row + half);
+              const float s = p.ssq_in ? inv[c0 + w8 + k] : 1.f;
+              a.x *= s, a.y *= s, a.z *= s, a.w *= s, b.x *= s, b.y *= s, b.z *= s, b.w *= s;
+              const int m = m0 + w8 + k, slot = len0 + m;
+              if (which < 2) {
+                const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)min(slot, p.rope_len - 1) * half + i);
+                const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);   // cos, sin of two frequencies each
+                const float4 c = make_float4(t0.x, t0.z, t1.x, t1.z), n = make_float4(t0.y, t0.w, t1.y, t1.w);
+                const float4 o = a;
+                a = make_float4(a.x * c.x - b.x * n.x, a.y * c.y - b.y * n.y, a.z * c.z - b.z * n.z, a.w * c.w - b.w * n.w);
+                b = make_float4(b.x * c.x + o.x * n.x, b.y * c.y + o.y * n.y, b.z * c.z + o.z * n.z, b.w * c.w + o.w * n.w);
+              }
+              if (which == 0) {
+                const size_t o = (size_t)m * p.out_ld + f;
+                pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
+                pf_store4(p.out_hi, p.out_lo, o + half, b.x, b.y, b.z, b.w);
+              } else if (slot < p.cap) {
+                __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
+                                     ((size_t)(p.seq * p.H + (f - i) / p.hd) * p.cap + slot) * p.hd + i;
+                *reinterpret_cast<uint2*>(dst) = make_uint2(pf_pack(a.x, a.y), pf_pack(a.z, a.w));
+                *reinterpret_cast<uint2*>(dst + half) = make_uint2(pf_pack(b.x, b.y), pf_pack(b.z, b.w));
+              } else if (lane == 0 || lane == 16) {
+                set_error(p.err, ERR_CAPACITY);
+              }
+              if (slot >= p.rope_len && which && (lane & 15) == 0) set_error(p.err, ERR_POSITION);
             }
           }
         } else {
-          const int n = 128 * wt + r;
-          const bool in = n < p.N;
-          float* dst = p.out + (size_t)m0 * p.out_ld + n;
-          const int valid = in ? min(PF_CHUNK, p.M - m0) : 0;
-          if (p.epi == EPI_RESID) {
-            float hv[PF_CHUNK];
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j) hv[j] = j < valid ? __ldcg(dst + (size_t)j * p.out_ld) : 0.f;
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j) y[j] += hv[j];
-          }
-#pragma unroll
-          for (int j = 0; j < PF_CHUNK; ++j)
-            if (j < valid) dst[(size_t)j * p.out_ld] = y[j];
-          if (p.gain_next) {
-            // the next RMSNorm's operand h * g, and this weight tile's sum of h^2 per position:
-            // halving exchanges leave position j's sum over the warp's rows on lane j, the
-            // group's four warps add up through shared memory (two buffers, one barrier)
-            const float gn = in ? __bfloat162float(p.gain_next[n]) : 0.f;
-            const size_t o = (size_t)m0 * p.out_ld + n;
-#pragma unroll
-            for (int j = 0; j < PF_CHUNK; ++j) {
-              const float x = y[j] * gn;
-              const __nv_bfloat16 h = __float2bfloat16_rn(x);
-              if (j < valid) {
-                p.out_hi[o + (size_t)j * p.out_ld] = h;
-                p.out_lo[o + (size_t)j * p.out_ld] = __float2bfloat16_rn(x - __bfloat162float(h));
-              }
-              y[j] = j < valid ? y[j] * y[j] : 0.f;
+          const int n = 128 * wt + 4 * lane;
+          const float* row = slab + w8 * 128 + 4 * lane;
+          float* dst = p.out + (size_t)(m0 + w8) * p.out_ld + n;
+          {
+            // (N and the row stride are multiples of 8.)  The residual row is updated; with gain_next
+            // also the next RMSNorm's operand h * g and this weight tile's sum of h^2 per position
+            const bool in = n < p.N;
+            float g[4] = {0.f, 0.f, 0.f, 0.f};
+            if (p.gain_next && in) {
+              const uint2 gb = __ldg(reinterpret_cast<const uint2*>(p.gain_next + n));
+              g[0] = __uint_as_float(gb.x << 16), g[1] = __uint_as_float(gb.x & 0xFFFF0000u);
+              g[2] = __uint_as_float(gb.y << 16), g[3] = __uint_as_float(gb.y & 0xFFFF0000u);
             }
+#pragma unroll 1
+            for (int k = 0; k < left; k += 4, row += 512, dst += 4 * (size_t)p.out_ld) {
+              float4 h[4];
+              float sq[4];
 #pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) {
-              const bool up = lane & o2;
+              for (int u = 0; u < 4; ++u) {
+                const bool on = in && k + u < left;
+                h[u] = *reinterpret_cast<const float4*>(row + u * 128);
+                sq[u] = on ? (h[u].x * h[u].x + h[u].y * h[u].y) + (h[u].z * h[u].z + h[u].w * h[u].w) : 0.f;
+                if (on) {
+                  *reinterpret_cast<float4*>(dst + (size_t)u * p.out_ld) = h[u];
+                  if (p.gain_next)
+                    pf_store4(p.out_hi, p.out_lo, (size_t)(m0 + w8 + k + u) * p.out_ld + n, h[u].x * g[0],
+                              h[u].y * g[1], h[u].z * g[2], h[u].w * g[3]);
+                }
+              }
+              if (p.gain_next) {
 #pragma unroll
-              for (int j = 0; j < o2; ++j) {
-                const float send = up ? y[j] : y[j + o2], keep = up ? y[j + o2] : y[j];
-                y[j] = keep + __shfl_xor_sync(0xffffffffu, send, o2);
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) sq[u] += __shfl_xor_sync(0xffffffffu, sq[u], o);
+                if (lane < 4 && k + lane < left && wt < p.n_wtiles)
+                  p.ssq_out[(size_t)(m0 + w8 + k + lane) * p.ssq_ld + wt] =
+                      lane == 0 ? sq[0] : (lane == 1 ? sq[1] : (lane == 2 ? sq[2] : sq[3]));
               }
             }
-            float* part = xch + (round++ & 1) * 128;
-            part[e * 32 + lane] = y[0];
-            named_bar_sync(2 + grp, 128);
-            if (e == 0 && m0 + lane < p.M && wt < p.n_wtiles)
-              p.ssq_out[(size_t)(m0 + lane) * p.ssq_ld + wt] =
-                  (part[lane] + part[32 + lane]) + (part[64 + lane] + part[96 + lane]);
           }
         }
       }
