@@ -181,10 +181,11 @@ struct PfGemmParams {
   int N;                    // output features (MAP_GATEUP: F)
   int kc;                   // 64-column chunks of K
   int n_wtiles;             // tiles of 128 weight rows
-  int n_pairs_w;            // pairs of weight tiles (set by launch_prefill_gemm, as the next four)
-  int n_tblocks;            // blocks of prefill_tok(M) positions
+  int n_pairs_w;            // pairs of weight tiles (set by plan_prefill_gemm, as the next five fields)
+  int tok, n_tblocks;       // blocks of tok = prefill_tok(M) positions
   int group;                // position blocks numbered together
   int sk_tiles, sk_pairs;   // the first sk_tiles tiles are split along K over the first sk_pairs CTA pairs
+  int publish;              // every tile is split and a second kernel sums the parts and runs the epilogue
   int M;                    // positions
   float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]
   int* counters;            // [2 * num_sms], zero between launches
@@ -213,7 +214,10 @@ struct PfGemmParams {
 cudaError_t prefill_prepare();
 int prefill_tok(int M);      // positions per tile of the GEMM over M positions: 64 or 128
 size_t prefill_partials(int num_sms);
-cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl);
+// The tile list and split of a GEMM (M, epi, N, kc and n_wtiles set).  With p.publish the next
+// operand of EPI_RESID (gain_next) is the normalised one, else h * g with sums of h^2 in ssq_out.
+void plan_prefill_gemm(PfGemmParams& p, int num_sms);
+cudaError_t launch_prefill_gemm(const PfGemmParams& p, cudaStream_t st, bool pdl);
 
 // ---- embedding, acceptance, block building ------------------------------------
 // x = h * rsqrt(mean h^2 + eps) * g, stored as bf16 hi + lo (tokens != null: h = E[tokens] first)

@@ -133,6 +133,31 @@ __device__ __forceinline__ void pf_store4(__nv_bfloat16* hi, __nv_bfloat16* lo, 
                  pf_pack(c - __uint_as_float(h1 << 16), d - __uint_as_float(h1 & 0xFFFF0000u)));
 }
 
+// rotate-half RoPE of a head's dimensions i .. i + 3 (a) and i + hd/2 .. (b) at position `slot`
+__device__ __forceinline__ void pf_rope4(const PfGemmParams& p, int slot, int i, float4& a, float4& b) {
+  const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)min(slot, p.rope_len - 1) * (p.hd >> 1) + i);
+  const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);   // cos, sin of two frequencies each
+  const float4 o = a;
+  a = make_float4(a.x * t0.x - b.x * t0.y, a.y * t0.z - b.y * t0.w, a.z * t1.x - b.z * t1.y, a.w * t1.z - b.w * t1.w);
+  b = make_float4(b.x * t0.x + o.x * t0.y, b.y * t0.z + o.y * t0.w, b.z * t1.x + o.z * t1.y, b.w * t1.z + o.w * t1.w);
+}
+// features f .. f + 3 (a) and f + hd/2 .. (b) of chunk position m: q as bf16 hi + lo, k and v into
+// the cache slot when there is one
+__device__ __forceinline__ void pf_qkv_store(const PfGemmParams& p, int which, int m, int slot, int f, int i,
+                                             const float4& a, const float4& b) {
+  const int half = p.hd >> 1;
+  if (which == 0) {
+    const size_t o = (size_t)m * p.out_ld + f;
+    pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
+    pf_store4(p.out_hi, p.out_lo, o + half, b.x, b.y, b.z, b.w);
+  } else if (slot < p.cap) {
+    __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
+                         ((size_t)(p.seq * p.H + (f - i) / p.hd) * p.cap + slot) * p.hd + i;
+    *reinterpret_cast<uint2*>(dst) = make_uint2(pf_pack(a.x, a.y), pf_pack(a.z, a.w));
+    *reinterpret_cast<uint2*>(dst + half) = make_uint2(pf_pack(b.x, b.y), pf_pack(b.z, b.w));
+  }
+}
+
 __device__ __forceinline__ void pf_drain(uint64_t* bar, uint32_t parity) {
   const uint64_t t0 = globaltimer_ns();
   while (!mbar_try_wait(bar, parity))
@@ -337,7 +362,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
       const int buf = seg & 1;
       const int mt = tb * TOK;   // the tile's first position
       const int vr = min(TOK, p.M - mt);   // the tile's positions
-      const bool shared = w.k1 - w.k0 < p.kc;
+      const bool shared = p.publish || w.k1 - w.k0 < p.kc;
       // EPI_RESID: a round's residual rows (512 bytes a position) go into the slabs by bulk
       // copies, for the first round of a whole tile while the tensor cores work; the values are
       // then added to them there.  Loading them when the sums were ready took 5 us per tile.
@@ -353,7 +378,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
       };
       if (p.epi == EPI_RESID && !shared) load_resid(0);
       const float* inv = s_inv + (seg & 1) * TOK;
-      if (p.ssq_in) {
+      if (p.ssq_in && !p.publish) {
         // RMSNorm factors of the tile's positions while the tensor cores work: eight lanes sum a
         // position's parts, in a fixed order (read after the barrier below)
         for (int c = tid >> 3; c < TOK; c += NE / 8) {
@@ -410,6 +435,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             if (c0 + j < vr) __stcg(mine + (c0 + j) * 128, y[j]);
         }
         drained();
+        if (p.publish) continue;   // a second kernel sums the parts
         lo = (w.tile * p.kc * p.sk_pairs + p.sk_pairs - 1) / U;
         hi = ((w.tile * p.kc + p.kc - 1) * p.sk_pairs + p.sk_pairs - 1) / U;
         named_bar_sync(1, NE);
@@ -568,26 +594,9 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
               const float s = p.ssq_in ? inv[c0 + w8 + k] : 1.f;
               a.x *= s, a.y *= s, a.z *= s, a.w *= s, b.x *= s, b.y *= s, b.z *= s, b.w *= s;
               const int m = m0 + w8 + k, slot = len0 + m;
-              if (which < 2) {
-                const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)min(slot, p.rope_len - 1) * half + i);
-                const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);   // cos, sin of two frequencies each
-                const float4 c = make_float4(t0.x, t0.z, t1.x, t1.z), n = make_float4(t0.y, t0.w, t1.y, t1.w);
-                const float4 o = a;
-                a = make_float4(a.x * c.x - b.x * n.x, a.y * c.y - b.y * n.y, a.z * c.z - b.z * n.z, a.w * c.w - b.w * n.w);
-                b = make_float4(b.x * c.x + o.x * n.x, b.y * c.y + o.y * n.y, b.z * c.z + o.z * n.z, b.w * c.w + o.w * n.w);
-              }
-              if (which == 0) {
-                const size_t o = (size_t)m * p.out_ld + f;
-                pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
-                pf_store4(p.out_hi, p.out_lo, o + half, b.x, b.y, b.z, b.w);
-              } else if (slot < p.cap) {
-                __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
-                                     ((size_t)(p.seq * p.H + (f - i) / p.hd) * p.cap + slot) * p.hd + i;
-                *reinterpret_cast<uint2*>(dst) = make_uint2(pf_pack(a.x, a.y), pf_pack(a.z, a.w));
-                *reinterpret_cast<uint2*>(dst + half) = make_uint2(pf_pack(b.x, b.y), pf_pack(b.z, b.w));
-              } else if (lane == 0 || lane == 16) {
-                set_error(p.err, ERR_CAPACITY);
-              }
+              if (which < 2) pf_rope4(p, slot, i, a, b);
+              pf_qkv_store(p, which, m, slot, f, i, a, b);
+              if (slot >= p.cap && which && (lane & 15) == 0) set_error(p.err, ERR_CAPACITY);
               if (slot >= p.rope_len && which && (lane & 15) == 0) set_error(p.err, ERR_POSITION);
             }
           }
@@ -649,6 +658,132 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
   }
 }
 
+// ---- the second kernel of a GEMM whose every tile is split -------------------------------
+// With fewer tiles than pairs (O and down projections up to some 500 positions, QKV up to 128)
+// the last contributors of the tiles, 32 of 152 CTAs at 99 positions, summed the parts and ran
+// the epilogue alone: 10 to 12 us after the last MMA, bound by the bytes and latency of one CTA
+// each.  Instead all CTAs only publish, and a kernel of one CTA per position (and matrix, for
+// QKV) does the rest on every SM (prefill of two 7B layers, 99 positions: 273 -> 239 us, 200:
+// 355 -> 337, 512: 609 -> 603).  A position's CTA has its whole row, so RMSNorm is applied here
+// and the next GEMM needs no factor.
+constexpr int PF_FIN_THREADS = 512;
+constexpr int PF_FIN_PARTS = 6;   // parts loaded together
+
+// the contributors lo .. hi of (weight tile wt, position block tb), and the start of lo's part of
+// row `pos`; the other parts follow from part_of()
+struct PfParts {
+  int lo, hi;
+  const float* base;
+  __device__ PfParts(const PfGemmParams& p, int wt, int tb, int pos) {
+    const int g = tb / p.group, width = min(p.group, p.n_tblocks - g * p.group);
+    const int tile = g * p.n_pairs_w * p.group + (wt >> 1) * width + tb - g * p.group;
+    const int U = p.sk_tiles * p.kc;
+    lo = (tile * p.kc * p.sk_pairs + p.sk_pairs - 1) / U;
+    hi = ((tile * p.kc + p.kc - 1) * p.sk_pairs + p.sk_pairs - 1) / U;
+    base = p.partials + (size_t)(wt & 1) * PF_TOK * 128 + pos * 128;
+  }
+  __device__ const float* part(int q) const { return base + (size_t)(q * 2 + (q == lo)) * 2 * PF_TOK * 128; }
+};
+
+__device__ __forceinline__ void pf_add(float4& a, const float4& b) {
+  a.x += b.x, a.y += b.y, a.z += b.z, a.w += b.w;
+}
+
+// sum of v over the CTA, in a fixed order
+__device__ __forceinline__ float pf_block_sum(float v, float* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = (threadIdx.x & 31) < PF_FIN_THREADS / 32 ? red[threadIdx.x & 31] : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// h += sum of the parts; with gain_next the next GEMM's operand RMSNorm(h)
+__global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_resid_kernel(const __grid_constant__ PfGemmParams p) {
+  constexpr int I = 64 * 128 / (4 * PF_FIN_THREADS);   // float4 of a row per thread: rows of up to 8192
+  __shared__ float red[32];
+  pdl_wait();
+  pdl_trigger();
+  const int m = blockIdx.x, tok = p.tok, tb = m / tok, pos = m - tb * tok;
+  float* row = p.out + (size_t)m * p.out_ld;
+  float4 h[I];
+  float sq = 0.f;
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const int n = 4 * ((int)threadIdx.x + i * PF_FIN_THREADS);
+    h[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n >= p.N) break;
+    const PfParts w(p, n >> 7, tb, pos);
+    const float4 old = __ldcg(reinterpret_cast<const float4*>(row + n));
+    for (int q = w.lo; q <= w.hi; q += PF_FIN_PARTS) {
+      float4 t[PF_FIN_PARTS];
+#pragma unroll
+      for (int u = 0; u < PF_FIN_PARTS; ++u)
+        t[u] = q + u <= w.hi ? __ldcg(reinterpret_cast<const float4*>(w.part(q + u) + (n & 127)))
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(h[i], t[u]);
+    }
+    pf_add(h[i], old);
+    *reinterpret_cast<float4*>(row + n) = h[i];
+    sq += (h[i].x * h[i].x + h[i].y * h[i].y) + (h[i].z * h[i].z + h[i].w * h[i].w);
+  }
+  if (!p.gain_next) return;
+  const float inv = 1.0f / sqrtf(pf_block_sum(sq, red) / (float)p.norm_dim + p.norm_eps);
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const int n = 4 * ((int)threadIdx.x + i * PF_FIN_THREADS);
+    if (n >= p.N) break;
+    const uint2 g = __ldg(reinterpret_cast<const uint2*>(p.gain_next + n));
+    pf_store4(p.out_hi, p.out_lo, (size_t)m * p.out_ld + n, h[i].x * inv * __uint_as_float(g.x << 16),
+              h[i].y * inv * __uint_as_float(g.x & 0xFFFF0000u), h[i].z * inv * __uint_as_float(g.y << 16),
+              h[i].w * inv * __uint_as_float(g.y & 0xFFFF0000u));
+  }
+}
+
+// RoPE on the queries and keys of a position, KV append (blockIdx.y: q, k, v)
+__global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_qkv_kernel(const __grid_constant__ PfGemmParams p) {
+  pdl_wait();
+  pdl_trigger();
+  const int m = blockIdx.x, which = blockIdx.y, tok = p.tok, tb = m / tok, pos = m - tb * tok;
+  const int R = p.rows_per_map, half = p.hd >> 1, slot = __ldcg(p.len + p.seq) + m;
+  float s = 1.f;
+  if (p.ssq_in) {
+    float q = 0.f;
+    for (int t = 0; t < p.ssq_ld; ++t) q += __ldcg(p.ssq_in + (size_t)m * p.ssq_ld + t);
+    s = 1.0f / sqrtf(q / (float)p.norm_dim + p.norm_eps);
+  }
+  if (threadIdx.x == 0 && which == 1) {
+    if (slot >= p.cap) set_error(p.err, ERR_CAPACITY);
+    if (slot >= p.rope_len) set_error(p.err, ERR_POSITION);
+  }
+  for (int x = 4 * (int)threadIdx.x; x < R / 2; x += 4 * PF_FIN_THREADS) {
+    // four pairs of features: i .. i + 3 of a head and those half a head further
+    const int i = x & (half - 1), f = (x - i) * 2 + i;   // head * hd + i
+    const PfParts w(p, (which * R + f) >> 7, tb, pos), v(p, (which * R + f + half) >> 7, tb, pos);
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+    for (int q = w.lo; q <= w.hi; q += PF_FIN_PARTS) {   // (a head lies in one tile: both rows have the same parts)
+      float4 t[PF_FIN_PARTS], u4[PF_FIN_PARTS];
+#pragma unroll
+      for (int u = 0; u < PF_FIN_PARTS; ++u) {
+        t[u] = u4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q + u <= w.hi) {
+          t[u] = __ldcg(reinterpret_cast<const float4*>(w.part(q + u) + (f & 127)));
+          u4[u] = __ldcg(reinterpret_cast<const float4*>(v.part(q + u) + ((f + half) & 127)));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(a, t[u]), pf_add(b, u4[u]);
+    }
+    a.x *= s, a.y *= s, a.z *= s, a.w *= s, b.x *= s, b.y *= s, b.z *= s, b.w *= s;
+    if (which < 2) pf_rope4(p, slot, i, a, b);
+    pf_qkv_store(p, which, m, slot, f, i, a, b);
+  }
+}
+
 namespace {
 int g_pf_pairs = 0;   // CTA pairs resident at once
 
@@ -676,6 +811,8 @@ cudaError_t prefill_prepare() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(prefill_gemm_kernel<64>, a, (int)PfCfg<64>::SMEM);
   if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<128>);
   if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<64>);
+  if (e == cudaSuccess) e = prefer_shared(prefill_finish_resid_kernel);
+  if (e == cudaSuccess) e = prefer_shared(prefill_finish_qkv_kernel);
   if (e != cudaSuccess || g_pf_pairs > 0) return e;
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = pf_config(128, 1, nullptr, false, attr);
@@ -689,8 +826,9 @@ int prefill_tok(int M) { return M <= 64 ? 64 : 128; }
 
 size_t prefill_partials(int num_sms) { return (size_t)(num_sms / 2) * 2 * 2 * PF_TOK * 128; }
 
-cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, bool pdl) {
+void plan_prefill_gemm(PfGemmParams& p, int num_sms) {
   const int tok = prefill_tok(p.M), P = std::max(1, std::min(num_sms / 2, g_pf_pairs));
+  p.tok = tok;
   p.n_pairs_w = (p.n_wtiles + 1) / 2;
   p.n_tblocks = (p.M + tok - 1) / tok;
   p.group = std::min(p.n_tblocks, PF_GROUP * (128 / tok));
@@ -699,14 +837,29 @@ cudaError_t launch_prefill_gemm(PfGemmParams& p, int num_sms, cudaStream_t st, b
   p.sk_pairs = 0;
   if (rem && (P - rem) * p.kc >= 8 * P) {
     p.sk_tiles = rem;
-    p.sk_pairs = std::max(rem, std::min(P, p.sk_tiles * p.kc / PF_SK_MIN));
+    p.sk_pairs = std::max(rem, std::min(P, rem * p.kc / PF_SK_MIN));
     if (p.sk_pairs == rem) p.sk_tiles = p.sk_pairs = 0;   // nothing to split
   }
+  p.publish = p.sk_tiles == T && (p.epi == EPI_RESID || p.epi == EPI_QKV);
+}
+
+cudaError_t launch_prefill_gemm(const PfGemmParams& p, cudaStream_t st, bool pdl) {
+  const int tok = prefill_tok(p.M), T = p.n_pairs_w * p.n_tblocks;
+  const int P = std::max(1, g_pf_pairs);
   cudaLaunchAttribute attr[2];
-  const cudaLaunchConfig_t cfg =
-      pf_config(tok, std::min(P, std::max(p.sk_pairs, T - p.sk_tiles)), st, pdl, attr);
-  return tok == 64 ? cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<64>, p)
-                   : cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<128>, p);
+  cudaLaunchConfig_t cfg = pf_config(tok, std::min(P, std::max(p.sk_pairs, T - p.sk_tiles)), st, pdl, attr);
+  const cudaError_t e = tok == 64 ? cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<64>, p)
+                                  : cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<128>, p);
+  if (e != cudaSuccess || !p.publish) return e;
+  cudaLaunchConfig_t fin = {};
+  fin.gridDim = p.epi == EPI_QKV ? dim3(p.M, 3) : dim3(p.M);
+  fin.blockDim = dim3(PF_FIN_THREADS);
+  fin.stream = st;
+  attr[0] = attr[1];
+  fin.attrs = attr;
+  fin.numAttrs = pdl ? 1 : 0;
+  return p.epi == EPI_QKV ? cudaLaunchKernelEx(&fin, prefill_finish_qkv_kernel, p)
+                          : cudaLaunchKernelEx(&fin, prefill_finish_resid_kernel, p);
 }
 
 }  // namespace sdsat

@@ -413,7 +413,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
   const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
   const int xi = prefill_tok(M) == 64;
   // RMSNorm folded into the GEMMs as in forward(): O and down emit the next operand and the
-  // sums of squares, gate/up and the next QKV scale by the factor
+  // sums of squares, gate/up and the next QKV scale by the factor (unless O or down ended in a
+  // kernel of its own, which normalises)
   auto fold_in = [&](PfGemmParams& g) {
     g.ssq_in = c->pf_ssq;
     g.ssq_ld = c->ssq_ld;
@@ -426,6 +427,8 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     g.out_lo = c->pf_lo[X_NORM];
     g.ssq_out = c->pf_ssq;
     g.ssq_ld = c->ssq_ld;
+    g.norm_dim = d;
+    g.norm_eps = cf.rms_eps;
   };
   auto base = [&](int xsrc, int K) {
     PfGemmParams g;
@@ -439,9 +442,12 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     g.err = c->err;
     return g;
   };
+  bool normed = true;   // the next GEMM's operand is already normalised (else h * g)
   auto gemm = [&](PfGemmParams& g) {
+    plan_prefill_gemm(g, c->num_sms);
+    if (g.epi == EPI_RESID) normed = g.publish;
     g.trace = next_trace(c, K_PF_GEMM);
-    return timed(c, K_PF_GEMM, [&] { return launch_prefill_gemm(g, c->num_sms, st, c->pdl); });
+    return timed(c, K_PF_GEMM, [&] { return launch_prefill_gemm(g, st, c->pdl); });
   };
   if (timed(c, K_RMSNORM, [&] {
         return launch_rmsnorm(tokens, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->pf_h, d, M,
@@ -472,7 +478,7 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gq.cap = kv->cap;
     gq.rope = c->rope;
     gq.rope_len = cf.max_position;
-    if (l > 0) fold_in(gq);
+    if (!normed) fold_in(gq);
     if (gemm(gq) != cudaSuccess) return SDSAT_ECUDA;
     // causal attention of the chunk's positions over the cache
     PfAttnParams a;
@@ -514,7 +520,7 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     gg.out_hi = c->pf_hi[X_FFN];
     gg.out_lo = c->pf_lo[X_FFN];
     gg.out_ld = F;
-    fold_in(gg);
+    if (!normed) fold_in(gg);
     if (gemm(gg) != cudaSuccess) return SDSAT_ECUDA;
     PfGemmParams gd = base(X_FFN, F);
     gd.tmap[0] = mp.down;
@@ -1123,7 +1129,8 @@ sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const
     g.err = c->err;
     g.trace = next_trace(c, K_GEMM_OP);
     if (launch_split(x_dev, M, K, c->xop_hi, c->xop_lo, c->stream, c->pdl) != cudaSuccess) return SDSAT_ECUDA;
-    return timed(c, K_GEMM_OP, [&] { return launch_prefill_gemm(g, c->num_sms, c->stream, c->pdl); }) == cudaSuccess
+    plan_prefill_gemm(g, c->num_sms);
+    return timed(c, K_GEMM_OP, [&] { return launch_prefill_gemm(g, c->stream, c->pdl); }) == cudaSuccess
                ? SDSAT_OK
                : SDSAT_ECUDA;
   }
