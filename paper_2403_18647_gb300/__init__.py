@@ -150,9 +150,20 @@ def attention_grid(pairs: int, max_clusters, cs_cap: int = 16, num_sms: int = 15
     return cs.value, nc.value
 
 
+_current_stream = None
+
+
 def _stream():
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    """The calling thread's current CUDA stream as an integer.  Every compute call asks for it:
+    torch.cuda.current_stream() builds a Stream object (2.8 us on the GB300's host, a third of a
+    small call's issue time); the raw query is 0.2 us."""
+    global _current_stream
+    if _current_stream is None:
+        import torch
+        torch.cuda.current_stream()   # CUDA is initialised before the raw query
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch._C._cuda_getDevice
+        _current_stream = (lambda: raw(device())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _current_stream()
 
 
 def make_config(shape, max_position: int = 8192, adaptive_ids=None) -> Config:
