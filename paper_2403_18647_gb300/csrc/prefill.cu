@@ -744,6 +744,32 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_resid_kernel(co
   }
 }
 
+// out = sum of the parts (blockIdx.y: 2048 features)
+__global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_store_kernel(const __grid_constant__ PfGemmParams p) {
+  pdl_wait();
+  pdl_trigger();
+  const int m = blockIdx.x, tb = m / p.tok, n = 4 * ((int)blockIdx.y * PF_FIN_THREADS + (int)threadIdx.x);
+  if (n >= p.N) return;
+  const PfParts w(p, n >> 7, tb, m - tb * p.tok);
+  float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int q = w.lo; q <= w.hi; q += PF_FIN_PARTS) {
+    float4 t[PF_FIN_PARTS];
+#pragma unroll
+    for (int u = 0; u < PF_FIN_PARTS; ++u)
+      t[u] = q + u <= w.hi ? __ldcg(reinterpret_cast<const float4*>(w.part(q + u) + (n & 127)))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(y, t[u]);
+  }
+  float* dst = p.out + (size_t)m * p.out_ld + n;
+  if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+    *reinterpret_cast<float4*>(dst) = y;
+  } else {
+    const float v[4] = {y.x, y.y, y.z, y.w};
+    for (int e = 0; e < 4 && n + e < p.N; ++e) dst[e] = v[e];
+  }
+}
+
 // RoPE on the queries and keys of a position, KV append (blockIdx.y: q, k, v)
 __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_qkv_kernel(const __grid_constant__ PfGemmParams p) {
   pdl_wait();
@@ -813,6 +839,7 @@ cudaError_t prefill_prepare() {
   if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<64>);
   if (e == cudaSuccess) e = prefer_shared(prefill_finish_resid_kernel);
   if (e == cudaSuccess) e = prefer_shared(prefill_finish_qkv_kernel);
+  if (e == cudaSuccess) e = prefer_shared(prefill_finish_store_kernel);
   if (e != cudaSuccess || g_pf_pairs > 0) return e;
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = pf_config(128, 1, nullptr, false, attr);
@@ -840,7 +867,7 @@ void plan_prefill_gemm(PfGemmParams& p, int num_sms) {
     p.sk_pairs = std::max(rem, std::min(P, rem * p.kc / PF_SK_MIN));
     if (p.sk_pairs == rem) p.sk_tiles = p.sk_pairs = 0;   // nothing to split
   }
-  p.publish = p.sk_tiles == T && (p.epi == EPI_RESID || p.epi == EPI_QKV);
+  p.publish = p.sk_tiles == T && p.epi != EPI_SWIGLU;
 }
 
 cudaError_t launch_prefill_gemm(const PfGemmParams& p, cudaStream_t st, bool pdl) {
@@ -852,14 +879,16 @@ cudaError_t launch_prefill_gemm(const PfGemmParams& p, cudaStream_t st, bool pdl
                                   : cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<128>, p);
   if (e != cudaSuccess || !p.publish) return e;
   cudaLaunchConfig_t fin = {};
-  fin.gridDim = p.epi == EPI_QKV ? dim3(p.M, 3) : dim3(p.M);
+  fin.gridDim = p.epi == EPI_RESID ? dim3(p.M)
+                                   : dim3(p.M, p.epi == EPI_QKV ? 3 : (p.N + 4 * PF_FIN_THREADS - 1) / (4 * PF_FIN_THREADS));
   fin.blockDim = dim3(PF_FIN_THREADS);
   fin.stream = st;
   attr[0] = attr[1];
   fin.attrs = attr;
   fin.numAttrs = pdl ? 1 : 0;
-  return p.epi == EPI_QKV ? cudaLaunchKernelEx(&fin, prefill_finish_qkv_kernel, p)
-                          : cudaLaunchKernelEx(&fin, prefill_finish_resid_kernel, p);
+  return p.epi == EPI_QKV     ? cudaLaunchKernelEx(&fin, prefill_finish_qkv_kernel, p)
+         : p.epi == EPI_RESID ? cudaLaunchKernelEx(&fin, prefill_finish_resid_kernel, p)
+                              : cudaLaunchKernelEx(&fin, prefill_finish_store_kernel, p);
 }
 
 }  // namespace sdsat
