@@ -1,8 +1,8 @@
 // Skinny-M weight-streaming GEMM on the 5th-generation tensor cores.
 //
 // Every projection of the block forward (QKV, O, gate/up, down, LM head) is
-// Y[M, N] = X[M, K] W[N, K]^T with M = b*q <= 64 rows and a weight matrix of
-// 30-330 MB.  The weights are read once per step, so the kernel is bound by
+// Y[M, N] = X[M, K] W[N, K]^T with M = b*q rows, up to 32 here (blocks of more rows than
+// GEMM_WIDE_ROWS run on the tiled GEMM of prefill.cu), and a weight matrix of 30-330 MB.  The weights are read once per step, so the kernel is bound by
 // HBM bandwidth (decoding is memory-bandwidth bound, Sec. 1; the loop time is
 // almost flat in k, Sec. 3.4.1).  Design:
 //
@@ -55,29 +55,21 @@ namespace sdsat {
 #ifndef SDSAT_GEMM_MINB
 #define SDSAT_GEMM_MINB 2
 #endif
-// Epilogue rows handled per group: a group's loads are all issued before its stores.
-#ifndef SDSAT_GEMM_EPI_GROUP
-#define SDSAT_GEMM_EPI_GROUP 16
-#endif
-constexpr int EG = SDSAT_GEMM_EPI_GROUP;
-
 template <int MPAD>
 struct GemmCfg {
-  static constexpr int STAGES = MPAD <= 16 ? SDSAT_GEMM_STAGES16 : 3;   // M <= 32: two CTAs per SM
+  static constexpr int STAGES = MPAD <= 16 ? SDSAT_GEMM_STAGES16 : 3;   // two CTAs per SM
   static constexpr int W_BYTES = 128 * 128;      // 128 rows x 64 bf16
   static constexpr int X_BYTES = MPAD * 128;     // MPAD rows x 64 bf16 (hi or lo)
   static constexpr int STAGE_BYTES = W_BYTES + 2 * X_BYTES;
   static constexpr int STAGING = 128 * (MPAD + 1) + 128;   // [128][MPAD+1] exchange + [PARTS][MPAD] sums
   static constexpr int ACC_COLS = 2 * MPAD;     // hi and lo products side by side
   // two accumulators (an allocation is a power of two, at least 32 columns)
-  static constexpr int TMEM_COLS = MPAD <= 8 ? 32 : (MPAD <= 16 ? 64 : (MPAD <= 32 ? 128 : 256));
+  static constexpr int TMEM_COLS = MPAD <= 8 ? 32 : (MPAD <= 16 ? 64 : 128);
   // parts of a tile's 128 rows that the sums of h^2 are first added up in
-  static constexpr int PARTS = MPAD <= 8 ? 16 : (MPAD <= 16 ? 8 : (MPAD <= 32 ? 4 : 2));
+  static constexpr int PARTS = MPAD <= 8 ? 16 : (MPAD <= 16 ? 8 : 4);
   static constexpr int NBAR = 2 * STAGES + 6;
   static constexpr int CS = MPAD * 64;           // EPI_QKV: RoPE (cos, sin) of every row and frequency
-  // residual rows loaded before the accumulator wait: every row up to 32 (MPAD 64 keeps
-  // the register budget with groups of EG)
-  static constexpr int EGR = MPAD <= 32 ? MPAD : EG;
+  static constexpr int EGR = MPAD;   // residual rows loaded before the accumulator wait: every row
   static constexpr size_t SMEM =
       1024 + (size_t)STAGES * STAGE_BYTES + STAGING * 4 + 2 * 64 * 4 + 64 * 8 + CS * 8 + NBAR * 8 + 128;
 };
@@ -609,13 +601,13 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
     trace_write(p.trace, (unsigned)s_mark[3], t_entry, t_wait, s_mark[0], s_mark[1], s_mark[2], globaltimer_ns());
 }
 
-// Rows are padded to a multiple of 8 up to 32 (16 is the smallest N of the MMA: 8 rows, hi and
-// lo), then to 64: the operand's padding costs L2 -> SM traffic, shared memory and epilogue time.
+// Rows are padded to a multiple of 8 (16 is the smallest N of the MMA: 8 rows, hi and lo): the
+// operand's padding costs L2 -> SM traffic, shared memory and epilogue time.
 // us per launch, 6 rows padded to 16 -> 8: QKV 21.6 -> 20.9, O 12.4 -> 11.4, gate/up 34.7 -> 33.4,
 // down 20.8 -> 19.6, LM head 46.5 -> 44.6; 24 rows, 32 -> 24: 24.7 -> 23.6, 16.3 -> 15.2, 39.5 -> 37.8,
 // 25.5 -> 24.1, 52.0 -> 49.9.  A fifth stage in the room that 8 rows leave was slower (386.9 against
-// 383.5 us for four layers and LM head); so were 48 rows with two CTAs per SM (gate/up 44.3 -> 47.4).
-int gemm_mpad(int M) { return M <= 32 ? (M + 7) / 8 * 8 : 64; }
+// 383.5 us for four layers and LM head).
+int gemm_mpad(int M) { return (M + 7) / 8 * 8; }
 
 namespace {
 template <typename F>
@@ -625,15 +617,14 @@ cudaError_t with_mpad(int mpad, F&& f) {   // f.operator()<MPAD>()
     case 16: return f.template operator()<16>();
     case 24: return f.template operator()<24>();
     case 32: return f.template operator()<32>();
-    default: return f.template operator()<64>();
+    default: return cudaErrorInvalidValue;
   }
 }
 struct PrepareGemm {
   template <int MPAD>
   cudaError_t operator()() const {
-    static_assert(GemmCfg<MPAD>::SMEM <= (MPAD <= 32 ? 115712 : 232448), "CTAs per SM");
-    // (MPAD 64 runs one CTA per SM and leaves no room for the next kernel's: it keeps its L1)
-    const cudaError_t e = MPAD <= 32 ? prefer_shared(gemm_kernel<MPAD>) : cudaSuccess;
+    static_assert(GemmCfg<MPAD>::SMEM <= 115712, "two CTAs per SM");
+    const cudaError_t e = prefer_shared(gemm_kernel<MPAD>);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(gemm_kernel<MPAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)GemmCfg<MPAD>::SMEM);
@@ -665,8 +656,7 @@ cudaError_t gemm_prepare() {
 constexpr int GEMM_WHOLE_KC = 16;
 static int gemm_grid(const GemmParams& p, int num_sms) {
   const long long T = (long long)p.n_tiles * p.kc;
-  const int per_sm = gemm_mpad(p.M) <= 32 ? GEMM_CTAS_PER_SM : 1;
-  const long long ctas = (long long)num_sms * per_sm;
+  const long long ctas = (long long)num_sms * GEMM_CTAS_PER_SM;
   if (p.kc <= GEMM_WHOLE_KC && p.n_tiles <= ctas) return p.n_tiles;
   return (int)std::min<long long>(ctas, T);
 }

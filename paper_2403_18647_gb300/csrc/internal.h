@@ -51,7 +51,7 @@ cudaError_t prefer_shared(K* kernel) {
 }
 
 // ---- skinny weight-streaming GEMM --------------------------------------------
-// CTAs per SM of the skinny GEMM's grid for M <= 32 (compile-time tuning; one beyond).
+// CTAs per SM of the skinny GEMM's grid (compile-time tuning).
 // Every user of the grid size (the split-K partials, the fixed scratch of the
 // scratch-free entry point) sizes its buffers from this constant.
 #ifndef SDSAT_GEMM_CTAS_PER_SM
@@ -118,8 +118,13 @@ struct GemmParams {
   Trace trace;
 };
 
-int gemm_mpad(int M);                 // rows of the operand boxes: 8, 16, 24, 32 or 64
-constexpr int GEMM_MPADS[] = {8, 16, 24, 32, 64};
+int gemm_mpad(int M);                 // rows of the operand boxes of M <= 32 rows: 8, 16, 24 or 32
+constexpr int GEMM_MPADS[] = {8, 16, 24, 32};
+// Blocks of more rows than this run on the tiled GEMM of prefill.cu (64-row tiles).  The skinny
+// GEMM's split-K tail grows with the rows: its last contributors summed 10 parts of 32 KB and
+// ran a 64-row epilogue in 13 us.  Four 7B layers and LM head, us per block step, skinny -> tiled:
+// 26 rows 481 -> 505, 30 rows 544 -> 533, 36 rows 576 -> 517, 64 rows 642 -> 527; 13B, 64 rows 857 -> 724.
+constexpr int GEMM_WIDE_ROWS = 28;
 cudaError_t gemm_prepare();           // set smem attributes (idempotent)
 cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 
@@ -190,7 +195,8 @@ struct PfGemmParams {
   float* partials;          // prefill_partials() floats: [pair][2][rank][128 positions][128 rows]
   int* counters;            // [2 * num_sms], zero between launches
   int epi;                  // EPI_STORE, EPI_RESID, EPI_QKV or EPI_SWIGLU
-  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID)
+  float* out;               // [M][out_ld] fp32 (EPI_STORE, EPI_RESID; optional: the rotated queries of EPI_QKV,
+                            // instead of hi + lo, and the activations of EPI_SWIGLU, beside them)
   int out_ld;
   __nv_bfloat16* out_hi;    // [M][out_ld] bf16 hi + lo: the next GEMM's operand (EPI_SWIGLU; EPI_RESID
                             // with gain_next), the rotated queries (EPI_QKV)
@@ -205,7 +211,9 @@ struct PfGemmParams {
   __nv_bfloat16* k_layer;   // this layer's caches [B][H][cap][hd]
   __nv_bfloat16* v_layer;
   const int* len;
-  int seq, H, hd, cap;
+  const int* positions;     // [M], or null: each row's cache slot
+  int seq0, q;              // row m belongs to sequence seq0 + m / q, slot len[that] + m % q
+  int H, hd, cap;
   const float2* rope;
   int rope_len;
   uint32_t* err;

@@ -133,26 +133,46 @@ __device__ __forceinline__ void pf_store4(__nv_bfloat16* hi, __nv_bfloat16* lo, 
                  pf_pack(c - __uint_as_float(h1 << 16), d - __uint_as_float(h1 & 0xFFFF0000u)));
 }
 
-// rotate-half RoPE of a head's dimensions i .. i + 3 (a) and i + hd/2 .. (b) at position `slot`
-__device__ __forceinline__ void pf_rope4(const PfGemmParams& p, int slot, int i, float4& a, float4& b) {
-  const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)min(slot, p.rope_len - 1) * (p.hd >> 1) + i);
+// sequence, cache slot and RoPE position of row m (len0: the length when all rows are of seq0)
+struct PfRow {
+  int seq, slot, pos;
+  __device__ PfRow(const PfGemmParams& p, int m, int len0) {
+    const int s = m < p.q ? 0 : m / p.q;
+    seq = p.seq0 + s;
+    slot = (p.q >= p.M ? len0 : __ldcg(p.len + seq)) + m - s * p.q;
+    pos = p.positions ? __ldcg(p.positions + m) : slot;
+  }
+  __device__ void report(const PfGemmParams& p) const {   // (by one thread of a row)
+    if (slot >= p.cap) set_error(p.err, ERR_CAPACITY);
+    if (pos < 0 || pos >= p.rope_len) set_error(p.err, ERR_POSITION);
+  }
+};
+// rotate-half RoPE of a head's dimensions i .. i + 3 (a) and i + hd/2 .. (b)
+__device__ __forceinline__ void pf_rope4(const PfGemmParams& p, int pos, int i, float4& a, float4& b) {
+  const float4* cs =
+      reinterpret_cast<const float4*>(p.rope + (size_t)min(max(pos, 0), p.rope_len - 1) * (p.hd >> 1) + i);
   const float4 t0 = __ldg(cs), t1 = __ldg(cs + 1);   // cos, sin of two frequencies each
   const float4 o = a;
   a = make_float4(a.x * t0.x - b.x * t0.y, a.y * t0.z - b.y * t0.w, a.z * t1.x - b.z * t1.y, a.w * t1.z - b.w * t1.w);
   b = make_float4(b.x * t0.x + o.x * t0.y, b.y * t0.z + o.y * t0.w, b.z * t1.x + o.z * t1.y, b.w * t1.z + o.w * t1.w);
 }
-// features f .. f + 3 (a) and f + hd/2 .. (b) of chunk position m: q as bf16 hi + lo, k and v into
-// the cache slot when there is one
-__device__ __forceinline__ void pf_qkv_store(const PfGemmParams& p, int which, int m, int slot, int f, int i,
+// features f .. f + 3 (a) and f + hd/2 .. (b) of row m: q in fp32 or as bf16 hi + lo, k and v into
+// the row's cache slot when there is one
+__device__ __forceinline__ void pf_qkv_store(const PfGemmParams& p, int which, int m, const PfRow& r, int f, int i,
                                              const float4& a, const float4& b) {
   const int half = p.hd >> 1;
   if (which == 0) {
     const size_t o = (size_t)m * p.out_ld + f;
-    pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
-    pf_store4(p.out_hi, p.out_lo, o + half, b.x, b.y, b.z, b.w);
-  } else if (slot < p.cap) {
+    if (p.out) {
+      *reinterpret_cast<float4*>(p.out + o) = a;
+      *reinterpret_cast<float4*>(p.out + o + half) = b;
+    } else {
+      pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
+      pf_store4(p.out_hi, p.out_lo, o + half, b.x, b.y, b.z, b.w);
+    }
+  } else if (r.slot < p.cap) {
     __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) +
-                         ((size_t)(p.seq * p.H + (f - i) / p.hd) * p.cap + slot) * p.hd + i;
+                         ((size_t)(r.seq * p.H + (f - i) / p.hd) * p.cap + r.slot) * p.hd + i;
     *reinterpret_cast<uint2*>(dst) = make_uint2(pf_pack(a.x, a.y), pf_pack(a.z, a.w));
     *reinterpret_cast<uint2*>(dst + half) = make_uint2(pf_pack(b.x, b.y), pf_pack(b.z, b.w));
   }
@@ -352,7 +372,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     uint32_t res_ph = 0;
     pdl_wait();   // residual rows and outputs belong to the previous kernels' results
     if (p.trace.rec) t_wait = globaltimer_ns();
-    const int len0 = p.epi == EPI_QKV ? __ldcg(p.len + p.seq) : 0;
+    const int len0 = p.epi == EPI_QKV ? __ldcg(p.len + p.seq0) : 0;
     int seg = 0;
     PfWalk w(p, pair);
     for (; w.next(); ++seg) {
@@ -574,9 +594,12 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             const float4 g = *reinterpret_cast<const float4*>(row), u = *reinterpret_cast<const float4*>(row + 64);
             const float s = p.ssq_in ? inv[c0 + w8 + k] : 1.f;
             auto act = [&](float x, float up) { return x * s / (1.0f + expf(-(x * s))) * (up * s); };
-            if (wt < p.n_wtiles && f < p.N)
-              pf_store4(p.out_hi, p.out_lo, (size_t)(m0 + w8 + k) * p.out_ld + f, act(g.x, u.x), act(g.y, u.y),
-                        act(g.z, u.z), act(g.w, u.w));
+            if (wt < p.n_wtiles && f < p.N) {
+              const size_t o = (size_t)(m0 + w8 + k) * p.out_ld + f;
+              const float4 a = make_float4(act(g.x, u.x), act(g.y, u.y), act(g.z, u.z), act(g.w, u.w));
+              if (p.out) *reinterpret_cast<float4*>(p.out + o) = a;
+              pf_store4(p.out_hi, p.out_lo, o, a.x, a.y, a.z, a.w);
+            }
           }
         } else if (p.epi == EPI_QKV) {
           // The tile lies in one of q, k, v and holds whole heads.  RoPE (rotate-half) pairs row
@@ -593,11 +616,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
               float4 a = *reinterpret_cast<const float4*>(row), b = *reinterpret_cast<const float4*>(row + half);
               const float s = p.ssq_in ? inv[c0 + w8 + k] : 1.f;
               a.x *= s, a.y *= s, a.z *= s, a.w *= s, b.x *= s, b.y *= s, b.z *= s, b.w *= s;
-              const int m = m0 + w8 + k, slot = len0 + m;
-              if (which < 2) pf_rope4(p, slot, i, a, b);
-              pf_qkv_store(p, which, m, slot, f, i, a, b);
-              if (slot >= p.cap && which && (lane & 15) == 0) set_error(p.err, ERR_CAPACITY);
-              if (slot >= p.rope_len && which && (lane & 15) == 0) set_error(p.err, ERR_POSITION);
+              const int m = m0 + w8 + k;
+              const PfRow row_of(p, m, len0);
+              if (which < 2) pf_rope4(p, row_of.pos, i, a, b);
+              pf_qkv_store(p, which, m, row_of, f, i, a, b);
+              if (which == 1 && (lane & 15) == 0) row_of.report(p);
             }
           }
         } else {
@@ -775,17 +798,15 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_qkv_kernel(cons
   pdl_wait();
   pdl_trigger();
   const int m = blockIdx.x, which = blockIdx.y, tok = p.tok, tb = m / tok, pos = m - tb * tok;
-  const int R = p.rows_per_map, half = p.hd >> 1, slot = __ldcg(p.len + p.seq) + m;
+  const int R = p.rows_per_map, half = p.hd >> 1;
+  const PfRow row_of(p, m, __ldcg(p.len + p.seq0));
   float s = 1.f;
   if (p.ssq_in) {
     float q = 0.f;
     for (int t = 0; t < p.ssq_ld; ++t) q += __ldcg(p.ssq_in + (size_t)m * p.ssq_ld + t);
     s = 1.0f / sqrtf(q / (float)p.norm_dim + p.norm_eps);
   }
-  if (threadIdx.x == 0 && which == 1) {
-    if (slot >= p.cap) set_error(p.err, ERR_CAPACITY);
-    if (slot >= p.rope_len) set_error(p.err, ERR_POSITION);
-  }
+  if (threadIdx.x == 0 && which == 1) row_of.report(p);
   for (int x = 4 * (int)threadIdx.x; x < R / 2; x += 4 * PF_FIN_THREADS) {
     // four pairs of features: i .. i + 3 of a head and those half a head further
     const int i = x & (half - 1), f = (x - i) * 2 + i;   // head * hd + i
@@ -805,8 +826,8 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_qkv_kernel(cons
       for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(a, t[u]), pf_add(b, u4[u]);
     }
     a.x *= s, a.y *= s, a.z *= s, a.w *= s, b.x *= s, b.y *= s, b.z *= s, b.w *= s;
-    if (which < 2) pf_rope4(p, slot, i, a, b);
-    pf_qkv_store(p, which, m, slot, f, i, a, b);
+    if (which < 2) pf_rope4(p, row_of.pos, i, a, b);
+    pf_qkv_store(p, which, m, row_of, f, i, a, b);
   }
 }
 

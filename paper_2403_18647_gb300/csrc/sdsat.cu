@@ -97,6 +97,7 @@ const char* const KCLASS_NAME[K_COUNT] = {"rmsnorm", "gemm_qkv", "attention", "g
                                           "gemm_op", "attention_op", "tree_prep", "tree_compact", "prefill_gemm",
                                           "prefill_attention"};
 
+static_assert(SDSAT_MAX_ROWS == 64, "block rows fill one 64-row tile of the prefill GEMM");
 constexpr int MAX_GEMM_TILES = 1 << 16;
 constexpr int OP_MAX_K = 32768;   // limits of sdsat_op_gemm (its operand scratch is sized at create)
 constexpr int OP_MAX_M = 512;
@@ -145,6 +146,7 @@ struct sdsat_ctx {
   __nv_bfloat16* x_hi[X_COUNT] = {};
   __nv_bfloat16* x_lo[X_COUNT] = {};
   CUtensorMap xmap[X_COUNT][N_MPADS][2];   // [source][GEMM_MPADS][hi/lo]
+  CUtensorMap xmap_wide[X_COUNT][2];       // boxes of 64 rows
   __nv_bfloat16* xop_hi = nullptr;     // operand scratch of sdsat_op_gemm
   __nv_bfloat16* xop_lo = nullptr;
   std::vector<void*> allocs;
@@ -250,6 +252,149 @@ void set_plain(GemmParams& g, const CUtensorMap& m, int N, int K) {
   g.kc = (K + 63) / 64;
 }
 
+// The decoder layers on the prefill GEMM: a chunk of a prompt, or a block of more rows than the
+// decode GEMM is good for.
+struct Tiled {
+  int M, seq0, q;              // row m: sequence seq0 + m / q, slot len[that] + m % q
+  const int32_t* positions;    // RoPE positions, or null: the slots
+  float* h;                    // [M][d] residual stream
+  float* ssq;                  // [M][ssq_ld]
+  __nv_bfloat16 *const *hi, *const *lo;   // operands by XSrc
+  const CUtensorMap* xmap[X_COUNT];       // their maps, hi and lo, boxes of prefill_tok(M) rows
+  float *qout, *act;           // fp32 queries (null: hi + lo below) and activations (optional)
+  __nv_bfloat16 *qhi, *qlo;
+  bool prefill;                // profiling class; no logits
+};
+
+// attention(l): the layer's attention, from the queries to the O projection's operand
+template <typename A>
+sdsat_status tiled_layers(sdsat_ctx* c, sdsat_kv* kv, const Tiled& t, const int32_t* tokens, float* logits,
+                          A&& attention) {
+  const sdsat_config& cf = c->cfg;
+  const int M = t.M, d = cf.d_model, H = cf.n_heads, hd = cf.head_dim, F = cf.ffn_dim, R = H * hd, L = cf.n_layers;
+  cudaStream_t st = c->stream;
+  const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
+  // RMSNorm folded into the GEMMs as in forward(): O and down emit the next operand and the
+  // sums of squares, gate/up and the next QKV scale by the factor (unless O or down ended in a
+  // kernel of its own, which normalises)
+  auto fold_in = [&](PfGemmParams& g) {
+    g.ssq_in = t.ssq;
+    g.ssq_ld = c->ssq_ld;
+    g.norm_dim = d;
+    g.norm_eps = cf.rms_eps;
+  };
+  auto fold_out = [&](PfGemmParams& g, const void* gain) {
+    g.gain_next = static_cast<const __nv_bfloat16*>(gain);
+    g.out_hi = t.hi[X_NORM];
+    g.out_lo = t.lo[X_NORM];
+    g.ssq_out = t.ssq;
+    g.ssq_ld = c->ssq_ld;
+    g.norm_dim = d;
+    g.norm_eps = cf.rms_eps;
+  };
+  auto base = [&](int xsrc, int K) {
+    PfGemmParams g;
+    std::memset(&g, 0, sizeof(g));
+    g.tmap_x[0] = t.xmap[xsrc][0];
+    g.tmap_x[1] = t.xmap[xsrc][1];
+    g.kc = (K + 63) / 64;
+    g.M = M;
+    g.partials = c->partials;
+    g.counters = c->gemm_counters;
+    g.err = c->err;
+    return g;
+  };
+  bool normed = true;   // the next GEMM's operand is already normalised (else h * g)
+  auto gemm = [&](PfGemmParams& g, int cls) {
+    plan_prefill_gemm(g, c->num_sms);
+    if (g.epi == EPI_RESID) normed = g.publish;
+    if (t.prefill) cls = K_PF_GEMM;
+    g.trace = next_trace(c, cls);
+    return timed(c, cls, [&] { return launch_prefill_gemm(g, st, c->pdl); });
+  };
+  if (timed(c, K_RMSNORM, [&] {
+        return launch_rmsnorm(tokens, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, t.h, d, M,
+                              static_cast<const __nv_bfloat16*>(c->layers[0].attn_norm), cf.rms_eps,
+                              t.hi[X_NORM], t.lo[X_NORM], c->err, st, c->pdl);
+      }) != cudaSuccess)
+    return SDSAT_ECUDA;
+  for (int l = 0; l < L; ++l) {
+    const LayerMaps& mp = c->maps[l];
+    PfGemmParams gq = base(X_NORM, d);
+    gq.tmap[0] = mp.q;
+    gq.tmap[1] = mp.k;
+    gq.tmap[2] = mp.v;
+    gq.map_mode = MAP_QKV3;
+    gq.rows_per_map = R;
+    gq.N = 3 * R;
+    gq.n_wtiles = 3 * R / 128;
+    gq.epi = EPI_QKV;
+    gq.out = t.qout;
+    gq.out_hi = t.qhi;
+    gq.out_lo = t.qlo;
+    gq.out_ld = R;
+    gq.k_layer = kv->k + l * layer_elems;
+    gq.v_layer = kv->v + l * layer_elems;
+    gq.len = kv->len;
+    gq.positions = t.positions;
+    gq.seq0 = t.seq0;
+    gq.q = t.q;
+    gq.H = H;
+    gq.hd = hd;
+    gq.cap = kv->cap;
+    gq.rope = c->rope;
+    gq.rope_len = cf.max_position;
+    if (!normed) fold_in(gq);
+    if (gemm(gq, K_GEMM_QKV) != cudaSuccess) return SDSAT_ECUDA;
+    if (attention(l) != cudaSuccess) return SDSAT_ECUDA;
+    PfGemmParams go = base(X_ATTN, R);
+    go.tmap[0] = mp.o;
+    go.map_mode = MAP_PLAIN;
+    go.N = d;
+    go.n_wtiles = (d + 127) / 128;
+    go.epi = EPI_RESID;
+    go.out = t.h;
+    go.out_ld = d;
+    fold_out(go, c->layers[l].ffn_norm);
+    if (gemm(go, K_GEMM_O) != cudaSuccess) return SDSAT_ECUDA;
+    PfGemmParams gg = base(X_NORM, d);
+    gg.tmap[0] = mp.gate;
+    gg.tmap[1] = mp.up;
+    gg.map_mode = MAP_GATEUP;
+    gg.N = F;
+    gg.n_wtiles = (F + 63) / 64;
+    gg.epi = EPI_SWIGLU;
+    gg.out = t.act;
+    gg.out_hi = t.hi[X_FFN];
+    gg.out_lo = t.lo[X_FFN];
+    gg.out_ld = F;
+    if (!normed) fold_in(gg);
+    if (gemm(gg, K_GEMM_GATEUP) != cudaSuccess) return SDSAT_ECUDA;
+    PfGemmParams gd = base(X_FFN, F);
+    gd.tmap[0] = mp.down;
+    gd.map_mode = MAP_PLAIN;
+    gd.N = d;
+    gd.n_wtiles = (d + 127) / 128;
+    gd.epi = EPI_RESID;
+    gd.out = t.h;
+    gd.out_ld = d;
+    if (l + 1 < L) fold_out(gd, c->layers[l + 1].attn_norm);
+    else if (logits) fold_out(gd, c->w.final_norm);
+    if (gemm(gd, K_GEMM_DOWN) != cudaSuccess) return SDSAT_ECUDA;
+  }
+  if (!logits) return SDSAT_OK;
+  PfGemmParams gh = base(X_NORM, d);
+  gh.tmap[0] = c->head_map;
+  gh.map_mode = MAP_PLAIN;
+  gh.N = cf.vocab;
+  gh.n_wtiles = (cf.vocab + 127) / 128;
+  gh.epi = EPI_STORE;
+  gh.out = logits;
+  gh.out_ld = cf.vocab;
+  if (!normed) fold_in(gh);
+  return gemm(gh, K_GEMM_LM_HEAD) == cudaSuccess ? SDSAT_OK : SDSAT_ECUDA;
+}
+
 // one block forward of sequences seq0 .. seq0+nb-1, q rows each (anc: tree attention masks)
 sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const int32_t* tokens,
                      const int32_t* positions, float* logits, const uint32_t* anc = nullptr) {
@@ -257,6 +402,46 @@ sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const 
   const int M = nb * q, d = cf.d_model, H = cf.n_heads, hd = cf.head_dim, F = cf.ffn_dim, R = H * hd, L = cf.n_layers;
   cudaStream_t st = c->stream;
   const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
+  auto attention = [&](int l) {
+    // block-causal attention; its merge emits the O projection's operand
+    AttnParams a;
+    std::memset(&a, 0, sizeof(a));
+    a.kmap = kv->kmap;
+    a.vmap = kv->vmap;
+    a.row0 = l * kv->batch * H * kv->cap;
+    a.Q = c->qbuf;
+    a.q_ld = R;
+    a.len = kv->len;
+    a.anc = anc;
+    a.seq0 = seq0;
+    a.nb = nb;
+    a.q = q;
+    a.H = H;
+    a.hd = hd;
+    a.cap = kv->cap;
+    a.out = c->attn;
+    a.out_ld = R;
+    a.out_hi = c->x_hi[X_ATTN];
+    a.out_lo = c->x_lo[X_ATTN];
+    a.err = c->err;
+    a.trace = next_trace(c, K_ATTENTION);
+    return timed(c, K_ATTENTION, [&] { return launch_attention(a, c->num_sms, st, c->pdl); });
+  };
+  if (M > GEMM_WIDE_ROWS) {
+    Tiled t{};
+    t.M = M;
+    t.seq0 = seq0;
+    t.q = q;
+    t.positions = positions;
+    t.h = c->h;
+    t.ssq = c->ssq;
+    t.hi = c->x_hi;
+    t.lo = c->x_lo;
+    for (int xs = 0; xs < X_COUNT; ++xs) t.xmap[xs] = c->xmap_wide[xs];
+    t.qout = c->qbuf;
+    t.act = c->act;
+    return tiled_layers(c, kv, t, tokens, logits, attention);
+  }
   auto norm = [&](const int32_t* toks, const void* gain) {
     return timed(c, K_RMSNORM, [&] {
       return launch_rmsnorm(toks, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->h, d, M,
@@ -371,30 +556,7 @@ sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const 
     if (l + 1 < L) gn = make_qkv(l + 1);
     else if (logits) gn = make_head();
     if (gemm(gq, K_GEMM_QKV) != cudaSuccess) return SDSAT_ECUDA;
-    // block-causal attention; its merge emits the O projection's operand
-    AttnParams a;
-    std::memset(&a, 0, sizeof(a));
-    a.kmap = kv->kmap;
-    a.vmap = kv->vmap;
-    a.row0 = l * kv->batch * H * kv->cap;
-    a.Q = c->qbuf;
-    a.q_ld = R;
-    a.len = kv->len;
-    a.anc = anc;
-    a.seq0 = seq0;
-    a.nb = nb;
-    a.q = q;
-    a.H = H;
-    a.hd = hd;
-    a.cap = kv->cap;
-    a.out = c->attn;
-    a.out_ld = R;
-    a.out_hi = c->x_hi[X_ATTN];
-    a.out_lo = c->x_lo[X_ATTN];
-    a.err = c->err;
-    a.trace = next_trace(c, K_ATTENTION);
-    if (timed(c, K_ATTENTION, [&] { return launch_attention(a, c->num_sms, st, c->pdl); }) != cudaSuccess)
-      return SDSAT_ECUDA;
+    if (attention(l) != cudaSuccess) return SDSAT_ECUDA;
     if (gemm(go, K_GEMM_O) != cudaSuccess || gemm(gg, K_GEMM_GATEUP) != cudaSuccess ||
         gemm(gd, K_GEMM_DOWN) != cudaSuccess)
       return SDSAT_ECUDA;
@@ -404,82 +566,23 @@ sdsat_status forward(sdsat_ctx* c, sdsat_kv* kv, int seq0, int nb, int q, const 
   return SDSAT_OK;
 }
 
-// one prefill chunk: M <= pf_rows prompt positions of sequence seq
-// through every layer on the tiled GEMM, then committed
+// one prefill chunk: M <= pf_rows prompt positions of sequence seq through every layer, then
+// committed
 sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* tokens, int M) {
   const sdsat_config& cf = c->cfg;
-  const int d = cf.d_model, H = cf.n_heads, hd = cf.head_dim, F = cf.ffn_dim, R = H * hd, L = cf.n_layers;
-  cudaStream_t st = c->stream;
-  const size_t layer_elems = (size_t)kv->batch * H * kv->cap * hd;
-  const int xi = prefill_tok(M) == 64;
-  // RMSNorm folded into the GEMMs as in forward(): O and down emit the next operand and the
-  // sums of squares, gate/up and the next QKV scale by the factor (unless O or down ended in a
-  // kernel of its own, which normalises)
-  auto fold_in = [&](PfGemmParams& g) {
-    g.ssq_in = c->pf_ssq;
-    g.ssq_ld = c->ssq_ld;
-    g.norm_dim = d;
-    g.norm_eps = cf.rms_eps;
-  };
-  auto fold_out = [&](PfGemmParams& g, const void* gain) {
-    g.gain_next = static_cast<const __nv_bfloat16*>(gain);
-    g.out_hi = c->pf_hi[X_NORM];
-    g.out_lo = c->pf_lo[X_NORM];
-    g.ssq_out = c->pf_ssq;
-    g.ssq_ld = c->ssq_ld;
-    g.norm_dim = d;
-    g.norm_eps = cf.rms_eps;
-  };
-  auto base = [&](int xsrc, int K) {
-    PfGemmParams g;
-    std::memset(&g, 0, sizeof(g));
-    g.tmap_x[0] = c->pf_xmap[xi][xsrc][0];
-    g.tmap_x[1] = c->pf_xmap[xi][xsrc][1];
-    g.kc = (K + 63) / 64;
-    g.M = M;
-    g.partials = c->partials;
-    g.counters = c->gemm_counters;
-    g.err = c->err;
-    return g;
-  };
-  bool normed = true;   // the next GEMM's operand is already normalised (else h * g)
-  auto gemm = [&](PfGemmParams& g) {
-    plan_prefill_gemm(g, c->num_sms);
-    if (g.epi == EPI_RESID) normed = g.publish;
-    g.trace = next_trace(c, K_PF_GEMM);
-    return timed(c, K_PF_GEMM, [&] { return launch_prefill_gemm(g, st, c->pdl); });
-  };
-  if (timed(c, K_RMSNORM, [&] {
-        return launch_rmsnorm(tokens, static_cast<const __nv_bfloat16*>(c->w.embed), cf.vocab, c->pf_h, d, M,
-                              static_cast<const __nv_bfloat16*>(c->layers[0].attn_norm), cf.rms_eps,
-                              c->pf_hi[X_NORM], c->pf_lo[X_NORM], c->err, st, c->pdl);
-      }) != cudaSuccess)
-    return SDSAT_ECUDA;
-  for (int l = 0; l < L; ++l) {
-    const LayerMaps& mp = c->maps[l];
-    PfGemmParams gq = base(X_NORM, d);
-    gq.tmap[0] = mp.q;
-    gq.tmap[1] = mp.k;
-    gq.tmap[2] = mp.v;
-    gq.map_mode = MAP_QKV3;
-    gq.rows_per_map = R;
-    gq.N = 3 * R;
-    gq.n_wtiles = 3 * R / 128;
-    gq.epi = EPI_QKV;
-    gq.out_hi = c->pf_qhi;
-    gq.out_lo = c->pf_qlo;
-    gq.out_ld = R;
-    gq.k_layer = kv->k + l * layer_elems;
-    gq.v_layer = kv->v + l * layer_elems;
-    gq.len = kv->len;
-    gq.seq = seq;
-    gq.H = H;
-    gq.hd = hd;
-    gq.cap = kv->cap;
-    gq.rope = c->rope;
-    gq.rope_len = cf.max_position;
-    if (!normed) fold_in(gq);
-    if (gemm(gq) != cudaSuccess) return SDSAT_ECUDA;
+  const int H = cf.n_heads, hd = cf.head_dim, R = H * hd, xi = prefill_tok(M) == 64;
+  Tiled t{};
+  t.M = t.q = M;
+  t.seq0 = seq;
+  t.h = c->pf_h;
+  t.ssq = c->pf_ssq;
+  t.hi = c->pf_hi;
+  t.lo = c->pf_lo;
+  for (int xs = 0; xs < X_COUNT; ++xs) t.xmap[xs] = c->pf_xmap[xi][xs];
+  t.qhi = c->pf_qhi;
+  t.qlo = c->pf_qlo;
+  t.prefill = true;
+  const sdsat_status s = tiled_layers(c, kv, t, tokens, nullptr, [&](int l) {
     // causal attention of the chunk's positions over the cache
     PfAttnParams a;
     std::memset(&a, 0, sizeof(a));
@@ -498,43 +601,11 @@ sdsat_status prefill_chunk(sdsat_ctx* c, sdsat_kv* kv, int seq, const int32_t* t
     a.out_hi = c->pf_hi[X_ATTN];
     a.out_lo = c->pf_lo[X_ATTN];
     a.err = c->err;
-    if (timed(c, K_PF_ATTENTION, [&] { return launch_prefill_attention(a, c->num_sms, st, c->pdl); }) != cudaSuccess)
-      return SDSAT_ECUDA;
-    PfGemmParams go = base(X_ATTN, R);
-    go.tmap[0] = mp.o;
-    go.map_mode = MAP_PLAIN;
-    go.N = d;
-    go.n_wtiles = (d + 127) / 128;
-    go.epi = EPI_RESID;
-    go.out = c->pf_h;
-    go.out_ld = d;
-    fold_out(go, c->layers[l].ffn_norm);
-    if (gemm(go) != cudaSuccess) return SDSAT_ECUDA;
-    PfGemmParams gg = base(X_NORM, d);
-    gg.tmap[0] = mp.gate;
-    gg.tmap[1] = mp.up;
-    gg.map_mode = MAP_GATEUP;
-    gg.N = F;
-    gg.n_wtiles = (F + 63) / 64;
-    gg.epi = EPI_SWIGLU;
-    gg.out_hi = c->pf_hi[X_FFN];
-    gg.out_lo = c->pf_lo[X_FFN];
-    gg.out_ld = F;
-    if (!normed) fold_in(gg);
-    if (gemm(gg) != cudaSuccess) return SDSAT_ECUDA;
-    PfGemmParams gd = base(X_FFN, F);
-    gd.tmap[0] = mp.down;
-    gd.map_mode = MAP_PLAIN;
-    gd.N = d;
-    gd.n_wtiles = (d + 127) / 128;
-    gd.epi = EPI_RESID;
-    gd.out = c->pf_h;
-    gd.out_ld = d;
-    if (l + 1 < L) fold_out(gd, c->layers[l + 1].attn_norm);
-    if (gemm(gd) != cudaSuccess) return SDSAT_ECUDA;
-  }
-  return timed(c, K_PREFILL_COMMIT, [&] { return launch_add_len(kv->len, seq, M, kv->cap, c->err, st, c->pdl); }) ==
-                 cudaSuccess
+    return timed(c, K_PF_ATTENTION, [&] { return launch_prefill_attention(a, c->num_sms, c->stream, c->pdl); });
+  });
+  if (s != SDSAT_OK) return s;
+  return timed(c, K_PREFILL_COMMIT,
+               [&] { return launch_add_len(kv->len, seq, M, kv->cap, c->err, c->stream, c->pdl); }) == cudaSuccess
              ? SDSAT_OK
              : SDSAT_ECUDA;
 }
@@ -678,7 +749,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
   bool ok = dalloc(c, &c->rope, rope.size()) && dalloc(c, &c->h, (size_t)rows * d) &&
             dalloc(c, &c->qbuf, (size_t)rows * R) && dalloc(c, &c->attn, (size_t)rows * R) &&
             dalloc(c, &c->act, (size_t)rows * F) &&
-            dalloc(c, &c->partials, std::max((size_t)c->num_sms * 2 * 2 * 64 * 128, prefill_partials(c->num_sms))) &&
+            dalloc(c, &c->partials,
+                   std::max((size_t)c->num_sms * GEMM_CTAS_PER_SM * 2 * 32 * 128, prefill_partials(c->num_sms))) &&
             dalloc(c, &c->gemm_counters, MAX_GEMM_TILES) &&
             dalloc(c, &c->acc_targets, rows) &&
             dalloc(c, &c->acc_counters, rows) && dalloc(c, &c->adaptive, SDSAT_MAX_ADAPTIVE) &&
@@ -693,6 +765,8 @@ sdsat_status sdsat_create(const sdsat_config* cfg, const sdsat_weights* w, void*
     for (int mi = 0; ok && mi < N_MPADS; ++mi)
       ok = make_xmap(&c->xmap[xs][mi][0], c->x_hi[xs], rows, xcols[xs], GEMM_MPADS[mi]) &&
            make_xmap(&c->xmap[xs][mi][1], c->x_lo[xs], rows, xcols[xs], GEMM_MPADS[mi]);
+    ok = ok && make_xmap(&c->xmap_wide[xs][0], c->x_hi[xs], rows, xcols[xs], 64) &&
+         make_xmap(&c->xmap_wide[xs][1], c->x_lo[xs], rows, xcols[xs], 64);
   }
   if (ok && c->has_weights) {
     // the prefill workspaces in one allocation; a prompt is no longer than max_position
@@ -1108,7 +1182,7 @@ sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const
   if (!c || !x_dev || !y_dev || !aligned16(w_dev) || !aligned16(x_dev)) return SDSAT_EINVAL;
   if (M < 1 || M > OP_MAX_M || K < 8 || K % 8 || K > OP_MAX_K || N < 1 || (N + 127) / 128 > MAX_GEMM_TILES)
     return SDSAT_EINVAL;
-  if (M > SDSAT_MAX_ROWS) {
+  if (M > GEMM_WIDE_ROWS) {
     // the prefill GEMM (tiles of 128 weight rows x 128 positions)
     const int rows = (M + 127) / 128 * 128;   // <= OP_MAX_M rows of the operand scratch
     PfGemmParams g;

@@ -1,6 +1,6 @@
-"""Block forwards whose row count lies at the edges of the decode GEMM's operand padding (8, 16,
-24, 32 and 64 rows): every sequence of a batch against the same sequence alone, logits and
-the K / V rows written."""
+"""Block forwards whose row count lies at the edges of the GEMMs they run on (operand padding to
+8, 16, 24 and 32 rows, and from 29 rows the tiled GEMM): every sequence of a batch against the
+same sequence alone: logits, the last layer's workspaces and the K / V rows written."""
 import pytest
 import torch
 
@@ -26,26 +26,61 @@ def _filled(ctx, b, lens, seqs):
     return kv
 
 
-@pytest.mark.parametrize("b,q", [(1, 7), (1, 8), (1, 9), (2, 8), (1, 16), (3, 8), (5, 5), (2, 16), (3, 11), (3, 16),
+@pytest.mark.parametrize("b,q", [(1, 7), (1, 8), (1, 9), (2, 8), (1, 16), (3, 8), (5, 5), (4, 7), (5, 6), (2, 16), (3, 11), (3, 16),
                                  (7, 7), (4, 16)])
 def test_batch_equals_single_sequences(ctx, b, q):
     shape, lens = ctx.shape, [60 + 17 * s for s in range(b)]
     toks = synth.uniform_ids(3, b * 16 + q, b * q, shape.vocab, device="cuda")
     kv, lg = _filled(ctx, b, lens, range(b)), torch.full((b * q, shape.vocab), float("nan"), device="cuda")
     ctx.block_forward(kv, toks, lg, b, q)
+    ws = [ctx.debug_workspace(i, b * q) for i in range(4)]
     for s in range(b):
         one, l1 = _filled(ctx, 1, lens, [s]), torch.empty(q, shape.vocab, device="cuda")
         ctx.block_forward(one, toks[s * q:(s + 1) * q].contiguous(), l1, 1, q)
         got = lg[s * q:(s + 1) * q]
         # the same operands in fp32 sums of another order; a cached row's bf16 rounding may flip
         assert ((got - l1).norm() / l1.norm()).item() <= 2e-3
+        for i in range(4):
+            x, y = ws[i][s * q:(s + 1) * q], ctx.debug_workspace(i, q)
+            assert ((x - y).norm() / y.norm()).item() <= 2e-3, i
         for l in range(shape.n_layers):
             for x, y in zip(ctx.kv_read(kv, l, s, lens[s], q), ctx.kv_read(one, l, 0, lens[s], q)):
                 assert (x.float() - y.float()).abs().max().item() <= 1e-2 * y.float().abs().max().item()
     assert ctx.get_error() == 0
 
 
-@pytest.mark.parametrize("M", [1, 8, 9, 16, 17, 24, 25, 32, 33, 48, 49, 64])
+@pytest.mark.parametrize("b,q", [(2, 11), (3, 11), (4, 15)])
+def test_tree_batch_equals_single_sequences(ctx, b, q):
+    """Tree blocks: positions and masks follow the parents on either GEMM."""
+    shape, lens = ctx.shape, [60 + 17 * s for s in range(b)]
+    parent = [-1, 0, 1, 2, 0, 4, 4, 1, 7, 0, 9, 10, 10, 3, 13][:q]
+    toks = synth.uniform_ids(4, b * 16 + q, b * q, shape.vocab, device="cuda")
+    par = torch.tensor(parent * b, dtype=torch.int32, device="cuda")
+    kv, lg = _filled(ctx, b, lens, range(b)), torch.full((b * q, shape.vocab), float("nan"), device="cuda")
+    ctx.block_forward_tree(kv, toks, par, lg, b, q)
+    for s in range(b):
+        one, l1 = _filled(ctx, 1, lens, [s]), torch.empty(q, shape.vocab, device="cuda")
+        ctx.block_forward_tree(one, toks[s * q:(s + 1) * q].contiguous(), par[:q].contiguous(), l1, 1, q)
+        assert ((lg[s * q:(s + 1) * q] - l1).norm() / l1.norm()).item() <= 2e-3
+    assert ctx.get_error() == 0
+
+
+def test_wide_block_past_the_capacity(ctx):
+    """Rows past the KV capacity on the tiled GEMM: flagged, not written, the others as usual."""
+    b, q = 2, 16
+    kv = ctx.kv(b, 100)
+    ctx.kv_commit(kv, torch.tensor([100 - q, 100 - 5], dtype=torch.int32, device="cuda"), b)
+    toks = synth.uniform_ids(5, 1, b * q, ctx.shape.vocab, device="cuda")
+    lg = torch.empty(b * q, ctx.shape.vocab, device="cuda")
+    ctx.block_forward(kv, toks, lg, b, q)
+    assert ctx.get_error() == 0x4
+    k, _ = ctx.kv_read(kv, 0, 0, 100 - q, q)
+    assert (k.float().abs().sum(dim=(0, 2)) > 0).all()
+    k, _ = ctx.kv_read(kv, 0, 1, 0, 100)
+    assert (k.float().abs().sum(dim=(0, 2))[:95] == 0).all() and (k.float().abs().sum(dim=(0, 2))[95:] > 0).all()
+
+
+@pytest.mark.parametrize("M", [1, 8, 9, 16, 17, 24, 25, 28, 29, 32, 33, 64])
 def test_gemm_row_padding(ctx, M):
     K, N = 4096, 1500   # split tiles, ragged N
     x, w = synth.normal_f32(12, M, (M, K), 1.0, device="cuda"), synth.normal_bf16(12, 1, (N, K), 0.02, device="cuda")
