@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
     const int e = warp & 3;   // TMEM lane quarter this warp may access (warps 2-5 -> 2, 3, 0, 1)
     const int r = e * 32 + lane;
     pdl_wait();
-    if (p.ssq_in) {   // RMSNorm factor of each operand row, summed in a fixed order
+    if (p.ssq_in && !p.publish) {   // RMSNorm factor of each operand row, summed in a fixed order
       const int n = p.M * p.ssq_n;            // <= MPAD * 64 <= the staging area
       for (int i = r; i < n; i += 128) staging[i] = __ldcg(p.ssq_in + (i / p.ssq_n) * p.ssq_ld + i % p.ssq_n);
       named_bar_sync(1, 128);
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
       }
       named_bar_sync(1, 128);
     }
-    if (p.epi == EPI_QKV) {   // cache slot and RoPE position of every row (fixed during the forward)
+    if (p.epi == EPI_QKV && !p.publish) {   // cache slot and RoPE position of every row (fixed during the forward)
       if (r < p.M) {
         const int seq = p.seq0 + r / p.q;
         const int slot = __ldcg(p.len + seq) + r % p.q;
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
       float pre_gn = 0.f;
       {
         const int n = 128 * tile + r;
-        const bool resid = p.epi == EPI_RESID && n < p.N;
+        const bool resid = p.epi == EPI_RESID && !p.publish && n < p.N;
 #pragma unroll
         for (int u = 0; u < C::EGR; ++u) pre[u] = (resid && u < p.M) ? __ldcg(p.out + (size_t)u * p.out_ld + n) : 0.f;
         if (resid && p.gain_next) pre_gn = __bfloat162float(p.gain_next[n]);
@@ -526,13 +526,17 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
       const bool edge = tile == tile_first || tile == tile_last;
       const int c_lo = edge ? s_share[sh] : cta, c_hi = edge ? s_share[sh + 1] : cta;
       const int lo_slot = s_share[sh + 2];
-      if (c_hi > c_lo) {
+      if (c_hi > c_lo || p.publish) {
         // this tile is shared: publish the partial, the last contributor reduces
         const int slot = (tile == tile_first) ? 0 : 1;
         float* mine = p.partials + (size_t)(cta * 2 + slot) * MPAD * 128;
 #pragma unroll
         for (int m = 0; m < MPAD; ++m)
           if (m < p.M) mine[m * 128 + r] = acc[m];
+        if (p.publish) {   // gemm_finish_kernel does the rest
+          if (r == 0 && last_seg && p.trace.rec) s_mark[2] = globaltimer_ns();
+          continue;
+        }
         // publish: the CTA's stores, then one release/acquire counter update (thread r = 0)
         named_bar_sync(1, 128);
         if (r == 0) *s_last = (atomic_add_acq_rel_gpu(&p.counters[tile], 1) == c_hi - c_lo);
@@ -601,6 +605,117 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
     trace_write(p.trace, (unsigned)s_mark[3], t_entry, t_wait, s_mark[0], s_mark[1], s_mark[2], globaltimer_ns());
 }
 
+// ---- the second kernel of O, down and QKV at 17 to 24 rows ----------------------------------
+// With many rows the last contributors' sums (ten parts of 12 KB at 24 rows) and epilogues take 5
+// to 7 us after the last accumulator, on few of the SMs.  At 24 padded rows every CTA only
+// publishes its parts, and one warp per (row, tile) of this kernel, on every SM, sums them in CTA
+// order and runs the epilogue.  Four 7B layers and the head, without and with it: 24 rows 486.9 ->
+// 476.5 us, 20 rows 468.4 -> 461.6, 18 rows 446.7 -> 445.1 (13B, 24 rows: 667.9 -> 665.5).  Fewer
+// rows end sooner by themselves (16: 418.4 -> 434.6, 11: 417.2 -> 444.8, 6: 386.2 -> 426.0), and
+// at 28 rows it is slower too (513.8 -> 527.4).
+constexpr int GEMM_PUBLISH_MPAD = 24;
+constexpr int FIN_PARTS = 6;   // parts loaded together
+
+__device__ __forceinline__ void fin_split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(a - __low2float(h), b - __high2float(h));
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+__global__ void __launch_bounds__(256) gemm_finish_kernel(const __grid_constant__ GemmParams p) {
+  pdl_trigger();
+  pdl_wait();
+  const int lane = threadIdx.x & 31, gw = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int m = gw / p.n_tiles, tile = gw - m * p.n_tiles;
+  if (m >= p.M) return;   // (whole warps)
+  const int T = p.n_tiles * p.kc;
+  const int lo = cta_of_chunk(tile * p.kc, T, p.P, p.kc, p.snap);
+  const int hi = cta_of_chunk(tile * p.kc + p.kc - 1, T, p.P, p.kc, p.snap);
+  const int lo_slot = unit_begin(lo, T, p.P, p.kc, p.snap) == tile * p.kc ? 0 : 1;
+  auto part = [&](int j) { return p.partials + ((size_t)(j * 2 + (j == lo ? lo_slot : 0)) * p.mpad + m) * 128; };
+  if (p.epi == EPI_RESID) {
+    // h += sum, the next norm's operand h * g and the tile's sum of h^2
+    const int n = 128 * tile + 4 * lane;
+    const bool in = n < p.N;   // (N is a multiple of 8)
+    float* dst = p.out + (size_t)m * p.out_ld + n;
+    float4 h = in ? __ldcg(reinterpret_cast<const float4*>(dst)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = lo; j <= hi; j += FIN_PARTS) {
+      float4 t[FIN_PARTS];
+#pragma unroll
+      for (int u = 0; u < FIN_PARTS; ++u)
+        t[u] = j + u <= hi ? __ldcg(reinterpret_cast<const float4*>(part(j + u)) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < FIN_PARTS; ++u) y.x += t[u].x, y.y += t[u].y, y.z += t[u].z, y.w += t[u].w;
+    }
+    float sq = 0.f;
+    if (in) {
+      h.x += y.x, h.y += y.y, h.z += y.z, h.w += y.w;
+      sq = (h.x * h.x + h.y * h.y) + (h.z * h.z + h.w * h.w);
+      *reinterpret_cast<float4*>(dst) = h;
+      const uint2 gb = __ldg(reinterpret_cast<const uint2*>(p.gain_next + n));
+      uint2 xh, xl;
+      fin_split2(h.x * __uint_as_float(gb.x << 16), h.y * __uint_as_float(gb.x & 0xFFFF0000u), xh.x, xl.x);
+      fin_split2(h.z * __uint_as_float(gb.y << 16), h.w * __uint_as_float(gb.y & 0xFFFF0000u), xh.y, xl.y);
+      *reinterpret_cast<uint2*>(p.xn_hi + (size_t)m * p.out_ld + n) = xh;
+      *reinterpret_cast<uint2*>(p.xn_lo + (size_t)m * p.out_ld + n) = xl;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) p.ssq_out[m * p.ssq_ld + tile] = sq;
+    return;
+  }
+  // EPI_QKV: the tile lies in one of q, k, v and holds whole heads; two rotate-half pairs a lane
+  const int R = p.rows_per_map, half = p.hd >> 1, x = 2 * lane, i = x & (half - 1), r1 = (x - i) * 2 + i;
+  const int which = (128 * tile >= R) + (128 * tile >= 2 * R), f = 128 * tile - which * R + r1;
+  float2 a = make_float2(0.f, 0.f), b = a;
+  for (int j = lo; j <= hi; j += FIN_PARTS) {
+    float2 t[FIN_PARTS], u2[FIN_PARTS];
+#pragma unroll
+    for (int u = 0; u < FIN_PARTS; ++u) {
+      t[u] = u2[u] = make_float2(0.f, 0.f);
+      if (j + u <= hi) {
+        t[u] = __ldcg(reinterpret_cast<const float2*>(part(j + u) + r1));
+        u2[u] = __ldcg(reinterpret_cast<const float2*>(part(j + u) + r1 + half));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < FIN_PARTS; ++u) a.x += t[u].x, a.y += t[u].y, b.x += u2[u].x, b.y += u2[u].y;
+  }
+  if (p.ssq_in) {   // the operand row's RMSNorm factor
+    float s = 0.f;
+    for (int t = lane; t < p.ssq_n; t += 32) s += __ldcg(p.ssq_in + m * p.ssq_ld + t);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    s = 1.0f / sqrtf(s / (float)p.norm_dim + p.norm_eps);
+    a.x *= s, a.y *= s, b.x *= s, b.y *= s;
+  }
+  const int seq = p.seq0 + m / p.q, slot = __ldcg(p.len + seq) + m % p.q;
+  int pos = p.positions ? __ldcg(p.positions + m) : slot;
+  if (pos < 0 || pos >= p.rope_len) {
+    if (lane == 0 && which == 1) set_error(p.err, ERR_POSITION);
+    pos = pos < 0 ? 0 : p.rope_len - 1;
+  }
+  if (which < 2) {
+    const float4 cs = __ldg(reinterpret_cast<const float4*>(p.rope + (size_t)pos * half + i));   // cos, sin twice
+    const float2 o = a;
+    a = make_float2(a.x * cs.x - b.x * cs.y, a.y * cs.z - b.y * cs.w);
+    b = make_float2(b.x * cs.x + o.x * cs.y, b.y * cs.z + o.y * cs.w);
+  }
+  if (which == 0) {
+    float* dst = p.out + (size_t)m * p.out_ld + f;
+    *reinterpret_cast<float2*>(dst) = a;
+    *reinterpret_cast<float2*>(dst + half) = b;
+  } else if (slot < p.cap) {
+    __nv_bfloat16* dst = (which == 1 ? p.k_layer : p.v_layer) + (((size_t)seq * p.H + (f - i) / p.hd) * p.cap + slot) * p.hd + i;
+    *reinterpret_cast<__nv_bfloat162*>(dst) = __floats2bfloat162_rn(a.x, a.y);
+    *reinterpret_cast<__nv_bfloat162*>(dst + half) = __floats2bfloat162_rn(b.x, b.y);
+  } else if (lane == 0 && which == 1) {
+    set_error(p.err, ERR_CAPACITY);
+  }
+}
+
 // Rows are padded to a multiple of 8 (16 is the smallest N of the MMA: 8 rows, hi and lo): the
 // operand's padding costs L2 -> SM traffic, shared memory and epilogue time.
 // us per launch, 6 rows padded to 16 -> 8: QKV 21.6 -> 20.9, O 12.4 -> 11.4, gate/up 34.7 -> 33.4,
@@ -642,6 +757,7 @@ struct LaunchGemm {
 }  // namespace
 
 cudaError_t gemm_prepare() {
+  if (const cudaError_t e = prefer_shared(gemm_finish_kernel); e != cudaSuccess) return e;
   for (int mpad : GEMM_MPADS) {
     const cudaError_t e = with_mpad(mpad, PrepareGemm{});
     if (e != cudaSuccess) return e;
@@ -677,7 +793,15 @@ cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return with_mpad(gemm_mpad(p.M), LaunchGemm{p, cfg});
+  p.mpad = gemm_mpad(p.M);
+  p.publish = p.mpad == GEMM_PUBLISH_MPAD && (p.epi == EPI_QKV || (p.epi == EPI_RESID && p.gain_next)) &&
+              p.P > p.n_tiles;   // ranges shorter than a tile: at most two parts per CTA
+  const cudaError_t e = with_mpad(p.mpad, LaunchGemm{p, cfg});
+  if (e != cudaSuccess || !p.publish) return e;
+  cfg.gridDim = dim3((p.M * p.n_tiles + 7) / 8);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, gemm_finish_kernel, p);
 }
 
 }  // namespace sdsat

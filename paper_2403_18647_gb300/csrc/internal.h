@@ -84,6 +84,8 @@ struct GemmParams {
   int P;              // CTAs
   int snap;           // stream-K split points within a tile's first `snap` units move to the tile start
   int M;              // activation rows (<= MPAD)
+  int mpad;           // set by launch_gemm
+  int publish;        // set by launch_gemm: CTAs only publish their parts, gemm_finish_kernel does the rest
   // epilogue
   int epi;
   float* out;

@@ -89,3 +89,25 @@ def test_gemm_row_padding(ctx, M):
     ref = x.double() @ w.double().t()
     tol = 5e-5 * K ** 0.5 * 0.02 + 1e-6 * ref.abs().max().item()   # as the other GEMM parity tests
     assert (y.double() - ref).abs().max().item() <= tol
+
+
+@pytest.mark.parametrize("H,hd,ffn", [(9, 128, 1184), (18, 64, 2000)])
+def test_second_kernel_of_split_tiles(H, hd, ffn):
+    """17 to 24 rows with tiles split along K (d 1152): O, down and QKV end in a second kernel.
+    Chains and trees against single sequences, and rows past the capacity."""
+    import paper_2403_18647_gb300 as sd
+    shape = synth.ModelShape("mid", 2, H * hd, H, hd, ffn, 1003, 1000)
+    ctx = sd.Context(shape, synth.make_model(shape, seed=0, device="cuda", gain_std=0.1), max_position=256)
+    for b, q in ((6, 3), (4, 5), (7, 3), (4, 6)):
+        test_batch_equals_single_sequences(ctx, b, q)
+    test_tree_batch_equals_single_sequences(ctx, 2, 11)
+    b, q = 2, 10
+    kv = ctx.kv(b, 100)
+    ctx.kv_commit(kv, torch.tensor([100 - q, 100 - 4], dtype=torch.int32, device="cuda"), b)
+    toks = synth.uniform_ids(5, 1, b * q, shape.vocab, device="cuda")
+    ctx.block_forward(kv, toks, torch.empty(b * q, shape.vocab, device="cuda"), b, q)
+    assert ctx.get_error() == 0x4
+    for i, n in ((0, q), (1, 4)):
+        for x in ctx.kv_read(kv, 1, i, 0, 100):
+            w = x.float().abs().sum(dim=(0, 2))
+            assert (w[:100 - n] == 0).all() and (w[100 - n:] > 0).all()
