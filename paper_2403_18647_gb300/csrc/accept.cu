@@ -76,10 +76,12 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32
 // One thread-block cluster per row: p.cs CTAs of ACC_THREADS threads; thread t of rank r owns
 // the ids [ACC_SPAN r + ACC_EPT t, + ACC_EPT) (ascending id order is rank, thread, slot order).
 // One CTA per row (1024 threads of 32 ids) left most SMs idle and ran its chain of dependent
-// steps on four times the work per thread.  us per call, 32016 logits a row, one CTA per row ->
-// a cluster: 24 rows, top-p 0.95, T 0.2: 48.4 -> 22.5; with top-k 10: 34.5 -> 16.7; T 1 (row-wide
-// searches): 101 -> 47; greedy 7.1 -> 5.0; 64 rows (512 CTAs, more than one wave): 48 -> 36, T 1:
-// 101 -> 93, greedy 7.35 -> 7.4.  What is left is the chain of barriers, not bytes (3 MB).
+// steps on four times the work per thread.  us per call, 32016 logits a row, one CTA per row (with
+// a sorted list, or binary searches over the row) -> a cluster, and cuts by digits: 24 rows, top-p
+// 0.95, T 0.2: 48.4 -> 14.4 (22.6 with the sort); with top-k 10: 34.5 -> 16.6; T 1 (row-wide):
+// 101 -> 22.7 (46.8 with the searches); greedy 7.1 -> 5.0; 64 rows (512 CTAs, four on an SM):
+// 48 -> 22.5, T 1: 101 -> 37.7, greedy 7.4 -> 6.3.  What is left is the chain of barriers and of
+// instructions fetched cold, not bytes (3 MB).
 // A sum over the row: the warps' totals meet in shared
 // memory, warp 0 writes the CTA's total into every CTA of the cluster (distributed shared
 // memory), and after one cluster barrier each warp reads the cluster's totals locally.  (Every
@@ -91,7 +93,8 @@ constexpr int ACC_EPT = 8;
 constexpr int ACC_SPAN = ACC_THREADS * ACC_EPT;   // 4096 ids per CTA, vocab <= 32768
 constexpr int ACC_WARPS = ACC_THREADS / 32;
 constexpr int ACC_CS = 8;                         // most CTAs of a row
-constexpr int ACC_WORDS = 5;                      // 64-bit words of one warp's slot
+constexpr int ACC_WORDS = 4;                      // most 64-bit words summed together
+static_assert(ACC_WARPS == 16 && ACC_CS == 8 && ACC_WORDS == 4, "eight lanes of a warp per word");
 
 struct AccSlots {
   unsigned long long w[2][ACC_WARPS * ACC_WORDS];   // this CTA's warps
@@ -100,6 +103,11 @@ struct AccSlots {
 
 __device__ __forceinline__ void st_dsmem_u64(uint32_t addr, uint64_t v) {
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ uint64_t ld_dsmem_u64(uint32_t addr) {
+  uint64_t v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
 #pragma unroll
@@ -116,37 +124,34 @@ struct Row {   // the row's cluster, seen from one thread
   AccSlots* slots;
   int cs, rank, ph;
   // v[n]: this warp's values (every lane); afterwards combine() of them over the row, and with
-  // `before` the sum of word 0 over the warps that come before this one in id order
+  // `before` the sum of word 0 over the warps that come before this one in id order.  Eight lanes
+  // per word, so all words go through the same three shuffles.
   template <int N, typename F>
   __device__ void reduce(uint64_t (&v)[N], uint64_t identity, F combine, uint64_t* before = nullptr) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = lane >> 3, i = lane & 7;
     unsigned long long* mine = slots->w[ph & 1];
     unsigned long long* all = slots->c[ph & 1];
     ++ph;
+    auto over8 = [&](uint64_t t) {
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) t = combine(t, (uint64_t)__shfl_xor_sync(0xffffffffu, t, o));
+      return t;
+    };
     if (lane == 0)
 #pragma unroll
-      for (int n = 0; n < N; ++n) mine[w * N + n] = v[n];
+      for (int k = 0; k < N; ++k) mine[k * ACC_WARPS + w] = v[k];
     __syncthreads();
     if (w == 0) {
-#pragma unroll
-      for (int n = 0; n < N; ++n) {
-        uint64_t t = lane < ACC_WARPS ? mine[lane * N + n] : identity;
-#pragma unroll
-        for (int o = ACC_WARPS / 2; o > 0; o >>= 1) t = combine(t, (uint64_t)__shfl_xor_sync(0xffffffffu, t, o));
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (lane < cs) st_dsmem_u64(mapa_shared(smem_u32(&all[rank * N + n]), lane), t);
-      }
+      const uint64_t t = over8(n < N ? combine((uint64_t)mine[n * ACC_WARPS + i], (uint64_t)mine[n * ACC_WARPS + 8 + i]) : identity);
+      if (n < N && i < cs) st_dsmem_u64(mapa_shared(smem_u32(&all[n * ACC_CS + rank]), i), t);
     }
     cluster_sync_all();
+    const uint64_t t = n < N && i < cs ? all[n * ACC_CS + i] : identity;
+    if (before)   // earlier CTAs, then earlier warps of this one
+      *before = warp_sum_u64((lane < rank ? t : 0) + (lane < w ? mine[lane] : 0));
+    const uint64_t r = over8(t);
 #pragma unroll
-    for (int n = 0; n < N; ++n) {
-      uint64_t t = lane < cs ? all[lane * N + n] : identity;
-      if (n == 0 && before)   // earlier CTAs, then earlier warps of this one
-        *before = warp_sum_u64((lane < rank ? t : 0) + (lane < w ? mine[lane * N] : 0));
-#pragma unroll
-      for (int o = ACC_CS / 2; o > 0; o >>= 1) t = combine(t, (uint64_t)__shfl_xor_sync(0xffffffffu, t, o));
-      v[n] = __shfl_sync(0xffffffffu, t, 0);
-    }
+    for (int k = 0; k < N; ++k) v[k] = __shfl_sync(0xffffffffu, r, 8 * k);
   }
   template <int N>
   __device__ void sum(uint64_t (&v)[N], uint64_t* before = nullptr) {
@@ -162,8 +167,8 @@ struct Row {   // the row's cluster, seen from one thread
     sum<1>(v);
     return v[0];
   }
-  // exclusive prefix over the row's threads, in id order, of v < 2^29
-  __device__ uint64_t exscan(uint32_t v) {
+  // exclusive prefix over the row's threads, in id order
+  __device__ uint64_t exscan(uint64_t v) {
     const int lane = threadIdx.x & 31;
     uint64_t x = v;
 #pragma unroll
@@ -259,293 +264,118 @@ __device__ int row_argmax(const float* row, int V, uint32_t* err, Row& rw) {
 }
 
 // ---- nucleus: the fixed-point top-k / top-p sampler ------------------------------------
-// A thread keeps the weights W (uint32, <= 2^24) of its ids in registers.  Selections are
-// predicates on (W, id); per-thread sums fit 32 bits, row sums 64.
-struct Cut {
-  uint32_t xk;  // top-k: candidates are W > xk, or W == xk and id <= idk
-  int idk;
-  uint32_t xp;  // top-p: kept candidates are W > xp, or W == xp and id <= idp
-  int idp;
-};
-enum Pred : int {
-  P_GE = 1,         // W >= x
-  P_GT = 2,         // W > x
-  P_EQ = 3,         // W == x
-  P_CAND = 4,       // candidate
-  P_CAND_GE = 5,    // candidate and W >= x
-  P_CAND_GT = 6,    // candidate and W > x
-  P_CAND_EQ = 7,    // candidate and W == x
-  P_KEPT = 8,       // kept
-};
-
-template <int P>
-__device__ __forceinline__ bool pred(uint32_t W, int id, const Cut& c, uint32_t x) {
-  const bool cand = W > c.xk || (W == c.xk && id <= c.idk);
-  switch (P) {
-    case P_GE: return W >= x;
-    case P_GT: return W > x;
-    case P_EQ: return W == x;
-    case P_CAND: return cand;
-    case P_CAND_GE: return cand && W >= x;
-    case P_CAND_GT: return cand && W > x;
-    case P_CAND_EQ: return cand && W == x;
-    default: return cand && (W > c.xp || (W == c.xp && id <= c.idp));
-  }
-}
-
-// per-thread sum of W (COUNT: number of ids) over the owned ids selected by P (< 2^28)
-template <int P, bool COUNT>
-__device__ __forceinline__ uint32_t lsum(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x) {
-  uint32_t s = 0;
-#pragma unroll
-  for (int e = 0; e < ACC_EPT; ++e)
-    if (pred<P>(W[e], base + e, c, x)) s += COUNT ? 1u : W[e];
-  return s;
-}
-template <int P, bool COUNT>
-__device__ __forceinline__ uint64_t row_sum(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x, Row& rw) {
-  return rw.sum(warp_total(lsum<P, COUNT>(W, base, c, x)));
-}
-
-// largest x in [0, 2^24] whose row total of lsum<P, COUNT>(x) is >= need (monotone in x); three
-// thresholds a step: a step is one cluster barrier, whose latency outweighs the sums
-template <int P, bool COUNT>
-__device__ __forceinline__ uint32_t search_threshold(const uint32_t (&W)[ACC_EPT], int base, const Cut& c,
-                                                     uint64_t need, Row& rw) {
-  uint32_t lo = 0, hi = 1u << 24;
-  while (lo < hi) {
-    const uint32_t d = (hi - lo + 3) / 4;
-    const uint32_t x[3] = {min(lo + d, hi), min(lo + 2 * d, hi), min(lo + 3 * d, hi)};
-    uint64_t t[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) t[i] = warp_total(lsum<P, COUNT>(W, base, c, x[i]));
-    rw.sum<3>(t);
-    uint32_t nlo = lo, nhi = hi;
-#pragma unroll
-    for (int i = 2; i >= 0; --i) {
-      if (t[i] >= need) nlo = max(nlo, x[i]);
-      else nhi = x[i] - 1;   // (the last assignment is the lowest failing threshold's)
-    }
-    lo = nlo;
-    hi = nhi;
-  }
-  return lo;
-}
-
-// the n-th (n >= 1) smallest id selected by P, or INT_MAX if there are fewer
-template <int P>
-__device__ __forceinline__ int nth_id(const uint32_t (&W)[ACC_EPT], int base, const Cut& c, uint32_t x,
-                                      uint64_t n, Row& rw) {
-  const uint32_t mine = lsum<P, true>(W, base, c, x);
-  uint64_t k = rw.exscan(mine);
-  uint32_t hit = 0;   // id + 1 in the one thread that holds it
-  if (k < n && k + mine >= n) {
-#pragma unroll
-    for (int e = 0; e < ACC_EPT; ++e)
-      if (pred<P>(W[e], base + e, c, x) && ++k == n) hit = base + e + 1;
-  }
-  const uint64_t id = rw.sum(warp_total(hit));
-  return id ? (int)id - 1 : 0x7FFFFFFF;
-}
-
-// ---- the sampler on a compacted list ----------------------------------------------------
-// The kept set is a prefix of the order (W desc, id asc), so it lies among the heaviest
-// weights.  With a floor F such that the elements with W >= F provably contain it (top-k:
-// at least k of them, or all non-zero weights; top-p alone: their mass reaches the top-p
-// threshold), those elements go in ascending id order into rank 0's shared memory, and that
-// CTA finishes the row.  Otherwise the row-wide searches over all ids run.
+// The kept set is a prefix of the order (W desc, id asc): every W above a cut x, and the first
+// `ties` ids with W == x.  The cut (of a count for top-k, of a mass for top-p) is found digit by
+// digit: three histograms of 256 bins over W - 1, highest digit first, each scanned from the
+// heaviest bin to the one where the running sum reaches what is needed.
+//
+// The kept set lies among the heaviest weights.  With a floor such that the elements with W >=
+// floor provably contain it (top-k: at least k of them, or all non-zero weights; top-p alone:
+// their mass reaches the top-p threshold), those elements go in ascending id order into rank 0's
+// shared memory, and that CTA finishes the row with block barriers only.  Otherwise (more than
+// NUC_LIST_MAX of them) the same steps run over all ids, with histograms summed over the cluster.
 constexpr int NUC_LIST_MAX = 4096;
 constexpr int NUC_FLOORS = 7;
-// floor f: 2^24 (the largest weight), 2^22, 2^20, 2^18, 2^16 (ratio 2^-8), 2^8 (2^-16), then 1
-// (every non-zero weight).  Weights of bucket b (nuc_bucket) are >= the floors f >= b.
-__device__ __forceinline__ int nuc_bucket(uint32_t w) {
-  if (w == 0) return NUC_FLOORS;
-  const int e = 31 - __clz(w);
-  return e >= 16 ? (25 - e) >> 1 : (e >= 8 ? 5 : 6);
-}
 
-struct NucList {
-  unsigned long long key[NUC_LIST_MAX];      // nuc_key of the list's elements, ascending id
-  unsigned long long sorted[NUC_LIST_MAX];   // the same in descending order
-  unsigned long long kstar, sk;              // the kept prefix's last key and its mass
-  int pick;
+struct NucSmem {
+  unsigned long long key[NUC_LIST_MAX];     // the list (rank 0): W << 32 | id, ascending id
+  uint32_t own[ACC_EPT * ACC_THREADS];      // [slot][thread]: the threads' logits, then their W
+  uint32_t lo[256], hi[256];                // histogram: sums of W & 4095 (or counts) and of W >> 12; 0 between uses
+  unsigned long long bins[2][256];          // row-wide: this CTA's histogram, for the cluster
+  unsigned long long above;
+  int digit, pick;
 };
 
-__device__ __forceinline__ uint64_t nuc_key(uint32_t w, int id) {   // larger: heavier, then lower id
-  return ((uint64_t)w << 32) | (uint32_t)(0x7FFFFFFF - id);
-}
-
-// Steps 4-7 on the list (warp 0) when the candidates (top-k, k <= 32) or, without top-k, the
-// kept prefix have at most 32 elements: up to 32 rounds of "largest key below the previous
-// one" put them on the lanes in (W desc, id asc) order.  Returns -1 when this does not apply.
-__device__ int list_small(const AcceptParams& p, const NucList& L, int n, uint64_t S_all, bool topk, uint64_t rnd) {
-  const int lane = threadIdx.x & 31;
-  if (topk && p.top_k > 32) return -1;
-  uint64_t thr = 0;
-  if (!topk) {
-    const uint64_t prod = (uint64_t)p.p_fixed * S_all;
-    thr = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-  }
-  const int rounds = topk ? min(p.top_k, n) : min(32, n);
-  uint64_t prev = ~0ull, mine = 0, C = 0;
-  int nc = 0;
-  bool done = topk;
-  for (int r = 0; r < rounds && !(nc > 0 && !topk && C >= thr); ++r) {
-    uint64_t best = 0;
-    for (int i = lane; i < n; i += 32) {
-      const uint64_t k = L.key[i];
-      if (k < prev && k > best) best = k;
-    }
-    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32));
-    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(best >> 32) == hi ? (uint32_t)best : 0u);
-    prev = ((uint64_t)hi << 32) | lo;
-    if (lane == r) mine = prev;
-    ++nc;
-    C += hi;   // the round's weight
-  }
-  if (!topk) done = C >= thr;   // the kept prefix: the first nc elements reach the threshold
-  if (!done) return -1;
-  const uint32_t w = lane < nc ? (uint32_t)(mine >> 32) : 0u;
-  const int id = 0x7FFFFFFF - (int)(uint32_t)mine;
-  bool kept = lane < nc;
-  if (topk) {
-    // candidates = the nc lanes; kept = the shortest prefix whose mass reaches thr
-    const uint64_t S = __reduce_add_sync(0xffffffffu, w);
-    const uint64_t prod = (uint64_t)p.p_fixed * S;
-    const uint64_t t = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-    uint32_t incl = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    kept = kept && (lane == 0 || (uint64_t)(incl - w) < t);
-  }
-  const uint32_t kw = kept ? w : 0u;
-  const uint64_t Sk = __reduce_add_sync(0xffffffffu, kw);
-  const uint64_t tau = __umul64hi(rnd, Sk);
-  // ascending-id cumulative weight of the kept elements up to and including this lane's
-  uint64_t cum = 0;
-  for (int j = 0; j < nc; ++j) {
-    const uint32_t wj = __shfl_sync(0xffffffffu, kw, j);
-    const int idj = __shfl_sync(0xffffffffu, id, j);
-    if (idj <= id) cum += wj;
-  }
-  const uint32_t m = __ballot_sync(0xffffffffu, kept && cum > tau && cum - kw <= tau);
-  return __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
-}
-
-// L.sorted = the n2 (a power of two >= 32, the list's n keys and zeros) keys in descending
-// order: bitonic; distances below 32 stay in the warp (element i is on lane i & 31), so 1024
-// keys take 15 block barriers and not 55.
-__device__ void list_sort(NucList& L, int n, int n2) {
-  constexpr int PER = NUC_LIST_MAX / ACC_THREADS;
-  auto in_warp = [&](uint64_t x, int i, int k, int j) {   // distances j .. 1 of the merge of size k
-    for (; j > 0; j >>= 1) {
-      const uint64_t y = __shfl_xor_sync(0xffffffffu, x, j);
-      // descending blocks where bit k of i is clear: the lower element keeps the larger key
-      const bool keep_max = ((i & k) == 0) == ((i & j) == 0);
-      x = keep_max ? max(x, y) : min(x, y);
-    }
-    return x;
-  };
+// The largest x whose sum over the elements with W >= x is >= need (1 <= need <= their total), W
+// itself summed or (COUNT) their number, and `above`, the sum over W > x.  each(f) calls f(W) for
+// this thread's elements; a W of 0 is in no sum.  ROW: over the cluster, otherwise over the block.
+template <bool COUNT, bool ROW, typename E>
+__device__ __forceinline__ uint32_t weight_cut(NucSmem& L, E each, uint64_t need, uint64_t& above, uint64_t* red, Row& rw) {
+  uint32_t prefix = 0;   // the digits of x - 1 found so far
+  above = 0;
 #pragma unroll 1
-  for (int r = 0; r < PER; ++r) {
-    const int i = threadIdx.x + r * ACC_THREADS;
-    if (i >= n2) break;   // (whole warps)
-    uint64_t x = i < n ? L.key[i] : 0ull;   // padding sorts last (every list W >= 1)
-    for (int k = 2; k <= 32; k <<= 1) x = in_warp(x, i, k, k >> 1);
-    L.sorted[i] = x;
-  }
-  for (int k = 64; k <= n2; k <<= 1) {
-    for (int j = k >> 1; j >= 32; j >>= 1) {
-      __syncthreads();
-      for (int i = threadIdx.x; i < n2; i += ACC_THREADS) {
-        const int l = i ^ j;
-        if (l > i) {
-          const uint64_t a = L.sorted[i], b = L.sorted[l];
-          if (((i & k) == 0) == (a < b)) {
-            L.sorted[i] = b;
-            L.sorted[l] = a;
-          }
-        }
-      }
+  for (int sh = 16; sh >= 0; sh -= 8) {
+    each([&](uint32_t W) {
+      const uint32_t u = W - 1;
+      if (W == 0 || (u >> sh) >> 8 != prefix) return;
+      const uint32_t b = (u >> sh) & 255u;
+      atomicAdd(&L.lo[b], COUNT ? 1u : W & 4095u);     // <= 2^24 with 4096 elements a CTA
+      if (!COUNT) atomicAdd(&L.hi[b], W >> 12);
+    });
+    __syncthreads();
+    const int b = 255 - (int)threadIdx.x;   // one bin per thread, heaviest first
+    uint64_t v = 0;
+    if (b >= 0) {
+      v = ((uint64_t)L.hi[b] << 12) + L.lo[b];
+      L.lo[b] = L.hi[b] = 0;
+    }
+    if (ROW) {   // (a buffer is written again after another cluster barrier, when every CTA has read it:
+                 // two steps later, or after the row sum between two cuts)
+      unsigned long long* mine = L.bins[(sh >> 3) & 1];
+      if (b >= 0) mine[b] = v;
+      cluster_sync_all();
+      v = 0;
+      if (b >= 0)
+        for (int c = 0; c < rw.cs; ++c) v += ld_dsmem_u64(mapa_shared(smem_u32(&mine[b]), c));
+    }
+    const uint64_t before = above + block_exscan_u64(v, red);
+    if (before < need && before + v >= need) {   // one thread
+      L.digit = b;
+      L.above = before;
     }
     __syncthreads();
-#pragma unroll 1
-    for (int r = 0; r < PER; ++r) {
-      const int i = threadIdx.x + r * ACC_THREADS;
-      if (i >= n2) break;
-      L.sorted[i] = in_warp(L.sorted[i], i, k, 16);
-    }
+    prefix = prefix << 8 | (uint32_t)L.digit;
+    above = L.above;
   }
-  __syncthreads();
+  return prefix + 1;
 }
 
-// Steps 4-7 on the list with the whole CTA.  The list holds the first n elements of the order
-// (W desc, id asc), in ascending id.  Its keys are sorted once, so the candidates (the first
-// min(k, n)), their mass, the kept prefix (the shortest one whose mass reaches
-// ceil(P S / 2^24)) and its mass are prefix sums of the sorted weights.  The pick then scans
-// the list itself in ascending id with "kept" = key >= the kept prefix's last key.
-__device__ int list_sorted_select(const AcceptParams& p, NucList& L, int n, uint64_t S_all, uint64_t rnd,
-                                  uint64_t* red) {
-  int n2 = 32;
-  while (n2 < n) n2 <<= 1;
-  list_sort(L, n, n2);
-  // candidates and the kept prefix: thread t holds `per` consecutive sorted elements
-  const int per = (n + ACC_THREADS - 1) / ACC_THREADS, i0 = threadIdx.x * per, i1 = min(i0 + per, n);
-  const bool topk = p.top_k > 0 && p.top_k < p.V;
-  const int nc = topk ? min(p.top_k, n) : n;
-  uint64_t wsum = 0;
-  for (int i = i0; i < min(i1, nc); ++i) wsum += L.sorted[i] >> 32;
-  const uint64_t S = topk ? block_sum_u64(wsum, red) : S_all;
-  const uint64_t prod = (uint64_t)p.p_fixed * S;
-  const uint64_t thr = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-  const uint64_t before = block_exscan_u64(wsum, red);
-  // the first sorted index whose inclusive mass reaches thr (index 0 when thr = 0); the list
-  // provably holds it
-  if (thr == 0 ? threadIdx.x == 0 : (before < thr && before + wsum >= thr)) {
-    uint64_t cum = before;
-    for (int i = i0; i < i1; ++i) {
-      cum += L.sorted[i] >> 32;
-      if (cum >= thr) {
-        L.kstar = L.sorted[i];
-        L.sk = cum;
-        break;
-      }
-    }
+// ceil(P S / 2^24), and 1 where that is 0 (the heaviest candidate is always kept)
+__device__ __forceinline__ uint64_t top_p_need(const AcceptParams& p, uint64_t S) {
+  const uint64_t prod = (uint64_t)p.p_fixed * S;   // P <= 2^24, S < 2^40
+  return max((uint64_t)1, (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0));
+}
+
+// Steps 4-5: the kept set's cut.  each as above; total: sum of
+// W over every id; k: candidates (0: all).  Kept are W > x and the first `ties` ids with W == x,
+// together `mass`.
+template <bool ROW, typename E, typename S>
+__device__ __forceinline__ void kept_cut(const AcceptParams& p, NucSmem& L, E each, S total_of, uint64_t total,
+                                         uint32_t k, uint64_t* red, Row& rw, uint32_t& x, uint64_t& ties, uint64_t& mass) {
+  uint64_t need, above;
+  x = 0;
+  if (k) {   // 4. the k largest, then their mass
+    const uint32_t xk = weight_cut<true, ROW>(L, each, k, above, red, rw);
+    uint64_t gt = 0;
+    each([&](uint32_t W) { gt += W > xk ? W : 0u; });
+    gt = total_of(gt);
+    need = top_p_need(p, gt + (k - above) * xk);
+    if (gt < need) x = xk, above = gt;   // the top-k cut's own weight; heavier ones otherwise
+  } else {
+    need = top_p_need(p, total);
   }
-  __syncthreads();
-  const uint64_t kstar = L.kstar, Sk = L.sk;
-  const uint64_t tau = __umul64hi(rnd, Sk);
-  // 7. the first kept id (ascending) whose inclusive cumulative weight exceeds tau
-  uint64_t mine = 0;
-  for (int i = i0; i < i1; ++i)
-    if (L.key[i] >= kstar) mine += L.key[i] >> 32;
-  const uint64_t below = block_exscan_u64(mine, red);
-  if (below <= tau && below + mine > tau) {
-    uint64_t cum = below;
-    for (int i = i0; i < i1; ++i)
-      if (L.key[i] >= kstar) {
-        cum += L.key[i] >> 32;
-        if (cum > tau) {
-          L.pick = 0x7FFFFFFF - (int)(uint32_t)L.key[i];
-          break;
-        }
-      }
-  }
-  __syncthreads();
-  return L.pick;
+  if (x == 0) x = weight_cut<false, ROW>(L, each, need, above, red, rw);   // 5.
+  ties = need - above <= x ? 1 : (need - above + x - 1) / x;
+  mass = above + ties * x;
+}
+
+// A prefix of elements in ascending id order as one word: the mass of those above the cut and
+// the number at it (mass <= 2^39, number <= 2^15), and the kept mass that it stands for.
+__device__ __forceinline__ uint64_t kept_word(uint32_t W, uint32_t x) { return W > x ? W : (W == x ? 1ull << 40 : 0ull); }
+__device__ __forceinline__ uint64_t kept_mass(uint64_t word, uint32_t x, uint64_t ties) {
+  return (word & ((1ull << 40) - 1)) + min(word >> 40, (uint64_t)ties) * x;
 }
 
 // The row's sampled id (valid in rank 0).  Every CTA of the cluster passes the same barriers:
-// every branch is taken on values that the whole row shares.
+// every branch is taken on values that the whole row shares.  These steps run once a call, so
+// their instructions are fetched cold: loops over a thread's ids stay rolled, through shared memory.
 __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* row, int position, int seq,
-                                           uint64_t* red, Row& rw, NucList& L) {
-  const int V = p.V;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int base = rw.rank * ACC_SPAN + threadIdx.x * ACC_EPT;
-  uint32_t W[ACC_EPT];
+                                           uint64_t* red, Row& rw, NucSmem& L) {
+  const int V = p.V, tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int base = rw.rank * ACC_SPAN + tid * ACC_EPT;
+  uint32_t* own = L.own + tid;   // slot e at own[e * ACC_THREADS]
+  if (tid < 256) L.lo[tid] = L.hi[tid] = 0;
+  float mx = -INFINITY;
   {
     // 1. logits (NaN -> -inf; ids >= V are -inf, hence W = 0) and the row maximum
     float l[ACC_EPT];
@@ -560,7 +390,6 @@ __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* r
       for (int e = 0; e < ACC_EPT; ++e) l[e] = base + e < V ? __ldcg(row + base + e) : -INFINITY;
     }
     bool nan = false;
-    float mx = -INFINITY;
 #pragma unroll
     for (int e = 0; e < ACC_EPT; ++e) {
       if (l[e] != l[e]) {
@@ -568,149 +397,138 @@ __device__ __forceinline__ int row_nucleus(const AcceptParams& p, const float* r
         l[e] = -INFINITY;
       }
       mx = fmaxf(mx, l[e]);
+      own[e * ACC_THREADS] = __float_as_uint(l[e]);
     }
     if (nan) set_error(p.err, ERR_NAN_LOGITS);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    // (ordered as in arg_key, with id bits that do not matter)
-    const uint32_t ord = (uint32_t)(rw.largest(arg_key(mx, 0)) >> 32);
+    // (ordered as in arg_key)
+    const uint32_t ord = (uint32_t)rw.largest(__reduce_max_sync(0xffffffffu, (uint32_t)(arg_key(mx, 0) >> 32)));
     mx = __uint_as_float((ord & 0x80000000u) ? ord & 0x7FFFFFFFu : ~ord);
-    // 2-3. W_i = floor(exp((l_i - max) / T) * 2^24)
-#pragma unroll
-    for (int e = 0; e < ACC_EPT; ++e) W[e] = fixed24(exp_sd(__fdiv_rn(__fsub_rn(l[e], mx), p.temperature)));
+  }
+  // 2-3. W_i = floor(exp((l_i - max) / T) * 2^24), which is 0 where (l_i - max) / T < -17 (e^-17 <
+  // 2^-24 by a third, far more than any rounding here).  Floors 0-6: 2^24 (the largest weight),
+  // 2^22, 2^20, 2^18, 2^16 (ratio 2^-8), 2^8 (2^-16), then 1 (every non-zero weight): the number
+  // of weights above each, 10 bits a field, and the mass above the last three.
+  const bool topk = p.top_k > 0 && p.top_k < V;
+  const float cut = -17.0f * p.temperature;
+  uint32_t c02 = 0, c35 = 0, c6 = 0, m4 = 0, m5 = 0, m6 = 0;   // (counts <= 8, masses <= 2^27)
+#pragma unroll 1
+  for (int e = 0; e < ACC_EPT; ++e) {
+    const float d = __fsub_rn(__uint_as_float(own[e * ACC_THREADS]), mx);
+    uint32_t W = 0;
+    if (!(d < cut)) W = fixed24(exp_sd(__fdiv_rn(d, p.temperature)));
+    own[e * ACC_THREADS] = W;
+    if (W) {
+      c02 += (W >> 24) + ((W >> 22 ? 1u : 0u) << 10) + ((W >> 20 ? 1u : 0u) << 20);
+      c35 += (W >> 18 ? 1u : 0u) + ((W >> 16 ? 1u : 0u) << 10) + ((W >> 8 ? 1u : 0u) << 20);
+      c6 += 1;
+      m4 += W >> 16 ? W : 0u;
+      m5 += W >> 8 ? W : 0u;
+      m6 += W;
+    }
   }
   // 6. the 64-bit draw keyed by (produced position, sequence)
   uint32_t ctr[4] = {(uint32_t)position, (uint32_t)seq, 0u, 0u};
   philox4x32_10(ctr, (uint32_t)(p.seed & 0xFFFFFFFFull), (uint32_t)(p.seed >> 32));
   const uint64_t rnd = ((uint64_t)ctr[0] << 32) | ctr[1];
 
-  // ---- the list path: counts (and, without top-k, masses) of the weights above each floor
-  const bool topk = p.top_k > 0 && p.top_k < V;
-  {
-    // per-thread counts (<= 8) of the floors in 16-bit fields: floors 0-3 and 4-6
-    uint64_t c03 = 0, c46 = 0;
-    uint32_t m4 = 0, m5 = 0, m6 = 0;   // masses >= floors 4, 5, 6 (< 2^28)
+  // Row totals.  Top-k: 16-bit counts (<= 32768) of floors 0-3 and 4-6; top-p alone: the counts
+  // of floors 4-6 and the three masses.
+  const uint32_t r35 = __reduce_add_sync(0xffffffffu, c35), r6 = __reduce_add_sync(0xffffffffu, c6);
+  const uint64_t n46 = (uint64_t)((r35 >> 10) & 1023u) | (uint64_t)(r35 >> 20) << 16 | (uint64_t)r6 << 32;
+  uint64_t t[ACC_WORDS] = {n46, warp_total(m6), 0, 0};
+  if (topk) {
+    const uint32_t r02 = __reduce_add_sync(0xffffffffu, c02);
+    t[2] = (uint64_t)(r02 & 1023u) | (uint64_t)((r02 >> 10) & 1023u) << 16 | (uint64_t)(r02 >> 20) << 32 |
+           (uint64_t)(r35 & 1023u) << 48;
+  } else {
+    t[2] = warp_total(m4);
+    t[3] = warp_total(m5);
+  }
+  const int buf = rw.ph & 1;
+  rw.sum<ACC_WORDS>(t);
+  const uint64_t S_all = t[1];
+  const int n_all = (int)((t[0] >> 32) & 0xFFFF);   // non-zero weights
+  if (n_all == 0) return 0;   // every weight 0 (all-NaN row): the lowest candidate, id 0
+  const uint32_t k = topk ? min((uint32_t)p.top_k, (uint32_t)n_all) : 0u;
+
+  // the highest floor whose elements provably hold the candidates (top-k) or the kept prefix
+  int f = -1, nf = 0;
+  const uint64_t need_all = top_p_need(p, S_all);
 #pragma unroll
-    for (int e = 0; e < ACC_EPT; ++e) {
-      const int b = nuc_bucket(W[e]);
+  for (int i = 0; i < NUC_FLOORS; ++i) {
+    if (i < 4 && !topk) continue;
+    const int n = (int)((i < 4 ? t[2] >> (16 * i) : t[0] >> (16 * (i - 4))) & 0xFFFF);
+    const bool holds = topk ? n >= (int)k : (i == 4 ? t[2] : i == 5 ? t[3] : S_all) >= need_all;
+    if (f < 0 && n <= NUC_LIST_MAX && holds) f = i, nf = n;
+  }
+  if (f >= 0) {
+    const uint32_t floor_w = f <= 4 ? 1u << (24 - 2 * f) : (f == 5 ? 256u : 1u);
+    // this thread's place in the list: the CTAs and warps before (from the totals just
+    // summed), then the lanes before
+    uint32_t mine = 0;
 #pragma unroll
-      for (int f = 0; f < 4; ++f) c03 += b <= f ? 1ull << (16 * f) : 0ull;
-#pragma unroll
-      for (int f = 4; f < NUC_FLOORS; ++f) c46 += b <= f ? 1ull << (16 * (f - 4)) : 0ull;
-      m4 += b <= 4 ? W[e] : 0u;
-      m5 += b <= 5 ? W[e] : 0u;
-      m6 += W[e];
-    }
-    // (warp totals of a field <= 256, row totals <= 32768)
-    auto add16 = [&](uint64_t v) {
-      return ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 32)) << 32) |
-             __reduce_add_sync(0xffffffffu, (uint32_t)v);
-    };
-    uint64_t t[ACC_WORDS] = {add16(c03), add16(c46), warp_total(m4), warp_total(m5), warp_total(m6)};
-    const int buf = rw.ph & 1;
-    rw.sum<ACC_WORDS>(t);
-    const unsigned long long *warps = rw.slots->w[buf], *ctas = rw.slots->c[buf];
-    int N[NUC_FLOORS];
-#pragma unroll
-    for (int f = 0; f < NUC_FLOORS; ++f) N[f] = (int)(((f < 4 ? t[0] : t[1]) >> (16 * (f & 3))) & 0xFFFF);
-    const uint64_t Sf[3] = {t[2], t[3], t[4]};
-    const uint64_t S_all = Sf[2];
-    uint64_t thr_all = 0;
-    if (!topk) {
-      const uint64_t prod = (uint64_t)p.p_fixed * S_all;
-      thr_all = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-    }
-    // the highest floor whose elements provably hold the candidates (top-k) or the kept prefix
-    int f = -1;
-#pragma unroll
-    for (int i = 0; i < NUC_FLOORS; ++i) {
-      const bool holds = topk ? (N[i] >= p.top_k || N[i] == N[6]) : (i >= 4 && Sf[i - 4] >= thr_all);
-      if (f < 0 && N[i] <= NUC_LIST_MAX && holds) f = i;
-    }
-    if (N[6] == 0) return 0;   // every weight 0 (all-NaN row): the lowest candidate, id 0
-    if (f >= 0) {
-      int nf = 0;
-#pragma unroll
-      for (int i = 0; i < NUC_FLOORS; ++i) nf = i == f ? N[i] : nf;
-      // this thread's place in the list: the CTAs and warps before (from the totals just
-      // summed), then the lanes before
-      const int word = f >> 2, sh = 16 * (f & 3);
-      uint64_t at = 0;
-      if (lane < rw.rank) at += (ctas[lane * ACC_WORDS + word] >> sh) & 0xFFFF;
-      if (lane < w) at += (warps[lane * ACC_WORDS + word] >> sh) & 0xFFFF;
-      at = warp_sum_u64(at);
-      uint32_t mine = 0;
-#pragma unroll
-      for (int e = 0; e < ACC_EPT; ++e) mine += nuc_bucket(W[e]) <= f;
-      uint32_t x = mine;
+    for (int e = 0; e < ACC_EPT; ++e) mine += own[e * ACC_THREADS] >= floor_w;
+    if (__any_sync(0xffffffffu, mine != 0)) {
+      const int word = f < 4 ? 2 : 0, sh = 16 * (f & 3);
+      uint32_t at = 0, x = mine;
+      if (lane < rw.rank) at += (uint32_t)(rw.slots->c[buf][word * ACC_CS + lane] >> sh) & 0xFFFFu;
+      if (lane < w) at += (uint32_t)(rw.slots->w[buf][word * ACC_WARPS + lane] >> sh) & 0xFFFFu;
+      at = __reduce_add_sync(0xffffffffu, at);
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
       }
-      uint32_t dst = mapa_shared(smem_u32(&L.key[0]), 0) + ((uint32_t)at + x - mine) * 8;
-#pragma unroll
-      for (int e = 0; e < ACC_EPT; ++e)
-        if (nuc_bucket(W[e]) <= f) {
-          st_dsmem_u64(dst, nuc_key(W[e], base + e));
+      uint32_t dst = mapa_shared(smem_u32(&L.key[0]), 0) + (at + x - mine) * 8;
+#pragma unroll 1
+      for (int e = 0; mine; ++e) {
+        const uint32_t W = own[e * ACC_THREADS];
+        if (W >= floor_w) {
+          st_dsmem_u64(dst, (uint64_t)W << 32 | (uint32_t)(base + e));
           dst += 8;
+          --mine;
         }
-      cluster_sync_all();   // the list is complete
-      if (rw.rank) return 0;
-      // a kept set (or top-k) of at most 32 on the lanes of one warp when that is cheap: a
-      // small top-k, or a short list; otherwise, or when it does not apply, the sorted list
-      if ((topk && p.top_k <= 32) || nf <= 64) {
-        if (w == 0) {
-          const int pick = list_small(p, L, nf, S_all, topk, rnd);
-          if (lane == 0) L.pick = pick;
-        }
-        __syncthreads();
-        const int pick = L.pick;
-        if (pick >= 0) return pick;
-        __syncthreads();   // L.pick is written again
       }
-      return list_sorted_select(p, L, nf, S_all, rnd, red);
     }
+    cluster_sync_all();   // the list is complete
+    if (rw.rank) return 0;
+    uint32_t x;
+    uint64_t ties, mass;
+    kept_cut<false>(
+        p, L, [&](auto f) { for (int i = tid; i < nf; i += ACC_THREADS) f((uint32_t)(L.key[i] >> 32)); },
+        [&](uint64_t v) { return block_sum_u64(v, red); }, S_all, k, red, rw, x, ties, mass);
+    // 7. the first kept id (ascending) whose inclusive cumulative weight exceeds tau
+    const uint64_t tau = __umul64hi(rnd, mass);
+    const int per = (nf + ACC_THREADS - 1) / ACC_THREADS, i0 = min(tid * per, nf), i1 = min(i0 + per, nf);
+    uint64_t sum = 0;
+    for (int i = i0; i < i1; ++i) sum += kept_word((uint32_t)(L.key[i] >> 32), x);
+    uint64_t word = block_exscan_u64(sum, red);
+    if (kept_mass(word, x, ties) <= tau && kept_mass(word + sum, x, ties) > tau) {
+      int i = i0 - 1;
+      do word += kept_word((uint32_t)(L.key[++i] >> 32), x);
+      while (kept_mass(word, x, ties) <= tau);
+      L.pick = (int)(uint32_t)L.key[i];
+    }
+    __syncthreads();
+    return L.pick;
   }
 
-  // ---- the row-wide path over all ids
-  Cut c;
-  c.xk = 0;
-  c.idk = 0x7FFFFFFF;
-  c.xp = 0;
-  c.idp = 0x7FFFFFFF;
-  // 4. top-k candidates
-  if (topk) {
-    c.xk = search_threshold<P_GE, true>(W, base, c, (uint64_t)p.top_k, rw);
-    const uint64_t above = row_sum<P_GT, true>(W, base, c, c.xk, rw);
-    c.idk = nth_id<P_EQ>(W, base, c, c.xk, (uint64_t)p.top_k - above, rw);
-  }
-  // 5. top-p over the candidates: thr = ceil(P * S / 2^24), P <= 2^24, S < 2^40
-  const uint64_t S = row_sum<P_CAND, false>(W, base, c, 0, rw);
-  const uint64_t prod = (uint64_t)p.p_fixed * S;
-  const uint64_t thr = (prod >> 24) + ((prod & 0xFFFFFFull) ? 1 : 0);
-  c.xp = search_threshold<P_CAND_GE, false>(W, base, c, thr, rw);
-  uint64_t ab[2] = {warp_total(lsum<P_CAND_GT, false>(W, base, c, c.xp)),
-                    warp_total(lsum<P_CAND_GT, true>(W, base, c, c.xp))};
-  rw.sum<2>(ab);
-  uint64_t ties = thr > ab[0] ? (thr - ab[0] + c.xp - 1) / c.xp : 0;
-  if (ab[1] == 0 && ties == 0) ties = 1;
-  c.idp = ties == 0 ? -1 : nth_id<P_CAND_EQ>(W, base, c, c.xp, ties, rw);
-  // 7. the first kept id (ascending) whose inclusive cumulative weight exceeds tau
-  const uint32_t mine = lsum<P_KEPT, false>(W, base, c, 0);
-  const uint64_t Sk = rw.sum(warp_total(mine));
-  const uint64_t tau = __umul64hi(rnd, Sk);
-  const uint64_t before = rw.exscan(mine);
+  // ---- the same over all ids
+  uint32_t x;
+  uint64_t ties, mass;
+  auto each = [&](auto f) { for (int e = 0; e < ACC_EPT; ++e) f(own[e * ACC_THREADS]); };
+  kept_cut<true>(
+      p, L, each, [&](uint64_t v) { return rw.sum(warp_sum_u64(v)); }, S_all, k, red, rw, x, ties, mass);
+  const uint64_t tau = __umul64hi(rnd, mass);
+  uint64_t sum = 0;
+  each([&](uint32_t W) { sum += kept_word(W, x); });
+  uint64_t word = rw.exscan(sum);
   uint32_t hit = 0;   // id + 1 in the one thread that holds it
-  if (before <= tau && before + mine > tau) {
-    uint64_t cum = before;
-#pragma unroll
-    for (int e = 0; e < ACC_EPT; ++e) {
-      if (pred<P_KEPT>(W[e], base + e, c, 0)) {
-        cum += W[e];
-        if (cum > tau && !hit) hit = base + e + 1;
-      }
-    }
+  if (kept_mass(word, x, ties) <= tau && kept_mass(word + sum, x, ties) > tau) {
+    int e = -1;
+    do word += kept_word(own[++e * ACC_THREADS], x);
+    while (kept_mass(word, x, ties) <= tau);
+    hit = base + e + 1;
   }
   return (int)rw.sum(warp_total(hit)) - 1;
 }
@@ -732,8 +550,11 @@ __device__ __forceinline__ int tree_depth(const int* par, int j, uint32_t* err) 
   return d;
 }
 
-__global__ void __launch_bounds__(ACC_THREADS) accept_kernel(const AcceptParams p) {
-  extern __shared__ __align__(16) uint8_t acc_smem[];   // NucList (nucleus only)
+// (greedy apart: 4.97 us instead of 5.19 with 24 rows; four CTAs an SM instead of two: 64 rows 22.5
+// instead of 24.2 us, greedy 6.3 instead of 7.3)
+template <bool NUCLEUS>
+__global__ void __launch_bounds__(ACC_THREADS, 4) accept_kernel(const AcceptParams p) {
+  extern __shared__ __align__(16) uint8_t acc_smem[];   // NucSmem (nucleus only)
   __shared__ AccSlots slots;
   __shared__ uint64_t red[ACC_WARPS];
   cluster_arrive_thread();
@@ -744,12 +565,12 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_kernel(const AcceptParams 
   const int j = blockIdx.x / p.cs, sl = blockIdx.y, s = p.seq0 + sl;
   const float* row = p.logits + (size_t)(sl * p.q + j) * p.V;
   int t;
-  if (p.temperature <= 0.f) {
+  if constexpr (!NUCLEUS) {
     t = row_argmax(row, p.V, p.err, rw);
   } else {
     // the produced token's position: one past the row's own (len + j, or len + depth(j))
     const int position = __ldcg(p.len + s) + (p.parent ? tree_depth(p.parent + sl * p.q, j, nullptr) : j) + 1;
-    t = row_nucleus(p, row, position, s, red, rw, *reinterpret_cast<NucList*>(acc_smem));
+    t = row_nucleus(p, row, position, s, red, rw, *reinterpret_cast<NucSmem*>(acc_smem));
   }
   // the last row of a sequence (per-sequence counter) verifies and commits
   if (rw.rank || threadIdx.x) return;
@@ -822,13 +643,13 @@ cudaError_t launch_accept(const AcceptParams& p0, cudaStream_t st, bool pdl) {
   p.cs = std::min(ACC_CS, (p.V + ACC_SPAN - 1) / ACC_SPAN);   // (a larger vocabulary is greedy only)
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = make_cfg(dim3(p.q * p.cs, p.nb), dim3(ACC_THREADS), st, pdl, attr);
-  cfg.dynamicSmemBytes = p.temperature > 0.f ? sizeof(NucList) : 0;
+  cfg.dynamicSmemBytes = p.temperature > 0.f ? sizeof(NucSmem) : 0;
   attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
   attr[cfg.numAttrs].val.clusterDim.x = p.cs;
   attr[cfg.numAttrs].val.clusterDim.y = 1;
   attr[cfg.numAttrs].val.clusterDim.z = 1;
   ++cfg.numAttrs;
-  return cudaLaunchKernelEx(&cfg, accept_kernel, p);
+  return p.temperature > 0.f ? cudaLaunchKernelEx(&cfg, accept_kernel<true>, p) : cudaLaunchKernelEx(&cfg, accept_kernel<false>, p);
 }
 
 // ---- RMSNorm into the GEMM operand ------------------------------------------------------
@@ -1092,8 +913,9 @@ __global__ void exp_kernel(const float* in, float* out, int n) {
 }
 
 cudaError_t accept_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NucList));
-  if (e == cudaSuccess) e = prefer_shared(accept_kernel);
+  cudaError_t e = cudaFuncSetAttribute(accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NucSmem));
+  if (e == cudaSuccess) e = prefer_shared(accept_kernel<true>);
+  if (e == cudaSuccess) e = prefer_shared(accept_kernel<false>);
   if (e == cudaSuccess) e = prefer_shared(rmsnorm_kernel);
   if (e == cudaSuccess) e = prefer_shared(split_kernel);
   if (e == cudaSuccess) e = prefer_shared(build_block_kernel);

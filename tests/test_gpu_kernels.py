@@ -471,3 +471,24 @@ def test_attention_grids(sd, b, q, H, hd):
         ref = torch.einsum("hqk,hkd->qhd", sc.masked_fill(~seen, float("-inf")).softmax(-1), v[s, :, :n + q].double())
         # operands as bf16 hi + lo (2^-16 relative), fp32 sums, outputs of order one
         assert (out[s * q:(s + 1) * q].double().view(q, H, hd) - ref).abs().max().item() <= 2e-5
+
+
+@pytest.mark.parametrize("T,top_p,top_k", [(1.0, 0.95, 0), (1.0, 0.9, 5000), (1.5, 0.0, 0), (0.2, 1.0, 20000), (3.0, 0.95, 4097)])
+def test_accept_nucleus_cuts(sd, T, top_p, top_k):
+    """Cuts by digits on 32016 ids, on the list and over the whole row: equal weights across the cut,
+    weights that differ in one digit only, one heavy weight, infinities, a flat row."""
+    V, b, q = 32016, 1, 7
+    big = synth.ModelShape("v32k", 1, 256, 4, 64, 688, V, 32011)
+    ctx = sd.Context(big, synth.make_model(big, seed=0, device="cuda"), max_position=4096)
+    g = torch.Generator().manual_seed(17)
+    lg = torch.randn(b * q, V, generator=g)
+    lg[1] = (lg[1] * 4).round() / 4
+    lg[2] = -torch.arange(V).float() * 2.0 ** -20          # 2^24 (1 - id / 2^20)
+    lg[3, 777] = 40.0
+    lg[4, :9000] = float("-inf")
+    lg[5] = 0.0
+    lg[6, 31000:] = float("inf")
+    _, rout = _oracle_accept(lg.numpy(), [0] * (b * q), b, q, 0, [60], T, top_p, 9, top_k)
+    acc, out, flags, _ = _run_accept(ctx, lg.cuda(), torch.zeros(b * q, dtype=torch.int32, device="cuda"), b, q, 0,
+                                     [60], T, top_p, 9, top_k)
+    assert out == rout
