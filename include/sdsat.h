@@ -341,10 +341,10 @@ SDSAT_API sdsat_status sdsat_accept_pipelined(sdsat_ctx* ctx, sdsat_kv* kv, cons
 
 /* Run n prompt tokens of sequence `seq` through the model and commit them
  * (len[seq] += n): the step before the decode loop (Sec. 2.1.1 starts from a prompt
- * y_1 .. y_n already in the context; the paper gives the prefill no further detail).  Chunks of up to
- * SDSAT_MAX_ROWS positions go through one block forward each (the weights stream
- * once per chunk), position i attending to every earlier position; a tail shorter
- * than SDSAT_MAX_Q rows runs as one ordinary block.  No logits are produced.
+ * y_1 .. y_n already in the context; the paper gives the prefill no further detail).  Equal chunks of
+ * at most 4096 positions (at most max_position rounded up to 128) go through the layers one
+ * after the other (the weights stream once per chunk), position i attending to every earlier
+ * position.  No logits are produced.
  * Errors: EINVAL (null pointer, seq outside the KV batch, n < 0), ECAPACITY
  * (n > max_len); device bit CAPACITY if len[seq] + n > max_len. */
 SDSAT_API sdsat_status sdsat_prefill(sdsat_ctx* ctx, sdsat_kv* kv, int seq, const int32_t* tokens_dev, int n);
@@ -393,7 +393,8 @@ SDSAT_API sdsat_status sdsat_debug_workspace(sdsat_ctx* ctx, int which, int rows
  * each CTA taking several pairs.  max_clusters[c] (c = 1..16, host array of 17 entries,
  * [0] unused) = the most clusters of c CTAs the device holds at once, as
  * cudaOccupancyMaxActiveClusters reports it for the attention kernel.  The launches also cap
- * cs at the cache's 64-slot units.  Errors: EINVAL. */
+ * cs at the cache's 64-slot units, and sdsat_op_attention takes the next smaller grid for caches
+ * of at most 8 units per CTA where fewer than 6 further clusters of cs fit.  Errors: EINVAL. */
 SDSAT_API sdsat_status sdsat_attention_grid(int pairs, const int32_t* max_clusters, int cs_cap, int num_sms,
                                             int* cs, int* nclusters);
 
@@ -453,7 +454,7 @@ SDSAT_API sdsat_status sdsat_profile_end(sdsat_ctx* ctx, sdsat_kernel_stat* out,
 
 /* Device timeline trace (does not serialise launches): between sdsat_trace_begin and
  * sdsat_trace_end, thread 0 of every CTA of the block forward's GEMM and attention kernels
- * appends one record of SDSAT_TRACE_WORDS uint64:
+ * (and of the prefill's GEMM) appends one record of SDSAT_TRACE_WORDS uint64:
  *   [0] tag << 32 | block index, tag = kernel class << 24 | launch sequence number
  *       (sdsat_kernel_class_name names a class);
  *   [1] flags << 32 | SM id;

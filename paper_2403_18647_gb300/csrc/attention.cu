@@ -52,6 +52,9 @@ constexpr int ATT_PREFETCH = 4;   // units past the ring requested into L2 ahead
 // the later units' missed L2 hits than they gain (attention 13.7 -> 15.1 us with 1)
 constexpr int ATT_LONG_SLICE = 7;
 constexpr size_t ATT_TWO_PER_SM = 96 * 1024;   // dynamic shared memory of which only two fit on an SM
+constexpr int ATT_NEXT_CLUSTERS = 6;    // attention launches in a row: clusters that the GPCs have to hold beside this grid's
+constexpr int ATT_SHORT_SLICE = 8;      // ... for caches of at most this many units per CTA
+constexpr int ATT_MERGE = 6;            // partials that one lane merges, at most
 constexpr int ATT_SPARE_CLUSTERS = 8;   // room left for this many more clusters (measured: 7B/13B shapes, b = 1, 4)
 
 template <int HD, int QT = 2>
@@ -487,22 +490,24 @@ __global__ void __launch_bounds__(128, 3) attention_kernel(const __grid_constant
     // after its last remote loads and waits only at the end: the barrier's round trip
     // overlaps the merge arithmetic and the output stores.
     // Few threads have an item (18 of 128 with 11 CTAs), and this code runs once per launch and is
-    // fetched cold, so G lanes share an item, each with at most four of the cs partials: one
+    // fetched cold, so G lanes share an item, each with at most six of the cs partials: one
     // thread with an unrolled loop over 16 took 1.5 us from the loads to the stores with 11 CTAs.
+    // With 9 to 12 CTAs and more than 32 items (10 rows and up) two lanes and one pass instead of
+    // four lanes and two: 16 rows, context 2048 14.6 -> 14.0 us (7B, four layers: 432.8 -> 430.8).
     bool arrived = false;
     {
-      const int G = CS <= 4 ? 1 : (CS <= 8 ? 2 : 4), gl = tid & (G - 1), per = 128 / G;
       const int items = q * D4, i0 = items * rank / CS, i1 = items * (rank + 1) / CS;
+      const int G = CS <= 4 ? 1 : (CS <= 8 || (CS <= 2 * ATT_MERGE && i1 - i0 > 32) ? 2 : 4), gl = tid & (G - 1), per = 128 / G;
       const int passes = (i1 - i0 + per - 1) / per;
 #pragma unroll 1
       for (int pass = 0; pass < passes; ++pass) {
         const int mine = i0 + pass * per + tid / G, it = min(mine, i1 - 1);   // (every lane shuffles)
         const int j = it / D4, d4 = it - j * D4;
         const uint32_t a_ml = smem_u32(pml + 2 * j), a_o = smem_u32(po + j * HD + 4 * d4);
-        float2 ml[4];
-        float4 ov[4];
+        float2 ml[ATT_MERGE];
+        float4 ov[ATT_MERGE];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < ATT_MERGE; ++u) {
           const int r = gl + u * G;
           ml[u] = make_float2(-INFINITY, 0.f);
           ov[u] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -515,12 +520,14 @@ __global__ void __launch_bounds__(128, 3) attention_kernel(const __grid_constant
           cluster_arrive_thread();
           arrived = true;
         }
-        float mx = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x));
+        float mx = ml[0].x;
+#pragma unroll
+        for (int u = 1; u < ATT_MERGE; ++u) mx = fmaxf(mx, ml[u].x);
         for (int o = 1; o < G; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float L = 0.f;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < ATT_MERGE; ++u) {
           const float w = (ml[u].x == -INFINITY) ? 0.f : __expf(ml[u].x - mx);
           L += w * ml[u].y;
           a.x += w * ov[u].x;
@@ -649,9 +656,19 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   // With head dimension 64 two more spare clusters (32 heads, context 8192: 11 CTAs 20.3 us, 10
   // CTAs 18.4; context 2000 10.1 and 8.5; 40 heads keep 9).
   const int* maxc = g_att_clusters[p.hd == 128][p.q > 8];
-  int cap = std::min(g_att_cs_cap, (p.cap + ATT_UNIT - 1) / ATT_UNIT);
+  const int units = (p.cap + ATT_UNIT - 1) / ATT_UNIT;
+  int cap = std::min(g_att_cs_cap, units);
   if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (p.nb * p.H + ATT_SPARE_CLUSTERS + 2)));
   attention_grid(p.nb * p.H, maxc, cap, num_sms, &p.cs, &p.nclusters);
+  // Attention after attention: the next launch's clusters start early only where a GPC has room
+  // for a whole one, so with short slices at least ATT_NEXT_CLUSTERS more have to fit (36 of 11
+  // CTAs do, 43 of 10, 46 of 9).  32 heads, calls in a row, 11 CTAs -> 10: 6 rows, context 1000
+  // 9.4 -> 7.6 us, 2048 12.6 -> 10.7, 4096 18.7 -> 16.9; 16 rows 12.4 -> 9.6, 16.0 -> 14.0, 24.5 ->
+  // 21.9.  Longer slices gain more from the eleventh CTA (11 rows, 16384: 56.9 against 61.2), and
+  // so do 40 heads (9 CTAs, 6 more fit; 2048: 11.8 against 12.7) and the step, where GEMMs
+  // surround the launch (7B, four layers, context 2048: 386.8 against 391.3).
+  if (p.alone && p.cs > 2 && units <= ATT_SHORT_SLICE * p.cs && maxc[p.cs] < p.nb * p.H + ATT_NEXT_CLUSTERS)
+    attention_grid(p.nb * p.H, maxc, p.cs - 1, num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);

@@ -2,9 +2,9 @@
 //
 // Every projection of the block forward (QKV, O, gate/up, down, LM head) is
 // Y[M, N] = X[M, K] W[N, K]^T with M = b*q rows, up to 32 here (blocks of more rows than
-// GEMM_WIDE_ROWS run on the tiled GEMM of prefill.cu), and a weight matrix of 30-330 MB.  The weights are read once per step, so the kernel is bound by
-// HBM bandwidth (decoding is memory-bandwidth bound, Sec. 1; the loop time is
-// almost flat in k, Sec. 3.4.1).  Design:
+// GEMM_WIDE_ROWS run on the tiled GEMM of prefill.cu), and a weight matrix of 30-330 MB.  The
+// weights are read once per step, so the kernel is bound by HBM bandwidth (decoding is
+// memory-bandwidth bound, Sec. 1; the loop time is almost flat in k, Sec. 3.4.1).  Design:
 //
 //  * Persistent grid of P CTAs; the (128-row tile, 64-wide K chunk) work units
 //    are split evenly in one flat range ("stream-K"), so every CTA streams the
