@@ -125,8 +125,9 @@ constexpr int GEMM_MPADS[] = {8, 16, 24, 32};
 // Blocks of more rows than this run on the tiled GEMM of prefill.cu (64-row tiles).  The skinny
 // GEMM's split-K tail grows with the rows: its last contributors summed 10 parts of 32 KB and
 // ran a 64-row epilogue in 13 us.  Four 7B layers and LM head, us per block step, skinny -> tiled:
-// 26 rows 481 -> 505, 30 rows 544 -> 533, 36 rows 576 -> 517, 64 rows 642 -> 527; 13B, 64 rows 857 -> 724.
-constexpr int GEMM_WIDE_ROWS = 28;
+// 36 rows 576 -> 517, 64 rows 642 -> 527; 13B, 64 rows 857 -> 724.  26 rows 481 -> 505; 30 rows of
+// 2 or 5 short sequences 486 -> 489 and 486 -> 497, 32 rows, context 1000: 535 -> 526.
+constexpr int GEMM_WIDE_ROWS = 32;
 cudaError_t gemm_prepare();           // set smem attributes (idempotent)
 cudaError_t launch_gemm(GemmParams& p, int num_sms, cudaStream_t st, bool pdl);
 

@@ -1178,12 +1178,21 @@ sdsat_status sdsat_get_error(sdsat_ctx* c, uint32_t* flags) {
   return f ? SDSAT_EDEVICE : SDSAT_OK;
 }
 
+// A plain product runs on the tiled GEMM above GEMM_WIDE_ROWS rows, and from 25 rows (the skinny
+// GEMM pads them to 32) where its 256-row tiles either are few or fill the CTA pairs.  In between
+// every tile is split in two or three and a second kernel adds them up: 30 rows, K 4096, us skinny /
+// tiled: N 2048 18.6 / 15.4, 4096 17.2 / 16.5, 6144 18.4 / 18.9, 12288 24.7 / 26.8, 15360 29.0 /
+// 30.6, 17408 31.1 / 29.7, 22016 41.1 / 37.0, 32016 (K 5120) 63.9 / 59.1.
+static bool op_gemm_tiled(int M, int N, int num_sms) {
+  const int tiles = (N + 255) / 256, pairs = num_sms / 2;
+  return M > GEMM_WIDE_ROWS || (gemm_mpad(M) == 32 && (4 * tiles <= pairs || 8 * tiles >= 7 * pairs));
+}
+
 sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const void* w_dev, int N, float* y_dev) {
   if (!c || !x_dev || !y_dev || !aligned16(w_dev) || !aligned16(x_dev)) return SDSAT_EINVAL;
   if (M < 1 || M > OP_MAX_M || K < 8 || K % 8 || K > OP_MAX_K || N < 1 || (N + 127) / 128 > MAX_GEMM_TILES)
     return SDSAT_EINVAL;
-  if (M > GEMM_WIDE_ROWS) {
-    // the prefill GEMM (tiles of 128 weight rows x 128 positions)
+  if (op_gemm_tiled(M, N, c->num_sms)) {
     const int rows = (M + 127) / 128 * 128;   // <= OP_MAX_M rows of the operand scratch
     PfGemmParams g;
     std::memset(&g, 0, sizeof(g));

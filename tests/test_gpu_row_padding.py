@@ -1,5 +1,5 @@
 """Block forwards whose row count lies at the edges of the GEMMs they run on (operand padding to
-8, 16, 24 and 32 rows, and from 29 rows the tiled GEMM): every sequence of a batch against the
+8, 16, 24 and 32 rows, and from 33 rows the tiled GEMM): every sequence of a batch against the
 same sequence alone: logits, the last layer's workspaces and the K / V rows written."""
 import pytest
 import torch
@@ -67,9 +67,9 @@ def test_tree_batch_equals_single_sequences(ctx, b, q):
 
 def test_wide_block_past_the_capacity(ctx):
     """Rows past the KV capacity on the tiled GEMM: flagged, not written, the others as usual."""
-    b, q = 2, 16
+    b, q = 3, 16
     kv = ctx.kv(b, 100)
-    ctx.kv_commit(kv, torch.tensor([100 - q, 100 - 5], dtype=torch.int32, device="cuda"), b)
+    ctx.kv_commit(kv, torch.tensor([100 - q, 100 - 5, 0], dtype=torch.int32, device="cuda"), b)
     toks = synth.uniform_ids(5, 1, b * q, ctx.shape.vocab, device="cuda")
     lg = torch.empty(b * q, ctx.shape.vocab, device="cuda")
     ctx.block_forward(kv, toks, lg, b, q)
@@ -80,9 +80,10 @@ def test_wide_block_past_the_capacity(ctx):
     assert (k.float().abs().sum(dim=(0, 2))[:95] == 0).all() and (k.float().abs().sum(dim=(0, 2))[95:] > 0).all()
 
 
-@pytest.mark.parametrize("M", [1, 8, 9, 16, 17, 24, 25, 28, 29, 32, 33, 64])
-def test_gemm_row_padding(ctx, M):
-    K, N = 4096, 1500   # split tiles, ragged N
+@pytest.mark.parametrize("M,N", [(M, 1500) for M in (1, 8, 9, 16, 17, 24, 25, 28, 29, 32, 33, 64)] +
+                         [(M, N) for M in (25, 32) for N in (4864, 4865, 16896, 16897)])
+def test_gemm_row_padding(ctx, M, N):
+    K = 4096   # split tiles, ragged N
     x, w = synth.normal_f32(12, M, (M, K), 1.0, device="cuda"), synth.normal_bf16(12, 1, (N, K), 0.02, device="cuda")
     y = torch.full((M, N), float("nan"), device="cuda")
     ctx.op_gemm(x, w, y)
