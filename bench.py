@@ -59,13 +59,13 @@ WORKLOADS = {
 
 
 # DRAM bytes (read + write) per algorithmic byte of the skinny GEMM, from one ncu capture
-# (--set full) of a gate/up-sized launch: K 4096, N 22016, M 6 -> 186.01 MB of traffic for
+# of a gate/up-sized launch: K 4096, N 22016, M 6 -> 185.91 MB of traffic for
 # 180.98 MB of weights + operand + output.  The bench line applies it to the step's gate/up
 # launch (the roofline's kernel).  GEMM_TRAFFIC_CURRENT says whether that capture was taken of
 # the kernel as it is now; while it is False the line reports traffic null.
-GEMM_TRAFFIC_RATIO = 186.01 / 180.98
+GEMM_TRAFFIC_RATIO = 185.91 / 180.98
 GEMM_TRAFFIC_CURRENT = True
-GEMM_TRAFFIC_SOURCE = ("ncu dram__bytes_read+write of one K=4096 N=22016 M=6 launch (186.01 MB for 180.98 MB "
+GEMM_TRAFFIC_SOURCE = ("ncu dram__bytes_read+write of one K=4096 N=22016 M=6 launch (185.91 MB for 180.98 MB "
                        "algorithmic, profiles/gemm_gateup_4096x22016_m6.md) times the gate/up launch's algorithmic "
                        "bytes; bytes per launch")
 
@@ -644,7 +644,7 @@ def run_ours(args, wl, rank, world):
     return r, out
 
 
-def prefill_line(r, chunk=512):
+def prefill_line(r, chunk=4096):
     """The prompt prefill (not part of the timed decode steps): tokens/s and its tensor-core
     rate.  FLOPs = 2 x positions x decoder-layer weights (the projections) + the causal
     attention products 2 x 2 x n^2/2 x H x hd per layer (algorithmic; the hi + lo operand
@@ -658,8 +658,8 @@ def prefill_line(r, chunk=512):
     tf = flops / sec / 1e12
     return {"tokens": n, "ms": round(r.prefill_ms, 3), "tokens_per_s": round(n / sec, 1), "chunk_rows": chunk,
             "tflops": round(tf, 1), "frac_of_measured_bf16": round(tf / tpk, 4), "peak": tpk, "peak_source": kind,
-            "note": "tiled tcgen05 GEMM (128 weight rows x 128 positions), causal flash attention over "
-                    "64-position blocks"}
+            "note": "tiled tcgen05 GEMM (256 weight rows x 128 positions on a CTA pair), causal tcgen05 flash "
+                    "attention; equal chunks of at most chunk_rows positions"}
 
 
 def step_calls(r):

@@ -12,9 +12,10 @@
 // Work: the grid is nclusters thread-block clusters of cs CTAs, all resident
 // at once (launch_attention picks the largest cs <= ATT_CS_MAX for which one
 // cluster per (sequence, head) pair fits on the GPU with room to spare; else
-// cs = 1 and each CTA takes several pairs).  Three CTAs fit on an SM.  Cluster c takes the pairs c, c + nclusters, ...; the
-// nu units of ATT_UNIT = 64 consecutive slots of a pair are split over the
-// cluster's CTAs as [r*nu/cs, (r+1)*nu/cs) for CTA rank r.  One thread keeps a
+// cs = 1 and each CTA takes several pairs).  Three CTAs fit on an SM.  Cluster c
+// takes the pairs c, c + nclusters, ...; the nu units of ATT_UNIT = 64
+// consecutive slots of a pair are split over the cluster's CTAs as
+// [r*nu/cs, (r+1)*nu/cs) for CTA rank r.  One thread keeps a
 // two-stage ring of K and V tiles (TMA, boxes of 64 dims x 64 rows, 128-byte
 // swizzle) full, walking the CTA's units pair by pair; tiles made of committed
 // slots only are requested before the QKV projection has finished, and the
@@ -672,8 +673,9 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
-  // Single CTAs that fit two to an SM: room for no third, or some SMs get three and others one
-  // (240 pairs, 10 rows, context 1000: 39.2 us against 32.9; 7 sequences of 4 rows, 32 heads, context 3000: 82 against 65).
+  // Single CTAs that fit two to an SM: room for no third, or some SMs get three and others one (240
+  // pairs, 10 rows, context 1000: 39.2 us against 32.9; 7 sequences of 4 rows, 32 heads, context
+  // 3000: 82 against 65).
   cfg.dynamicSmemBytes = attention_smem_bytes(p.hd, p.q);
   if (p.cs == 1 && p.nclusters <= 2 * num_sms)
     cfg.dynamicSmemBytes = std::max<size_t>(cfg.dynamicSmemBytes, ATT_TWO_PER_SM);

@@ -175,7 +175,7 @@ def accept_env(sd):
 
 
 def _run_accept(ctx, logits, drafts, b, q, n_verify, lens, temperature=0.0, top_p=1.0, seed=0, top_k=0):
-    kv = ctx.kv(b, min(4000, ctx.cfg.max_position))
+    kv = ctx.kv(b, 4000)
     ln = torch.tensor(lens, dtype=torch.int32, device="cuda")
     ctx.kv_commit(kv, ln, b)
     acc = torch.empty(b, dtype=torch.int32, device="cuda")
@@ -425,7 +425,7 @@ def test_accept_vocabulary_edges(sd, V):
 def test_argmax_signed_zero_and_minus_infinity(sd):
     """-0 ties with +0 (the lowest id wins), rows of -inf or NaN alone give id 0."""
     shape = synth.ModelShape("v9000", 1, 128, 1, 128, 256, 9000, 0)
-    ctx = sd.Context(shape, None, max_position=64)
+    ctx = sd.Context(shape, None, max_position=4096)
     lg = torch.full((3, 9000), -1.0, device="cuda")
     lg[0, 8000], lg[0, 5000] = 0.0, -0.0
     lg[1] = float("-inf")
