@@ -17,10 +17,9 @@
 // O is rescaled only when a row's maximum has grown by more than 2^8 since the last time
 // (exact: the reference value cancels in the division by the row's sum; P stays below 2^8).
 //
-// Measured, 32 heads x 128, us per launch: 2047 positions 91 (256 with mma.sync m16n8k16 on
-// 64-position blocks, whose K and V fragments each warp read from shared memory again),
-// 512 positions 23 (43), 99 positions 12.5 (20); 4095 positions in two chunks 322 (872),
-// 0.85 PFLOP/s executed.
+// Measured, 32 heads x 128, us per launch: 4095 positions 254 (872 with mma.sync m16n8k16 on
+// 64-position blocks, whose K and V fragments each warp read from shared memory again), 2047
+// 81 (256), 512 23 (43), 99 12.3 (20); at 4095 1.08 PFLOP/s executed.
 //
 // Warps 0-3: TMA (warp 0), MMA issue and TMEM (warp 1), two idle; warps 4-7 and 8-11: softmax
 // and output of tile 0 and 1.  Shared memory: Q 64 KB per tile, a ring of three 32 KB slots in
