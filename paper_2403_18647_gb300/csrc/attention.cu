@@ -657,10 +657,10 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   // With head dimension 64 two more spare clusters (32 heads, context 8192: 11 CTAs 20.3 us, 10
   // CTAs 18.4; context 2000 10.1 and 8.5; 40 heads keep 9).
   const int* maxc = g_att_clusters[p.hd == 128][p.q > 8];
-  const int units = (p.cap + ATT_UNIT - 1) / ATT_UNIT;
+  const int units = (p.cap + ATT_UNIT - 1) / ATT_UNIT, pairs = p.nb * p.H;
   int cap = std::min(g_att_cs_cap, units);
-  if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (p.nb * p.H + ATT_SPARE_CLUSTERS + 2)));
-  attention_grid(p.nb * p.H, maxc, cap, num_sms, &p.cs, &p.nclusters);
+  if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (pairs + ATT_SPARE_CLUSTERS + 2)));
+  attention_grid(pairs, maxc, cap, num_sms, &p.cs, &p.nclusters);
   // Attention after attention: the next launch's clusters start early only where a GPC has room
   // for a whole one, so with short slices at least ATT_NEXT_CLUSTERS more have to fit (36 of 11
   // CTAs do, 43 of 10, 46 of 9).  32 heads, calls in a row, 11 CTAs -> 10: 6 rows, context 1000
@@ -668,8 +668,14 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   // 21.9.  Longer slices gain more from the eleventh CTA (11 rows, 16384: 56.9 against 61.2), and
   // so do 40 heads (9 CTAs, 6 more fit; 2048: 11.8 against 12.7) and the step, where GEMMs
   // surround the launch (7B, four layers, context 2048: 386.8 against 391.3).
-  if (p.alone && p.cs > 2 && units <= ATT_SHORT_SLICE * p.cs && maxc[p.cs] < p.nb * p.H + ATT_NEXT_CLUSTERS)
-    attention_grid(p.nb * p.H, maxc, p.cs - 1, num_sms, &p.cs, &p.nclusters);
+  // In the step, a tenth more clusters than pairs have to fit: 80 pairs (13B, two sequences) need
+  // nearly every place that the QKV projection's CTAs leave for clusters of 5 (87 fit), and some of
+  // them enter late.  13B, four layers, 5 CTAs -> 4: 6 rows, context 1024 589.6 -> 571.7 us, 8 rows,
+  // 3000 662.9 -> 627.3, 14 rows, 1000 691 -> 654.5.  (32, 40, 64, 96, 120 and 128 pairs: 12 to 23 %
+  // more fit, and smaller clusters are no faster.)
+  const bool tight = p.alone ? units <= ATT_SHORT_SLICE * p.cs && maxc[p.cs] < pairs + ATT_NEXT_CLUSTERS
+                             : 10 * maxc[p.cs] < 11 * pairs;
+  if (tight && p.cs > 2) attention_grid(pairs, maxc, p.cs - 1, num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
