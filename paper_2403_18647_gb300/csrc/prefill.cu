@@ -26,10 +26,10 @@
 //
 // Epilogues: store; RoPE and the KV append (QKV); residual add (O and down projections), which
 // also emits the next RMSNorm's operand h * g and per-tile sums of h^2, as the decode GEMM
-// does, so that the consuming GEMM only scales its result by each position's factor; SiLU(gate)
-// * up as the down projection's bf16 hi + lo operand.  RMSNorm and RoPE as row kernels of their
-// own cost two more passes over the chunk's rows each (2047 positions: 34 us per RMSNorm, 59
-// us per RoPE + append).  Attention is prefill_attention.cu.
+// does, so that the consuming GEMM (QKV, gate/up, the LM head) only scales its result by each
+// position's factor; SiLU(gate) * up as the down projection's bf16 hi + lo operand.  RMSNorm and
+// RoPE as row kernels of their own cost two more passes over the chunk's rows each (2047
+// positions: 34 us per RMSNorm, 59 us per RoPE + append).  Attention is prefill_attention.cu.
 #include <algorithm>
 
 #include "common.cuh"
@@ -521,6 +521,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             const int n = 128 * wt + r;
             float* dst = p.out + (size_t)m0 * p.out_ld + n;
             const int cnt = n < p.N ? vr - c0 : 0;
+            if (p.ssq_in) {   // the LM head after a down projection that left its operand unscaled
+#pragma unroll
+              for (int j = 0; j < PF_CHUNK; ++j) y[j] *= inv[c0 + j];
+            }
 #pragma unroll
             for (int j = 0; j < PF_CHUNK; ++j)
               if (j < cnt) dst[(size_t)j * p.out_ld] = y[j];
@@ -565,6 +569,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             for (int k = 0; k < 8; ++k)
               if (k < cnt) {
                 float* d = dst + (size_t)k * p.out_ld;
+                if (p.ssq_in) {
+                  const float f = inv[c0 + w8 + k];
+                  v[k].x *= f, v[k].y *= f, v[k].z *= f, v[k].w *= f;
+                }
                 if (vec) {
                   *reinterpret_cast<float4*>(d) = v[k];
                 } else {
@@ -727,6 +735,14 @@ __device__ __forceinline__ float pf_block_sum(float v, float* red) {
   return v;
 }
 
+// RMSNorm factor of operand row m (1 when the operand is normalised already)
+__device__ __forceinline__ float pf_row_factor(const PfGemmParams& p, int m) {
+  if (!p.ssq_in) return 1.f;
+  float q = 0.f;
+  for (int t = 0; t < p.ssq_ld; ++t) q += __ldcg(p.ssq_in + (size_t)m * p.ssq_ld + t);
+  return 1.0f / sqrtf(q / (float)p.norm_dim + p.norm_eps);
+}
+
 // h += sum of the parts; with gain_next the next GEMM's operand RMSNorm(h)
 __global__ void __launch_bounds__(PF_FIN_ROW_THREADS) prefill_finish_resid_kernel(const __grid_constant__ PfGemmParams p) {
   constexpr int I = 64 * 128 / (4 * PF_FIN_ROW_THREADS);   // float4 of a row per thread: rows of up to 8192
@@ -770,7 +786,7 @@ __global__ void __launch_bounds__(PF_FIN_ROW_THREADS) prefill_finish_resid_kerne
   }
 }
 
-// out = sum of the parts (blockIdx.y: 2048 features)
+// out = sum of the parts, times the operand row's factor (blockIdx.y: 2048 features)
 __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_store_kernel(const __grid_constant__ PfGemmParams p) {
   pdl_wait();
   pdl_trigger();
@@ -786,6 +802,10 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_store_kernel(co
                            : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(y, t[u]);
+  }
+  if (p.ssq_in) {
+    const float s = pf_row_factor(p, m);
+    y.x *= s, y.y *= s, y.z *= s, y.w *= s;
   }
   float* dst = p.out + (size_t)m * p.out_ld + n;
   if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
@@ -803,12 +823,7 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_qkv_kernel(cons
   const int m = blockIdx.x, which = blockIdx.y, tok = p.tok, tb = m / tok, pos = m - tb * tok;
   const int R = p.rows_per_map, half = p.hd >> 1;
   const PfRow row_of(p, m, __ldcg(p.len + p.seq0));
-  float s = 1.f;
-  if (p.ssq_in) {
-    float q = 0.f;
-    for (int t = 0; t < p.ssq_ld; ++t) q += __ldcg(p.ssq_in + (size_t)m * p.ssq_ld + t);
-    s = 1.0f / sqrtf(q / (float)p.norm_dim + p.norm_eps);
-  }
+  const float s = pf_row_factor(p, m);
   if (threadIdx.x == 0 && which == 1) row_of.report(p);
   for (int x = 4 * (int)threadIdx.x; x < R / 2; x += 4 * PF_FIN_THREADS) {
     // four pairs of features: i .. i + 3 of a head and those half a head further
