@@ -394,9 +394,8 @@ SDSAT_API sdsat_status sdsat_debug_workspace(sdsat_ctx* ctx, int which, int rows
  * each CTA taking several pairs.  max_clusters[c] (c = 1..16, host array of 17 entries,
  * [0] unused) = the most clusters of c CTAs the device holds at once, as
  * cudaOccupancyMaxActiveClusters reports it for the attention kernel.  The launches also cap
- * cs at the cache's 64-slot units, and take the next smaller grid where few further clusters of
- * cs fit (block forward: less than a tenth of pairs; sdsat_op_attention: fewer than 6, for caches
- * of at most 8 units per CTA).  Errors: EINVAL. */
+ * cs at the cache's 64-slot units, and take the next smaller grid where fewer than a tenth more
+ * clusters of cs than pairs fit.  Errors: EINVAL. */
 SDSAT_API sdsat_status sdsat_attention_grid(int pairs, const int32_t* max_clusters, int cs_cap, int num_sms,
                                             int* cs, int* nclusters);
 

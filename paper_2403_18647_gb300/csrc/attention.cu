@@ -53,8 +53,6 @@ constexpr int ATT_PREFETCH = 4;   // units past the ring requested into L2 ahead
 // the later units' missed L2 hits than they gain (attention 13.7 -> 15.1 us with 1)
 constexpr int ATT_LONG_SLICE = 7;
 constexpr size_t ATT_TWO_PER_SM = 96 * 1024;   // dynamic shared memory of which only two fit on an SM
-constexpr int ATT_NEXT_CLUSTERS = 6;    // attention launches in a row: clusters that the GPCs have to hold beside this grid's
-constexpr int ATT_SHORT_SLICE = 8;      // ... for caches of at most this many units per CTA
 constexpr int ATT_MERGE = 6;            // partials that one lane merges, at most
 constexpr int ATT_SPARE_CLUSTERS = 8;   // room left for this many more clusters (measured: 7B/13B shapes, b = 1, 4)
 
@@ -135,15 +133,24 @@ __global__ void __launch_bounds__(128, 3) attention_kernel(const __grid_constant
   const int CS = p.cs, NC = p.nclusters;
   const int rank = (int)cluster_ctarank(), cl = (int)blockIdx.x / CS;
   const unsigned long long t_entry = p.trace.rec ? globaltimer_ns() : 0;
-  pdl_trigger();
+  // In a forward the O projection starts beside this kernel.  A launch by itself lets nothing
+  // start early: the clusters that a next attention launch could place beside this grid's (4 of 32
+  // with 32 heads) leave the others to enter late.  32 heads, calls in a row, us, with an early
+  // start -> without: 6 rows, context 500 6.9 -> 6.5, 1000 11.0 -> 8.7, 2048 13.4 -> 11.3; 16 rows,
+  // 2048 15.1 -> 13.9, 4096 24.8 -> 22.4; 40 heads, 4096 21.1 -> 21.4; 16384 the same.
+  if (!p.op) pdl_trigger();
   if (tid == 64) {   // the tensor maps into the TMA unit while the lengths are read
     tma_prefetch_desc(&p.kmap);
     tma_prefetch_desc(&p.vmap);
   }
 
-  // The committed lengths are final before this kernel can start: the block forward's
-  // first kernel (RMSNorm) lets its dependents launch only after every earlier kernel
-  // has completed.  Slots below them are not written during this forward either.
+  // In a block forward the committed lengths are final before this kernel can start: the
+  // forward's first kernel (RMSNorm) lets its dependents launch only after every earlier kernel
+  // has completed.  Slots below them are not written during this forward either.  Launched by
+  // itself there is no such kernel in front: whatever precedes it (a commit, which lets its
+  // dependents launch before it writes the lengths, a compaction of rows, the caller's own
+  // kernels) has to complete before a length or a row is read.
+  if (p.op) pdl_wait();
   if (tid < p.nb) {
     const int len = __ldcg(p.len + p.seq0 + tid);
     len_seq[tid] = len;
@@ -661,20 +668,13 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   int cap = std::min(g_att_cs_cap, units);
   if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (pairs + ATT_SPARE_CLUSTERS + 2)));
   attention_grid(pairs, maxc, cap, num_sms, &p.cs, &p.nclusters);
-  // Attention after attention: the next launch's clusters start early only where a GPC has room
-  // for a whole one, so with short slices at least ATT_NEXT_CLUSTERS more have to fit (36 of 11
-  // CTAs do, 43 of 10, 46 of 9).  32 heads, calls in a row, 11 CTAs -> 10: 6 rows, context 1000
-  // 9.4 -> 7.6 us, 2048 12.6 -> 10.7, 4096 18.7 -> 16.9; 16 rows 12.4 -> 9.6, 16.0 -> 14.0, 24.5 ->
-  // 21.9.  Longer slices gain more from the eleventh CTA (11 rows, 16384: 56.9 against 61.2), and
-  // so do 40 heads (9 CTAs, 6 more fit; 2048: 11.8 against 12.7) and the step, where GEMMs
-  // surround the launch (7B, four layers, context 2048: 386.8 against 391.3).
-  // In the step, a tenth more clusters than pairs have to fit: 80 pairs (13B, two sequences) need
-  // nearly every place that the QKV projection's CTAs leave for clusters of 5 (87 fit), and some of
-  // them enter late.  13B, four layers, 5 CTAs -> 4: 6 rows, context 1024 589.6 -> 571.7 us, 8 rows,
-  // 3000 662.9 -> 627.3, 14 rows, 1000 691 -> 654.5.  (32, 40, 64, 96, 120 and 128 pairs: 12 to 23 %
-  // more fit, and smaller clusters are no faster.)
-  const bool tight = p.alone ? units <= ATT_SHORT_SLICE * p.cs && maxc[p.cs] < pairs + ATT_NEXT_CLUSTERS
-                             : 10 * maxc[p.cs] < 11 * pairs;
+  // A tenth more clusters than pairs have to fit: 80 pairs (13B, two sequences) need nearly every
+  // place that the QKV projection's CTAs leave for clusters of 5 (87 fit), and some of them enter
+  // late.  13B, four layers, 5 CTAs -> 4: 6 rows, context 1024 589.6 -> 571.7 us, 8 rows, 3000 662.9
+  // -> 627.3, 14 rows, 1000 691 -> 654.5.  (32, 40, 64, 96, 120 and 128 pairs: 12 to 23 % more fit,
+  // and smaller clusters are no faster; with 32, 36 clusters of 11 fit, context 2048: 386.8 us for
+  // four 7B layers against 391.3 with 10.)
+  const bool tight = 10 * maxc[p.cs] < 11 * pairs;
   if (tight && p.cs > 2) attention_grid(pairs, maxc, p.cs - 1, num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);

@@ -149,7 +149,7 @@ struct AttnParams {
   int out_ld;
   __nv_bfloat16* out_hi;    // the same as bf16 hi + lo (the O projection's operand)
   __nv_bfloat16* out_lo;
-  bool alone;           // op_attention: the next kernel is likely another attention launch
+  bool op;              // launched by itself (op_attention), not between a forward's kernels
   int cs, nclusters;    // set by launch_attention: CTAs per cluster, clusters in the grid
   uint32_t* err;
   Trace trace;

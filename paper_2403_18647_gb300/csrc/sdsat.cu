@@ -1259,7 +1259,7 @@ sdsat_status sdsat_op_attention(sdsat_ctx* c, const float* q_dev, const void* k_
   a.out_hi = c->x_hi[X_ATTN];
   a.out_lo = c->x_lo[X_ATTN];
   a.err = c->err;
-  a.alone = true;
+  a.op = true;
   return timed(c, K_ATTENTION_OP, [&] { return launch_attention(a, c->num_sms, c->stream, c->pdl); }) == cudaSuccess
              ? SDSAT_OK
                                                                                                    : SDSAT_ECUDA;
