@@ -480,8 +480,9 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
         s_share[3 * i + 2] = unit_begin(lo, T, p.P, p.kc, p.snap) == t * p.kc ? 0 : 1;
       }
     }
-    // partials per bulk-copy round of the last reducer (the idle stage ring holds them)
-    const int red_per = max(1, (int)((S * C::STAGE_BYTES) / ((uint32_t)p.M * 512)));
+    // partials per bulk-copy round of the last reducer: the idle stage ring holds them, and each of
+    // the 128 epilogue threads copies one (one row of a tile with more contributors: 144 fit)
+    const int red_per = min(128, max(1, (int)((S * C::STAGE_BYTES) / ((uint32_t)p.M * 512))));
     int seg = 0, tile = tile_first - 1;
     long long g = g0;
     while (g < g1) {

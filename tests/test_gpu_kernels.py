@@ -93,6 +93,20 @@ def test_gemm_full_size_sampled(tiny_ctx, M, N, K):
     assert err <= 5e-5 * math.sqrt(K) * 0.02 + 1e-6 * np.abs(ref).max(), err
 
 
+@pytest.mark.parametrize("M,K,N", [(1, 8192, 128), (1, 8256, 128), (1, 9216, 1), (1, 9280, 128), (1, 32768, 128),
+                                   (1, 8256, 256), (1, 32768, 250), (1, 32768, 257), (2, 32768, 128)])
+def test_gemm_many_contributors(tiny_ctx, M, K, N):
+    """Tiles that more CTAs share than a reduction round has copies (128): one row, one or two
+    tiles, more than 128 chunks."""
+    x = synth.normal_f32(4, M, (M, K), 1.0, device="cuda")
+    w = synth.normal_bf16(4, N, (N, K), 0.02, device="cuda")
+    y = torch.full((M, N), float("nan"), device="cuda")
+    tiny_ctx.op_gemm(x, w, y)
+    ref = x.double() @ w.double().t()
+    assert tiny_ctx.get_error() == 0
+    assert (y.double() - ref).abs().max().item() <= 5e-5 * math.sqrt(K) * 0.02 + 1e-6 * ref.abs().max().item()
+
+
 def test_gemm_deterministic(tiny_ctx):
     x = synth.normal_f32(3, 1, (6, 4096), 1.0, device="cuda")
     w = synth.normal_bf16(3, 2, (4096, 4096), 0.02, device="cuda")
