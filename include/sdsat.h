@@ -390,12 +390,13 @@ SDSAT_API sdsat_status sdsat_debug_workspace(sdsat_ctx* ctx, int which, int rows
  * (sequence, head) pairs (host only, no GPU): one thread-block cluster of *cs CTAs per
  * pair, *nclusters = pairs, for the largest cs <= min(cs_cap, 16) with
  * max_clusters[cs] >= pairs and cs * (pairs + 8) <= max_clusters[1] (the CTAs resident
- * at once, else 2 * num_sms); otherwise *cs = 1 and *nclusters = min(pairs, resident),
- * each CTA taking several pairs.  max_clusters[c] (c = 1..16, host array of 17 entries,
- * [0] unused) = the most clusters of c CTAs the device holds at once, as
- * cudaOccupancyMaxActiveClusters reports it for the attention kernel.  The launches also cap
- * cs at the cache's 64-slot units, and take the next smaller grid where fewer than a tenth more
- * clusters of cs than pairs fit.  Errors: EINVAL. */
+ * at once, else 2 * num_sms), or, where that cs is above 2 and fewer than a tenth more
+ * clusters of it than pairs fit, the next smaller such cs; otherwise *cs = 1 and
+ * *nclusters = min(pairs, resident), each CTA taking several pairs.  max_clusters[c]
+ * (c = 1..16, host array of 17 entries, [0] unused) = the most clusters of c CTAs the
+ * device holds at once, as cudaOccupancyMaxActiveClusters reports it for the attention
+ * kernel.  The launches' cs_cap is the number of 64-slot units of the cache and, for head
+ * dimension 64 and q <= 8, also max_clusters[1] / (pairs + 10).  Errors: EINVAL. */
 SDSAT_API sdsat_status sdsat_attention_grid(int pairs, const int32_t* max_clusters, int cs_cap, int num_sms,
                                             int* cs, int* nclusters);
 

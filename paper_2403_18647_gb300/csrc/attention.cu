@@ -648,12 +648,19 @@ void attention_grid(int pairs, const int* maxc, int cs_cap, int num_sms, int* cs
   // a second wave.  If not even pairs of CTAs fit, single CTAs (as many as are resident
   // at once) take several pairs each.
   const int resident = maxc[1] > 0 ? maxc[1] : 2 * num_sms;
-  *cs = 1;
-  for (int c = std::min(cs_cap, ATT_CS_MAX); c >= 2; --c)
-    if (maxc[c] >= pairs && c * (pairs + ATT_SPARE_CLUSTERS) <= resident) {
-      *cs = c;
-      break;
-    }
+  auto largest = [&](int cap) {
+    for (int c = std::min(cap, ATT_CS_MAX); c >= 2; --c)
+      if (maxc[c] >= pairs && c * (pairs + ATT_SPARE_CLUSTERS) <= resident) return c;
+    return 1;
+  };
+  *cs = largest(cs_cap);
+  // A tenth more clusters than pairs have to fit: 80 pairs (13B, two sequences) need nearly every
+  // place that the QKV projection's CTAs leave for clusters of 5 (87 fit), and some of them enter
+  // late.  13B, four layers, 5 CTAs -> 4: 6 rows, context 1024 589.6 -> 571.7 us, 8 rows, 3000 662.9
+  // -> 627.3, 14 rows, 1000 691 -> 654.5.  (32, 40, 64, 96, 120 and 128 pairs: 12 to 23 % more fit,
+  // and smaller clusters are no faster; with 32, 36 clusters of 11 fit, context 2048: 386.8 us for
+  // four 7B layers against 391.3 with 10.)
+  if (*cs > 2 && 10 * maxc[*cs] < 11 * pairs) *cs = largest(*cs - 1);
   *nclusters = *cs > 1 ? pairs : std::max(1, std::min(pairs, resident));
 }
 
@@ -668,14 +675,6 @@ cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st,
   int cap = std::min(g_att_cs_cap, units);
   if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (pairs + ATT_SPARE_CLUSTERS + 2)));
   attention_grid(pairs, maxc, cap, num_sms, &p.cs, &p.nclusters);
-  // A tenth more clusters than pairs have to fit: 80 pairs (13B, two sequences) need nearly every
-  // place that the QKV projection's CTAs leave for clusters of 5 (87 fit), and some of them enter
-  // late.  13B, four layers, 5 CTAs -> 4: 6 rows, context 1024 589.6 -> 571.7 us, 8 rows, 3000 662.9
-  // -> 627.3, 14 rows, 1000 691 -> 654.5.  (32, 40, 64, 96, 120 and 128 pairs: 12 to 23 % more fit,
-  // and smaller clusters are no faster; with 32, 36 clusters of 11 fit, context 2048: 386.8 us for
-  // four 7B layers against 391.3 with 10.)
-  const bool tight = 10 * maxc[p.cs] < 11 * pairs;
-  if (tight && p.cs > 2) attention_grid(pairs, maxc, p.cs - 1, num_sms, &p.cs, &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);

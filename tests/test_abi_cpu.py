@@ -75,5 +75,15 @@ def test_attention_grid_choice_on_the_host():
     holes = list(three)
     holes[11] = holes[10] = 0
     assert sd.attention_grid(32, holes) == (9, 32)
+    # a tenth more clusters than pairs have to fit, else the next smaller size (down to 2)
+    tight = list(three)
+    for fit, cs in ((88, 5), (87, 4), (80, 4)):      # 80 pairs: 13B, two sequences
+        tight[5] = fit
+        assert sd.attention_grid(80, tight) == (cs, 80)
+    tight[4] = 0
+    assert sd.attention_grid(80, tight) == (3, 80)
+    tight[3], tight[2] = 87, 80
+    assert sd.attention_grid(80, tight, cs_cap=3) == (2, 80)
+    assert sd.attention_grid(80, tight, cs_cap=2) == (2, 80)
     lib = sd.lib()
     assert lib.sdsat_attention_grid(0, None, 16, 152, None, None) == 1
