@@ -395,8 +395,7 @@ SDSAT_API sdsat_status sdsat_debug_workspace(sdsat_ctx* ctx, int which, int rows
  * *nclusters = min(pairs, resident), each CTA taking several pairs.  max_clusters[c]
  * (c = 1..16, host array of 17 entries, [0] unused) = the most clusters of c CTAs the
  * device holds at once, as cudaOccupancyMaxActiveClusters reports it for the attention
- * kernel.  The launches' cs_cap is the number of 64-slot units of the cache and, for head
- * dimension 64 and q <= 8, also max_clusters[1] / (pairs + 10).  Errors: EINVAL. */
+ * kernel.  The launches' cs_cap is the number of 64-slot units of the cache.  Errors: EINVAL. */
 SDSAT_API sdsat_status sdsat_attention_grid(int pairs, const int32_t* max_clusters, int cs_cap, int num_sms,
                                             int* cs, int* nclusters);
 

@@ -667,20 +667,17 @@ void attention_grid(int pairs, const int* maxc, int cs_cap, int num_sms, int* cs
 cudaError_t launch_attention(const AttnParams& p0, int num_sms, cudaStream_t st, bool pdl) {
   AttnParams p = p0;
   // No more CTAs per pair than the cache has units: the others only widened the merge (one
-  // sequence, 32 heads, us per launch: capacity 106 6.64 -> 5.28, 506 6.72 -> 6.41).
-  // With head dimension 64 two more spare clusters (32 heads, context 8192: 11 CTAs 20.3 us, 10
-  // CTAs 18.4; context 2000 10.1 and 8.5; 40 heads keep 9).
-  const int* maxc = g_att_clusters[p.hd == 128][p.q > 8];
-  const int units = (p.cap + ATT_UNIT - 1) / ATT_UNIT, pairs = p.nb * p.H;
-  int cap = std::min(g_att_cs_cap, units);
-  if (p.hd == 64 && p.q <= 8) cap = std::min(cap, std::max(1, maxc[1] / (pairs + ATT_SPARE_CLUSTERS + 2)));
-  attention_grid(pairs, maxc, cap, num_sms, &p.cs, &p.nclusters);
+  // sequence, 32 heads, 6 rows, us: capacity 106 6.5 -> 5.5 a launch, 367 -> 362 for a 7B step of
+  // four layers; 506 6.8 -> 6.5).
+  const int units = (p.cap + ATT_UNIT - 1) / ATT_UNIT;
+  attention_grid(p.nb * p.H, g_att_clusters[p.hd == 128][p.q > 8], std::min(g_att_cs_cap, units), num_sms, &p.cs,
+                 &p.nclusters);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nclusters * p.cs);
   cfg.blockDim = dim3(128);
-  // Single CTAs that fit two to an SM: room for no third, or some SMs get three and others one (240
-  // pairs, 10 rows, context 1000: 39.2 us against 32.9; 7 sequences of 4 rows, 32 heads, context
-  // 3000: 82 against 65).
+  // Single CTAs that fit two to an SM: room for no third, or some SMs get three and others one
+  // while the QKV projection's CTAs leave (four layers and LM head, us, without -> with: 7B, 7
+  // sequences of 4 rows, context 2000 678 -> 665, 13B, 6 of 10 rows, context 1000 762 -> 736).
   cfg.dynamicSmemBytes = attention_smem_bytes(p.hd, p.q);
   if (p.cs == 1 && p.nclusters <= 2 * num_sms)
     cfg.dynamicSmemBytes = std::max<size_t>(cfg.dynamicSmemBytes, ATT_TWO_PER_SM);
