@@ -36,10 +36,11 @@ namespace sdsat {
 
 // Pipeline depth and CTAs per SM (compile-time tuning).  Measured on GB300: one CTA
 // per SM streams ~5 TB/s whatever its depth (3..10 stages), two CTAs per SM ~7 TB/s.
-// For M <= 16 a CTA has 4 stages (~91 KB of shared memory), so exactly two fit on an
-// SM.  With 3 stages (~71 KB) a third fits: the next kernel's CTAs then start early,
-// but the scheduler also stacks three CTAs of one GEMM on some SMs and one on others,
-// and the equal stream-K shares finish unevenly (7B step 3.80 ms vs 3.70 with 4).
+// For M <= 16 a CTA has 4 stages (83 KB of shared memory with 8 padded rows, 99 KB with 16;
+// 3 stages with 24 rows take 93 KB, with 32 107 KB), so exactly two fit on an SM.  With 3 stages
+// (65 KB with 8 rows) a third fits: the next kernel's CTAs then start early, but the scheduler
+// also stacks three CTAs of one GEMM on some SMs and one on others, and the equal stream-K shares
+// finish unevenly (7B step 3.80 ms vs 3.70 with 4).
 #ifndef SDSAT_GEMM_STAGES16
 #define SDSAT_GEMM_STAGES16 4
 #endif
@@ -69,7 +70,6 @@ struct GemmCfg {
   static constexpr int PARTS = MPAD <= 8 ? 16 : (MPAD <= 16 ? 8 : 4);
   static constexpr int NBAR = 2 * STAGES + 6;
   static constexpr int CS = MPAD * 64;           // EPI_QKV: RoPE (cos, sin) of every row and frequency
-  static constexpr int EGR = MPAD;   // residual rows loaded before the accumulator wait: every row
   static constexpr size_t SMEM =
       1024 + (size_t)STAGES * STAGE_BYTES + STAGING * 4 + 2 * 64 * 4 + 64 * 8 + CS * 8 + NBAR * 8 + 128;
 };
@@ -122,10 +122,9 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity) 
 template <int MPAD>
 __device__ __forceinline__ void epilogue_final(const GemmParams& p, int tile, int r, float (&acc)[MPAD],
                                                float* staging, const float* sinv, const long long* s_rowbase,
-                                               const float (&pre)[GemmCfg<MPAD>::EGR], float pre_gn,
+                                               const float (&pre)[MPAD], float pre_gn,
                                                const float2* s_cs) {
   const int M = p.M;
-  constexpr int GR = GemmCfg<MPAD>::EGR;
   if (p.ssq_in) {
 #pragma unroll
     for (int m = 0; m < MPAD; ++m) acc[m] *= sinv[m];
@@ -137,18 +136,10 @@ __device__ __forceinline__ void epilogue_final(const GemmParams& p, int tile, in
     const int n = 128 * tile + r;
     const bool valid = n < p.N;
 #pragma unroll
-    for (int m0 = 0; m0 < MPAD; m0 += GR) {
-      float hv[GR];
-#pragma unroll
-      for (int u = 0; u < GR; ++u)
-        hv[u] = m0 == 0 ? pre[u] : (m0 + u < M && valid) ? __ldcg(p.out + (size_t)(m0 + u) * p.out_ld + n) : 0.f;
-#pragma unroll
-      for (int u = 0; u < GR; ++u) {
-        const int m = m0 + u;
-        if (m >= M) break;
-        acc[m] = valid ? hv[u] + acc[m] : 0.f;   // h after the update
-        staging[r * (MPAD + 1) + m] = acc[m] * acc[m];
-      }
+    for (int m = 0; m < MPAD; ++m) {
+      if (m >= M) break;
+      acc[m] = valid ? pre[m] + acc[m] : 0.f;   // h after the update
+      staging[r * (MPAD + 1) + m] = acc[m] * acc[m];
     }
     named_bar_sync(1, 128);
     // pass 1: thread (part, m) sums lanes part*RPP .. part*RPP+RPP-1 of row m
@@ -191,14 +182,7 @@ __device__ __forceinline__ void epilogue_final(const GemmParams& p, int tile, in
     if (n < p.N) {
       if (p.epi == EPI_RESID) {
 #pragma unroll
-        for (int m0 = 0; m0 < MPAD; m0 += GR) {
-          float hv[GR];
-#pragma unroll
-          for (int u = 0; u < GR; ++u)
-            hv[u] = m0 == 0 ? pre[u] : (m0 + u < M) ? __ldcg(p.out + (size_t)(m0 + u) * p.out_ld + n) : 0.f;
-#pragma unroll
-          for (int u = 0; u < GR; ++u) acc[m0 + u] += hv[u];
-        }
+        for (int m = 0; m < MPAD; ++m) acc[m] += pre[m];
       }
 #pragma unroll
       for (int m = 0; m < MPAD; ++m)
@@ -489,15 +473,15 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
       ++tile;   // segments are consecutive tiles
       g = std::min(g1, (long long)(tile + 1) * p.kc);
       const int buf = seg & 1;
-      // what this tile's epilogue reads from global memory (first row group), loaded while
-      // the tensor cores work: residual rows and gain
-      float pre[C::EGR];
+      // what this tile's epilogue reads from global memory, loaded while the tensor cores
+      // work: residual rows and gain
+      float pre[MPAD];
       float pre_gn = 0.f;
       {
         const int n = 128 * tile + r;
         const bool resid = p.epi == EPI_RESID && !p.publish && n < p.N;
 #pragma unroll
-        for (int u = 0; u < C::EGR; ++u) pre[u] = (resid && u < p.M) ? __ldcg(p.out + (size_t)u * p.out_ld + n) : 0.f;
+        for (int m = 0; m < MPAD; ++m) pre[m] = (resid && m < p.M) ? __ldcg(p.out + (size_t)m * p.out_ld + n) : 0.f;
         if (resid && p.gain_next) pre_gn = __bfloat162float(p.gain_next[n]);
       }
       // the four epilogue warps decide together (lanes leave the polling loop at different

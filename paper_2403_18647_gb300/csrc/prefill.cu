@@ -54,7 +54,6 @@ struct PfCfg {
   static constexpr int STAGE = PF_W_BYTES + X_BYTES;     // per CTA: 32 KB (24 KB)
   static constexpr int RING = STAGES * STAGE;
   static constexpr int ACC = 2 * TOK;                    // TMEM columns of one accumulator (hi, lo)
-  static constexpr int ROUNDS = TOK / (2 * PF_CHUNK);    // epilogue rounds of each of the two warp groups
   static constexpr int NBAR = 2 * STAGES + 7;
   static constexpr size_t SMEM = 1024 + (size_t)RING + PF_STAGING * 4 + 2 * TOK * 4 + NBAR * 8 + 64;
   static_assert(SMEM <= 232448, "shared memory of one CTA");
