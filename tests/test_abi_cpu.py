@@ -58,13 +58,13 @@ def _gpc_model(ctas_per_sm, gpcs=8, sms_per_gpc=19):
 
 def test_attention_grid_choice_on_the_host():
     """The cluster size the attention picks (host logic, no GPU) on a 152-SM, 8-GPC model:
-    the sizes the measured 7B / 13B / batch-4 / 11-row workloads ran with."""
+    the sizes the measured 7B / 13B / batch-4 workloads run with, and devices that hold fewer."""
     import paper_2403_18647_gb300 as sd
-    three, two = _gpc_model(3), _gpc_model(2)     # q <= 8: three CTAs per SM; q <= 16: two
+    three, two = _gpc_model(3), _gpc_model(2)     # three CTAs per SM (every q <= 16), or two
     assert sd.attention_grid(32, three) == (11, 32)      # 7B, one sequence: 352 CTAs
     assert sd.attention_grid(40, three) == (9, 40)       # 13B: 360 CTAs
     assert sd.attention_grid(128, three) == (3, 128)     # 7B, four sequences: 384 CTAs
-    assert sd.attention_grid(32, two) == (7, 32)         # 11-row blocks: 224 CTAs
+    assert sd.attention_grid(32, two) == (7, 32)         # 224 CTAs
     assert sd.attention_grid(512, three) == (1, 456)     # more pairs than fit: single CTAs
     assert sd.attention_grid(200, three) == (2, 200)
     assert sd.attention_grid(300, three) == (1, 300)

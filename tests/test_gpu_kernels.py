@@ -449,10 +449,11 @@ def test_argmax_signed_zero_and_minus_infinity(sd):
 
 
 @pytest.mark.parametrize("M,K,N", [(6, 1024, 300), (6, 1032, 300), (6, 1000, 38912), (6, 1024, 38913),
-                                   (24, 1024, 4097), (48, 1024, 19456), (48, 1024, 19457), (64, 1032, 130)])
+                                   (24, 1024, 4097), (24, 1032, 4097), (24, 1024, 38912), (24, 1024, 38913),
+                                   (17, 1032, 38912), (48, 1024, 19456), (48, 1024, 19457), (64, 1032, 130)])
 def test_gemm_whole_and_split_tiles(tiny_ctx, M, K, N):
     """Both sides of the rule that leaves tiles whole: 16 and 17 chunks, as many tiles as CTAs
-    and one more (two CTAs per SM up to 32 rows, one beyond)."""
+    (two per SM) and one more; the same widths on the tiled GEMM of more than 32 rows."""
     x = synth.normal_f32(11, M, (M, K), 1.0, device="cuda")
     w = synth.normal_bf16(11, N, (N, K), 0.02, device="cuda")
     y = torch.full((M, N), float("nan"), device="cuda")
@@ -462,13 +463,14 @@ def test_gemm_whole_and_split_tiles(tiny_ctx, M, K, N):
     assert (y.double() - ref).abs().max().item() <= tol
 
 
-@pytest.mark.parametrize("b,q,H,hd", [(6, 10, 40, 128), (4, 16, 40, 64), (8, 8, 38, 128), (8, 8, 40, 128),
-                                      (5, 9, 32, 128), (1, 16, 1, 128), (1, 11, 32, 64), (7, 3, 44, 64)])
-def test_attention_grids(sd, b, q, H, hd):
+@pytest.mark.parametrize("b,q,H,hd,cap", [(6, 10, 40, 128, 700), (4, 16, 40, 64, 700), (8, 8, 38, 128, 700),
+                                          (8, 8, 40, 128, 700), (5, 9, 32, 128, 700), (1, 16, 1, 128, 700),
+                                          (1, 11, 32, 64, 700), (7, 3, 44, 64, 700), (2, 16, 1, 128, 1100),
+                                          (2, 5, 40, 128, 700), (1, 6, 32, 64, 700)])
+def test_attention_grids(sd, b, q, H, hd, cap):
     """One to sixteen CTAs per (sequence, head), single CTAs that fit two to an SM and more of
     them, both query-tile counts and head dimensions, ragged lengths down to an empty cache and
     a cache filled to its last slot; against the explicit softmax in fp64."""
-    cap = 700
     lens = [0, cap - q, 63, 64, 65, 300, 511, 129][:b]
     shape = synth.ModelShape("att", 1, H * hd, H, hd, 256, 256, 0)
     ctx = sd.Context(shape, None, max_position=64) if (H * hd) % 128 == 0 and H * hd <= 8192 else None

@@ -1,11 +1,11 @@
 """Parity of the prefill path (the step before the decode loop) against the oracle.
 
-Prefill runs chunks of up to 64 positions through one block forward each, attended as causal
-groups of 16 rows that share the sequence's cache; a tail shorter than a group runs as one
-block.  Checked:
-  * tiny model, prompt lengths that exercise full chunks, partial chunks and the tail: every
-    layer's K / V rows against the oracle's prefill, then the logits of a decode block on top;
-  * grouped prefill equals the same prompt fed as 16-row blocks (the decode path) on the GPU;
+Prefill runs a prompt of up to 16 positions as one block forward, a longer one in equal chunks of
+at most 4096 positions on the tiled GEMM and the prefill attention.  Checked:
+  * tiny model, prompts that run as one block, as one partial tile of 64 or 128 positions, and
+    as more tiles: every layer's K / V rows against the oracle's prefill, then the logits of a
+    decode block on top;
+  * a prefill equals the same prompt fed as 16-row blocks (the decode path) on the GPU;
   * 7B shape at the bench's prompt length (2047): layer 0's K / V rows of every position
     against the oracle's arithmetic for that layer, and the last layer against 16-row blocks.
 """
@@ -70,7 +70,7 @@ def test_prefill_matches_oracle(sd, tiny, n):
 
 
 def test_prefill_equals_blocks_on_gpu(sd, tiny):
-    """Grouped chunks and 16-row decode blocks write the same cache (up to rounding order)."""
+    """A prefill and 16-row decode blocks write the same cache (up to rounding order)."""
     shape, ctx, W = tiny
     n = 150
     prompt = synth.prompt_ids(0, 70, n, 4096).cuda()
@@ -112,7 +112,7 @@ def test_prefill_full_size_7b(sd):
     k, v = ctx.kv_read(kv, 0, 0, 0, P)
     _kv_close(k.float().cpu().numpy(), kref.transpose(1, 0, 2))
     _kv_close(v.float().cpu().numpy(), vref.transpose(1, 0, 2))
-    # the last layer: grouped chunks against 16-row blocks
+    # the last layer: the prefill against 16-row blocks
     kv2 = ctx.kv(1, P + 16)
     pc = prompt.cuda()
     lg = torch.empty(16, shape.vocab, device="cuda")

@@ -1,7 +1,7 @@
 """The prefill attention at the edges of its tiles (128 positions, 128 keys) and launch forms
 (one or two tiles per CTA, one or two chunks, a cache that already holds slots): the second
 layer's K and V rows, which depend on the first layer's attention, against the same prompt fed
-as 16-row decode blocks."""
+as 16-row decode blocks.  And the sequences of a batch: each prefill writes its own rows only."""
 import dataclasses
 
 import pytest
@@ -11,17 +11,25 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-# heads x head_dim: with 40 heads, 1000 positions take two tiles per CTA
+# heads x head_dim: with 40 heads, more than 768 positions take two tiles per CTA
 SHAPES = {(4, 128): 1, (40, 64): 2}
+
+
+def _model(H, hd):
+    import paper_2403_18647_gb300 as sd
+    shape = dataclasses.replace(synth.SHAPES["7b"], name="edge", n_layers=2, d_model=512, n_heads=H, head_dim=hd,
+                                ffn_dim=384, vocab=1000, adaptive_id=999)
+    return shape, sd.Context(shape, synth.make_model(shape, seed=5, device="cuda", gain_std=0.1), max_position=8192)
 
 
 @pytest.fixture(scope="module", params=list(SHAPES))
 def model(request):
-    import paper_2403_18647_gb300 as sd
-    H, hd = request.param
-    shape = dataclasses.replace(synth.SHAPES["7b"], name="edge", n_layers=2, d_model=512, n_heads=H, head_dim=hd,
-                                ffn_dim=384, vocab=1000, adaptive_id=999)
-    return shape, sd.Context(shape, synth.make_model(shape, seed=5, device="cuda", gain_std=0.1), max_position=8192)
+    return _model(*request.param)
+
+
+@pytest.fixture(scope="module")
+def wide_model():
+    return _model(40, 128)
 
 
 def _blocks(ctx, kv, ids, start):
@@ -51,3 +59,34 @@ def test_prefill_attention_edges(model, n, start):
         assert torch.isfinite(a).all()
         assert (a - b).abs().max().item() <= 1e-2 * b.abs().max().item()
         assert ((a - b).norm() / b.norm()).item() <= 2e-3
+
+
+# two tiles of 128 dimensions per CTA: the last CTA with two tiles, one, and one of a single position
+@pytest.mark.parametrize("start", [0, 37])
+@pytest.mark.parametrize("n", [1000, 1025, 1100, 2200])
+def test_prefill_attention_two_tiles_of_128_dimensions(wide_model, n, start):
+    test_prefill_attention_edges(wide_model, n, start)
+
+
+@pytest.mark.parametrize("lens", [(70, 17, 40), (300, 1100, 129)])
+def test_prefill_of_each_sequence(model, lens):
+    """Sequences 1, 2 and 0 of one cache: the rows of each are, bit for bit, those of the same prompt
+    in a cache of its own, and nothing else in the cache changes."""
+    shape, ctx = model
+    cap = max(lens) + 9
+    kv = ctx.kv(3, cap)
+    fill = [[[synth.kv_values(3 + s, l, w, (shape.n_heads, cap, shape.head_dim), device="cuda") for w in (0, 1)]
+             for l in range(shape.n_layers)] for s in range(3)]
+    for s in range(3):
+        for l in range(shape.n_layers):
+            ctx.kv_write(kv, l, s, 0, *fill[s][l])
+    ids = [synth.prompt_ids(9, s, n, 900).cuda() for s, n in enumerate(lens)]
+    for s in (1, 2, 0):
+        ctx.prefill(kv, s, ids[s])
+    assert ctx.kv_lengths(kv).tolist() == list(lens) and ctx.get_error() == 0
+    for s, n in enumerate(lens):
+        one = ctx.kv(1, cap)
+        ctx.prefill(one, 0, ids[s])
+        for l in range(shape.n_layers):
+            for got, ref, old in zip(ctx.kv_read(kv, l, s, 0, cap), ctx.kv_read(one, l, 0, 0, cap), fill[s][l]):
+                assert torch.equal(got[:, :n], ref[:, :n]) and torch.equal(got[:, n:], old[:, n:])
