@@ -66,7 +66,7 @@ WORKLOADS = {
 GEMM_TRAFFIC_RATIO = 185.91 / 180.98
 GEMM_TRAFFIC_CURRENT = True
 GEMM_TRAFFIC_SOURCE = ("ncu dram__bytes_read+write of one K=4096 N=22016 M=6 launch (185.91 MB for 180.98 MB "
-                       "algorithmic, profiles/gemm_gateup_4096x22016_m6.md) times the gate/up launch's algorithmic "
+                       "algorithmic) times the gate/up launch's algorithmic "
                        "bytes; bytes per launch")
 
 
@@ -183,6 +183,12 @@ def gemm_bytes(shape, M):
         "gemm_down": d * F * 2 + M * F * 4 + 2 * M * d * 4,
         "gemm_lm_head": V * d * 2 + M * d * 4 + M * V * 4,
     }
+
+
+def layer_kernels(rows):
+    """Kernels of one decoder layer in a block forward of at most 32 rows (7B and 13B shapes): QKV,
+    attention, O, gate/up, down; at 17 to 24 rows QKV, O and down end in a second kernel each."""
+    return 8 if 17 <= rows <= 24 else 5
 
 
 def weight_bytes(shape):
@@ -546,7 +552,7 @@ def run_ours(args, wl, rank, world):
     # --- profiled pass (per-kernel CUDA events; launches serialised) for the roofline
     r.reset()
     n_prof = min(args.steps, steps_per_gen)
-    launches_per_step = 4 + 5 * shape.n_layers   # build, embed+norm, 5 per layer, head, accept
+    launches_per_step = 4 + layer_kernels(r.b * r.q) * shape.n_layers   # build, embed+norm, layers, head, accept
     r.ctx.profile_begin(n_prof * (launches_per_step + 2) + 16)
     r.run_steps(n_prof, steps_per_gen, None)
     kstats = r.ctx.profile_end()
@@ -582,7 +588,8 @@ def run_ours(args, wl, rank, world):
     # compaction kernels)
     resets = sum(1 for i in range(args.steps) if i % steps_per_gen == 0 and i > 0)
     tree_steps = sum(1 for i in range(args.steps) if (i % steps_per_gen) % 2 == 1) if r.tree else 0
-    gpu_launches = args.steps * launches_per_step + 2 * tree_steps + resets
+    tree_extra = 2 + (layer_kernels(r.b * r.q2) - layer_kernels(r.b * r.q)) * shape.n_layers
+    gpu_launches = args.steps * launches_per_step + tree_extra * tree_steps + resets
     out = {
         "metric": METRIC, "value": round(value, 2), "unit": "tokens/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_step, 4), "higher_is_better": True, "scaling": "weak",
