@@ -516,14 +516,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
           float y[PF_CHUNK];
           load_acc(c0, y);
           if (b0 + 2 * PF_CHUNK >= TOK || c0 + 2 * PF_CHUNK >= vr) drained();
-          if (p.epi == EPI_STORE) {   // nothing to combine: straight to memory, a row per thread
+          if (p.epi == EPI_STORE && !p.ssq_in) {   // nothing to combine: straight to memory, a row per thread
             const int n = 128 * wt + r;
             float* dst = p.out + (size_t)m0 * p.out_ld + n;
             const int cnt = n < p.N ? vr - c0 : 0;
-            if (p.ssq_in) {   // the LM head after a down projection that left its operand unscaled
-#pragma unroll
-              for (int j = 0; j < PF_CHUNK; ++j) y[j] *= inv[c0 + j];
-            }
 #pragma unroll
             for (int j = 0; j < PF_CHUNK; ++j)
               if (j < cnt) dst[(size_t)j * p.out_ld] = y[j];
@@ -560,7 +556,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
 #pragma unroll
             for (int k = 0; k < 8; ++k) v[k].x += t[k].x, v[k].y += t[k].y, v[k].z += t[k].z, v[k].w += t[k].w;
           }
-          if (p.epi == EPI_STORE) {
+          if (p.epi == EPI_STORE && !p.ssq_in) {
             const int n = 128 * wt + 4 * lane, cnt = vr - c0 - w8;
             float* dst = p.out + (size_t)(m0 + w8) * p.out_ld + n;
             const bool vec = (p.out_ld & 3) == 0 && (reinterpret_cast<uintptr_t>(p.out) & 15u) == 0 && n + 4 <= p.N;
@@ -568,10 +564,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
             for (int k = 0; k < 8; ++k)
               if (k < cnt) {
                 float* d = dst + (size_t)k * p.out_ld;
-                if (p.ssq_in) {
-                  const float f = inv[c0 + w8 + k];
-                  v[k].x *= f, v[k].y *= f, v[k].z *= f, v[k].w *= f;
-                }
                 if (vec) {
                   *reinterpret_cast<float4*>(d) = v[k];
                 } else {
@@ -629,6 +621,14 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
               pf_qkv_store(p, which, m, row_of, f, i, a, b);
               if (which == 1 && (lane & 15) == 0) row_of.report(p);
             }
+          }
+        } else if (p.epi == EPI_STORE) {
+          // the LM head whose operand still needs the positions' RMSNorm factors
+#pragma unroll 1
+          for (int k = 0; k < left; ++k) {
+            float* dst = p.out + (size_t)(m0 + w8 + k) * p.out_ld;
+            for (int i = lane, n = 128 * wt + lane; i < 128 && n < p.N; i += 32, n += 32)
+              dst[n] = slab[(w8 + k) * 128 + i] * inv[c0 + w8 + k];
           }
         } else {
           const int n = 128 * wt + 4 * lane;
@@ -785,7 +785,8 @@ __global__ void __launch_bounds__(PF_FIN_ROW_THREADS) prefill_finish_resid_kerne
   }
 }
 
-// out = sum of the parts, times the operand row's factor (blockIdx.y: 2048 features)
+// out = sum of the parts (SCALED: times the operand row's RMSNorm factor; blockIdx.y: 2048 features)
+template <bool SCALED>
 __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_store_kernel(const __grid_constant__ PfGemmParams p) {
   pdl_wait();
   pdl_trigger();
@@ -802,7 +803,7 @@ __global__ void __launch_bounds__(PF_FIN_THREADS) prefill_finish_store_kernel(co
 #pragma unroll
     for (int u = 0; u < PF_FIN_PARTS; ++u) pf_add(y, t[u]);
   }
-  if (p.ssq_in) {
+  if constexpr (SCALED) {
     const float s = pf_row_factor(p, m);
     y.x *= s, y.y *= s, y.z *= s, y.w *= s;
   }
@@ -877,7 +878,8 @@ cudaError_t prefill_prepare() {
   if (e == cudaSuccess) e = prefer_shared(prefill_gemm_kernel<64>);
   if (e == cudaSuccess) e = prefer_shared(prefill_finish_resid_kernel);
   if (e == cudaSuccess) e = prefer_shared(prefill_finish_qkv_kernel);
-  if (e == cudaSuccess) e = prefer_shared(prefill_finish_store_kernel);
+  if (e == cudaSuccess) e = prefer_shared(prefill_finish_store_kernel<false>);
+  if (e == cudaSuccess) e = prefer_shared(prefill_finish_store_kernel<true>);
   if (e != cudaSuccess || g_pf_pairs > 0) return e;
   cudaLaunchAttribute attr[2];
   const cudaLaunchConfig_t cfg = pf_config(128, 1, nullptr, false, attr);
@@ -926,7 +928,8 @@ cudaError_t launch_prefill_gemm(const PfGemmParams& p, cudaStream_t st, bool pdl
   fin.numAttrs = pdl ? 1 : 0;
   return p.epi == EPI_QKV     ? cudaLaunchKernelEx(&fin, prefill_finish_qkv_kernel, p)
          : p.epi == EPI_RESID ? cudaLaunchKernelEx(&fin, prefill_finish_resid_kernel, p)
-                              : cudaLaunchKernelEx(&fin, prefill_finish_store_kernel, p);
+         : p.ssq_in           ? cudaLaunchKernelEx(&fin, prefill_finish_store_kernel<true>, p)
+                              : cudaLaunchKernelEx(&fin, prefill_finish_store_kernel<false>, p);
 }
 
 }  // namespace sdsat
