@@ -344,7 +344,10 @@ SDSAT_API sdsat_status sdsat_accept_pipelined(sdsat_ctx* ctx, sdsat_kv* kv, cons
  * y_1 .. y_n already in the context; the paper gives the prefill no further detail).  Equal chunks of
  * at most 4096 positions (at most max_position rounded up to 128) go through the layers one
  * after the other (the weights stream once per chunk), position i attending to every earlier
- * position.  No logits are produced.
+ * position.  No logits are produced.  The workspaces of the largest chunk belong to the context
+ * (sdsat_create allocates them with the weights): per position 8 d_model + 8 R + 4 ffn_dim bytes
+ * and 4 bytes per 128 of d_model, R = n_heads * head_dim; 449 MB for a 7B context, 563 MB at 13B,
+ * of max_position 4096 or more.
  * Errors: EINVAL (null pointer, seq outside the KV batch, n < 0), ECAPACITY
  * (n > max_len); device bit CAPACITY if len[seq] + n > max_len. */
 SDSAT_API sdsat_status sdsat_prefill(sdsat_ctx* ctx, sdsat_kv* kv, int seq, const int32_t* tokens_dev, int n);

@@ -69,8 +69,9 @@ struct AttCfg {
   static constexpr size_t OFF_Q = (size_t)ATT_STAGES * STAGE;
   // P hi + lo tiles in their own area; with two query tiles of 128 dimensions over the unit's K
   // tile, whose last reader has passed the barrier before P is written, so that three CTAs fit
-  // on an SM (75.9 KB instead of 81.5): 32 heads, 11 rows, context 16384 66.7 -> 55.9 us, three
-  // sequences of 16 rows, context 8000 110 -> 73, context 2048 13.3 -> 13.2
+  // on an SM (75.9 KB instead of 81.5): 32 heads, 11 rows, context 16384 67.8 -> 58.5 us, three
+  // sequences of 16 rows, context 8000 111 -> 76, 11 rows, context 2048 14.5 -> 13.6.  (Three CTAs
+  // leave 168 registers a thread, at which this instance spills 32 bytes; at two, 254 and no spill.)
   static constexpr bool P_OVER_K = QT == 2 && HD == 128;
   static constexpr size_t OFF_P = OFF_Q + 2 * ROWS * QSTRIDE;
   static constexpr size_t OFF_RED = OFF_P + (P_OVER_K ? 0 : 2 * ROWS * PSTRIDE);   // unit row max, sums; partial stats
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(128, 3) attention_kernel(const __grid_constant
     // fetched cold, so G lanes share an item, each with at most six of the cs partials: one
     // thread with an unrolled loop over 16 took 1.5 us from the loads to the stores with 11 CTAs.
     // With 9 to 12 CTAs and more than 32 items (10 rows and up) two lanes and one pass instead of
-    // four lanes and two: 16 rows, context 2048 14.6 -> 14.0 us (7B, four layers: 432.8 -> 430.8).
+    // four lanes and two: 16 rows, context 2048 14.8 -> 13.9 us (7B, four layers: 432.8 -> 430.8).
     bool arrived = false;
     {
       const int items = q * D4, i0 = items * rank / CS, i1 = items * (rank + 1) / CS;

@@ -596,8 +596,9 @@ __global__ void __launch_bounds__(192, SDSAT_GEMM_MINB) gemm_kernel(const __grid
 // publishes its parts, and one warp per (row, tile) of this kernel, on every SM, sums them in CTA
 // order and runs the epilogue.  Four 7B layers and the head, without and with it: 24 rows 486.9 ->
 // 476.5 us, 20 rows 468.4 -> 461.6, 18 rows 446.7 -> 445.1 (13B, 24 rows: 667.9 -> 665.5).  Fewer
-// rows end sooner by themselves (16: 418.4 -> 434.6, 11: 417.2 -> 444.8, 6: 386.2 -> 426.0), and
-// at 28 rows it is slower too (513.8 -> 527.4).
+// rows end sooner by themselves (16: 418.4 -> 434.6, 11: 417.2 -> 444.8, 6: 386.2 -> 426.0).  At 28
+// rows (the 32-row instance, parts of 16 KB) it measured slower too (513.8 -> 527.4); why was not
+// found, so the line is a measured one, on these two models, and not derived.
 constexpr int GEMM_PUBLISH_MPAD = 24;
 constexpr int FIN_PARTS = 6;   // parts loaded together
 

@@ -182,7 +182,10 @@ cudaError_t prefill_attention_prepare();
 cudaError_t launch_prefill_attention(PfAttnParams& p, int num_sms, cudaStream_t st, bool pdl);
 
 // ---- prefill (prompt chunks of up to PF_ROWS positions) -------------------------
-constexpr int PF_ROWS = 4096;   // 4095 positions, two 7B layers: 4.53 ms in one chunk, 4.64 in two
+// 4095 positions, two 7B layers: 4.53 ms in one chunk, 4.64 in two.  The workspaces (h in fp32, the
+// queries and the three operands as hi + lo: 8 d + 8 R + 4 F bytes a row) take 449 MB in a 7B context
+// that holds 4096 positions or more, 563 MB at 13B (225 and 281 with chunks of 2048).
+constexpr int PF_ROWS = 4096;
 struct PfGemmParams {
   CUtensorMap tmap[3];      // weights, as GemmParams::tmap (map_mode)
   CUtensorMap tmap_x[2];    // positions' operand, bf16 hi / lo [rows][K], boxes of 64 x prefill_tok(M)
