@@ -755,11 +755,20 @@ cudaError_t gemm_prepare() {
 // costs a CTA about 0.2 us, publishing and reducing a split tile 3 us.  us per launch, split ->
 // whole: K = 256, N = 768 7.4 -> 5.6; K = 1024, N = 8192 10.3 -> 9.5, N = 32000 17.6 -> 13.7, 24
 // rows x N = 4096 12.5 -> 10.6, N = 1024 8.7 -> 9.1; K = 2048, N = 2048 (32 chunks) 10.5 -> 14.0.
-constexpr int GEMM_WHOLE_KC = 16;
+// A plain product of up to 8 padded rows has the cheapest split (parts of 4 KB, no row sums, RoPE or
+// operand to emit): its tiles stay whole up to 7 chunks, and one more for every 5 tiles, with which
+// a CTA's share of the split grows.  6 rows, split / whole: K = 512, N = 128 6.6 / 6.7, N = 1024 6.9 /
+// 6.7; 768, 2048 7.7 / 8.0, 768, 4096 8.0 / 8.0, 768, 5000 10.2 / 8.1; 1024, 1024 7.4 / 9.1, 1024, 4096
+// 8.3 / 9.3, 1024, 6000 9.6 / 9.3, 1024, 8192 10.2 / 9.5.  (A decoder of d 1024, four layers and head, 6 rows: 158 us with every tile
+// whole, 176 with every tile split.)
+static bool gemm_whole_tiles(const GemmParams& p, long long ctas) {
+  if (p.kc > GEMM_WHOLE_KC || p.n_tiles > ctas) return false;
+  return p.epi != EPI_STORE || gemm_mpad(p.M) > 8 || p.kc <= 7 + p.n_tiles / 5;
+}
 static int gemm_grid(const GemmParams& p, int num_sms) {
   const long long T = (long long)p.n_tiles * p.kc;
   const long long ctas = (long long)num_sms * GEMM_CTAS_PER_SM;
-  if (p.kc <= GEMM_WHOLE_KC && p.n_tiles <= ctas) return p.n_tiles;
+  if (gemm_whole_tiles(p, ctas)) return p.n_tiles;
   return (int)std::min<long long>(ctas, T);
 }
 

@@ -122,6 +122,7 @@ struct GemmParams {
 
 int gemm_mpad(int M);                 // rows of the operand boxes of M <= 32 rows: 8, 16, 24 or 32
 constexpr int GEMM_MPADS[] = {8, 16, 24, 32};
+constexpr int GEMM_WHOLE_KC = 16;     // 64-column chunks of K up to which the skinny GEMM may leave tiles whole
 // Blocks of more rows than this run on the tiled GEMM of prefill.cu (64-row tiles).  The skinny
 // GEMM's split-K tail grows with the rows: its last contributors summed 10 parts of 32 KB and
 // ran a 64-row epilogue in 13 us.  Four 7B layers and LM head, us per block step, skinny -> tiled:

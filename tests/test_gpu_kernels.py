@@ -449,11 +449,14 @@ def test_argmax_signed_zero_and_minus_infinity(sd):
 
 
 @pytest.mark.parametrize("M,K,N", [(6, 1024, 300), (6, 1032, 300), (6, 1000, 38912), (6, 1024, 38913),
+                                   (1, 448, 100), (8, 456, 100), (8, 512, 640), (8, 512, 512), (6, 1024, 5760), (6, 1024, 5632),
+                                   (9, 1024, 100),
                                    (24, 1024, 4097), (24, 1032, 4097), (24, 1024, 38912), (24, 1024, 38913),
                                    (17, 1032, 38912), (48, 1024, 19456), (48, 1024, 19457), (64, 1032, 130)])
 def test_gemm_whole_and_split_tiles(tiny_ctx, M, K, N):
     """Both sides of the rule that leaves tiles whole: 16 and 17 chunks, as many tiles as CTAs
-    (two per SM) and one more; the same widths on the tiled GEMM of more than 32 rows."""
+    (two per SM) and one more, for plain products of up to 8 rows 7 and 8 chunks of one tile, 8 of
+    four and five, 16 of 44 and 45; the same widths on the tiled GEMM of more than 32 rows."""
     x = synth.normal_f32(11, M, (M, K), 1.0, device="cuda")
     w = synth.normal_bf16(11, N, (N, K), 0.02, device="cuda")
     y = torch.full((M, N), float("nan"), device="cuda")
