@@ -365,8 +365,8 @@ SDSAT_API const char* sdsat_status_string(sdsat_status s);
 /* ---- single kernels (unit parity tests and kernel sweeps) ------------------------- */
 
 /* y[m][n] = sum_k x[m][k] * W[n][k] for m < M, n < N.  M <= 32 runs the weight-streaming
- * skinny GEMM of the block forward, 32 < M <= 512 (and 24 < M <= 32 for narrow and wide W) the
- * tiled GEMM of wider blocks and of the prefill path (256 weight rows x 64 or 128 positions per
+ * skinny GEMM of the block forward, 32 < M <= 512 (and 24 < M <= 32 for narrow W of more than 512
+ * columns and wide W of more than 1024) the tiled GEMM of wider blocks and of the prefill path (256 weight rows x 64 or 128 positions per
  * tile of a CTA pair).  x fp32
  * [M][K] (row stride K), W bf16 [N][K], y fp32 [M][N]; x and W 16-byte aligned,
  * K a multiple of 8, K <= 32768.  Errors: EINVAL. */

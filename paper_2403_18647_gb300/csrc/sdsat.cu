@@ -1182,17 +1182,25 @@ sdsat_status sdsat_get_error(sdsat_ctx* c, uint32_t* flags) {
 // GEMM pads them to 32) where its 256-row tiles either are few or fill the CTA pairs.  In between
 // every tile is split in two or three and a second kernel adds them up: 30 rows, K 4096, us skinny /
 // tiled: N 2048 18.6 / 15.4, 4096 17.2 / 16.5, 6144 18.4 / 18.9, 12288 24.7 / 26.8, 15360 29.0 /
-// 30.6, 17408 31.1 / 29.7, 22016 41.1 / 37.0, 32016 (K 5120) 63.9 / 59.1.
-static bool op_gemm_tiled(int M, int N, int num_sms) {
+// 30.6, 17408 31.1 / 29.7, 22016 41.1 / 37.0, 32016 (K 5120) 63.9 / 59.1.  Where the skinny GEMM
+// leaves its tiles whole it has nothing to add up: wide W go there then, and few tiles up to 8
+// chunks, up to which the tiled GEMM leaves them whole too.  25 rows, skinny / tiled: K 64, N 100 4.9 /
+// 5.6; 256, 1024 6.2 / 6.9; 512, 4096 7.9 / 8.6; 1024, 1024 10.6 / 8.6; 640, 20000 10.0 / 15.9; 640,
+// 38912 12.5 / 14.3; 1024, 32016 14.8 / 17.7.
+static bool op_gemm_tiled(int M, int K, int N, int num_sms) {
+  if (M > GEMM_WIDE_ROWS) return true;
+  if (gemm_mpad(M) != 32) return false;
   const int tiles = (N + 255) / 256, pairs = num_sms / 2;
-  return M > GEMM_WIDE_ROWS || (gemm_mpad(M) == 32 && (4 * tiles <= pairs || 8 * tiles >= 7 * pairs));
+  const bool whole = K <= 64 * GEMM_WHOLE_KC && (N + 127) / 128 <= GEMM_CTAS_PER_SM * num_sms;
+  if (4 * tiles <= pairs) return !(whole && K <= 512);
+  return 8 * tiles >= 7 * pairs && !whole;
 }
 
 sdsat_status sdsat_op_gemm(sdsat_ctx* c, const float* x_dev, int M, int K, const void* w_dev, int N, float* y_dev) {
   if (!c || !x_dev || !y_dev || !aligned16(w_dev) || !aligned16(x_dev)) return SDSAT_EINVAL;
   if (M < 1 || M > OP_MAX_M || K < 8 || K % 8 || K > OP_MAX_K || N < 1 || (N + 127) / 128 > MAX_GEMM_TILES)
     return SDSAT_EINVAL;
-  if (op_gemm_tiled(M, N, c->num_sms)) {
+  if (op_gemm_tiled(M, K, N, c->num_sms)) {
     const int rows = (M + 127) / 128 * 128;   // <= OP_MAX_M rows of the operand scratch
     PfGemmParams g;
     std::memset(&g, 0, sizeof(g));

@@ -65,6 +65,18 @@ def test_tree_batch_equals_single_sequences(ctx, b, q):
     assert ctx.get_error() == 0
 
 
+@pytest.mark.parametrize("M", [25, 32])
+@pytest.mark.parametrize("K,N", [(64, 100), (512, 4864), (520, 4864), (512, 4865), (1024, 16897), (1032, 16897), (1024, 38912), (1024, 38913)])
+def test_gemm_of_25_to_32_rows(ctx, M, K, N):
+    """Skinny and tiled GEMM on both sides of the lines in K and N."""
+    x, w = synth.normal_f32(13, M, (M, K), 1.0, device="cuda"), synth.normal_bf16(13, 1, (N, K), 0.02, device="cuda")
+    y = torch.full((M, N), float("nan"), device="cuda")
+    ctx.op_gemm(x, w, y)
+    ref = x.double() @ w.double().t()
+    tol = 5e-5 * K ** 0.5 * 0.02 + 1e-6 * ref.abs().max().item()   # as the other GEMM parity tests
+    assert (y.double() - ref).abs().max().item() <= tol and ctx.get_error() == 0
+
+
 def test_wide_block_past_the_capacity(ctx):
     """Rows past the KV capacity on the tiled GEMM: flagged, not written, the others as usual."""
     b, q = 3, 16
