@@ -1,13 +1,16 @@
 """The prefill attention at the edges of its tiles (128 positions, 128 keys) and launch forms
 (one or two tiles per CTA, one or two chunks, a cache that already holds slots): the second
 layer's K and V rows, which depend on the first layer's attention, against the same prompt fed
-as 16-row decode blocks.  And the sequences of a batch: each prefill writes its own rows only."""
+as 16-row decode blocks, and against the oracle.  And the sequences of a batch: each prefill
+writes its own rows only."""
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
 import synth
+from oracle import model as OM
 
 pytestmark = pytest.mark.gpu
 
@@ -90,3 +93,21 @@ def test_prefill_of_each_sequence(model, lens):
         for l in range(shape.n_layers):
             for got, ref, old in zip(ctx.kv_read(kv, l, s, 0, cap), ctx.kv_read(one, l, 0, 0, cap), fill[s][l]):
                 assert torch.equal(got[:, :n], ref[:, :n]) and torch.equal(got[:, n:], old[:, n:])
+
+
+# one and two tiles of 128 positions per CTA, a last tile of 44 and of 32 positions
+@pytest.mark.parametrize("H,hd,n", [(4, 128, 300), (40, 64, 800), (40, 128, 800)])
+def test_prefill_attention_matches_oracle(H, hd, n):
+    """The second layer's K and V rows, which depend on the first layer's attention."""
+    shape, ctx = _model(H, hd)
+    W = OM.Weights(shape, tensors=synth.make_model(shape, seed=5, device="cpu", gain_std=0.1))
+    ids = synth.prompt_ids(8, n, n, 900)
+    kvo = OM.KVCache(shape, 1, n, kv_bf16=True)
+    OM.prefill(W, kvo, 0, ids.tolist())
+    kv = ctx.kv(1, n + 8)
+    ctx.prefill(kv, 0, ids.cuda())
+    for got, ref in zip(ctx.kv_read(kv, 1, 0, 0, n), (kvo.K[1][0][:, :n], kvo.V[1][0][:, :n])):
+        err = got.float().cpu().double().numpy() - ref
+        # both sides store bf16 rows: a rounding that falls the other way is 2^-8 of the value
+        assert np.abs(err).max() <= 1e-2 * np.abs(ref).max() and np.linalg.norm(err) <= 2e-3 * np.linalg.norm(ref)
+    assert ctx.get_error() == 0
